@@ -27,6 +27,7 @@
 
 #include "mg3d.h"
 #include "profiles.h"
+#include "fixed_weights.cuh"
 #include "mg3d_internal.h"
 #include "sc_step.cuh"
 
@@ -82,7 +83,8 @@ struct Level {
     // intensity [kRays][nf][nvox]
     void *jnu = nullptr, *jnu_new = nullptr, *rho = nullptr, *rhoS = nullptr;
     StepGeom *geom = nullptr;    // [kRays][nz]
-    void *psteps = nullptr;      // [kRays][nz] PlaneStep<T> of the shifted-plane sweep
+    void *psteps = nullptr;      // [kRays][nz] PlaneLerp<T> (two-level) or PlaneStep<T>
+                                 // (multi-level) of the shifted-plane sweep
     SweepShape shape{};
     // formal solutions in the precision other than the handle's (built on the
     // first request, two-level static CRD handles): chi0, S, the bottom
@@ -178,7 +180,8 @@ struct mg3d_handle {
     double *d_wphin = nullptr;   // [nf] normalised w phi, natural order
     int *d_fidx = nullptr;       // [2][nf] natural frequency of each table position
     bool moving = false;         // the atmosphere has a velocity field
-    double *d_exp_tab = nullptr;         // [64] table of the FP64 exp in the sweep
+    double *d_exp_tab = nullptr;         // [kExpTab] table of the FP64 exp, then the tables
+    fx::u64 *d_fx_tab = nullptr;         // of the integer weights in the same allocation
     double exp_l1 = 0, exp_l2 = 0;
     void *pj = nullptr, *pu = nullptr;
     size_t partial_elems = 0;
@@ -333,9 +336,9 @@ void build_geometry(const mg3d_handle *h, const Level &L, std::vector<StepGeom> 
     }
 }
 
-// Per-step constants of the shifted-plane sweep from the upwind geometry:
-// the bilinear weights and half path of step t, and the corner offsets of
-// step t+1 as the shift of the plane written at step t.
+// Per-step constants of the multi-level shifted-plane sweep from the upwind
+// geometry: the bilinear weights and half path of step t, and the corner
+// offsets of step t+1 as the shift of the plane written at step t.
 template <typename T>
 std::vector<PlaneStep<T>> plane_steps(const Level &L, const std::vector<StepGeom> &g) {
     std::vector<PlaneStep<T>> out((size_t)kRays * L.nz);
@@ -355,6 +358,64 @@ std::vector<PlaneStep<T>> plane_steps(const Level &L, const std::vector<StepGeom
     return out;
 }
 
+// The rounded ratios and scale of the shifted-plane sweep's interpolation.  The
+// weights are the same for every node of a step, and for every step of evenly
+// spaced planes, so a sum c (1 + rx)(1 + ry) that is off 1 by a rounding shifts
+// the intensities of a thin ray by it at every step.  FP32: of the ratios within
+// 4 units in the last place (an offset of the crossing by less than 3e-7
+// cells) the pair whose sum is nearest to 1 (within 1e-9 as a rule).
+template <typename T>
+void round_lerp(PlaneLerp<T> &p, double rx, double ry) {
+    p.rx = (T)rx;
+    p.ry = (T)ry;
+    p.c = (T)(1.0 / ((1.0 + rx) * (1.0 + ry)));
+    if (sizeof(T) == 8) return;
+    const T ulp = (T)std::ldexp(1.0, -24);
+    double best = 2.0;
+    const T rx0 = p.rx, ry0 = p.ry;
+    for (int i = -4; i <= 4; ++i)
+        for (int j = -4; j <= 4; ++j) {
+            const T x = (T)((double)rx0 + i * ulp), y = (T)((double)ry0 + j * ulp);
+            if (x < T(0) || x > T(1) || y < T(0) || y > T(1)) continue;
+            const double sum = (1.0 + (double)x) * (1.0 + (double)y);
+            const T c = (T)(1.0 / sum);
+            const double off = std::fabs((double)c * sum - 1.0) + 1e-12 * (std::abs(i) + std::abs(j));
+            if (off < best) {
+                best = off;
+                p.rx = x;
+                p.ry = y;
+                p.c = c;
+            }
+        }
+}
+
+// The same for the two-level shifted-plane sweep: the weights of each
+// direction as their ratio (at most 1) and the product of the larger ones.
+template <typename T>
+std::vector<PlaneLerp<T>> plane_lerps(const Level &L, const std::vector<StepGeom> &g) {
+    std::vector<PlaneLerp<T>> out((size_t)kRays * L.nz);
+    for (int r = 0; r < kRays; ++r)
+        for (int t = 0; t < L.nz; ++t) {
+            const StepGeom &e = g[(size_t)r * L.nz + t];
+            PlaneLerp<T> &p = out[(size_t)r * L.nz + t];
+            const double bx = std::max(e.tx, 1.0 - e.tx), by = std::max(e.ty, 1.0 - e.ty);
+            const StepGeom &e1 = g[(size_t)r * L.nz + std::max(t - 1, 0)];
+            if (t > 1 && e1.tx == e.tx && e1.ty == e.ty) {
+                p.rx = out[(size_t)r * L.nz + t - 1].rx;
+                p.ry = out[(size_t)r * L.nz + t - 1].ry;
+                p.c = out[(size_t)r * L.nz + t - 1].c;
+            } else {
+                round_lerp(p, std::min(e.tx, 1.0 - e.tx) / bx, std::min(e.ty, 1.0 - e.ty) / by);
+            }
+            p.half_s = (T)(0.5 * e.s);
+            const bool last = t + 1 >= L.nz;
+            p.sx = last ? 0 : g[(size_t)r * L.nz + t + 1].ix0;
+            p.sy = last ? 0 : g[(size_t)r * L.nz + t + 1].iy0;
+            p.near = (e.tx > 0.5 ? 1 : 0) | (e.ty > 0.5 ? 2 : 0);
+        }
+    return out;
+}
+
 int plane_np_index(int np) {
     for (int i = 0; i < kPlaneNpCount; ++i)
         if (kPlaneNp[i] == np) return i;
@@ -366,7 +427,7 @@ template <typename T>
 PlaneArgs<T> plane_args(const mg3d_handle *h, const Level &L, const SweepShape &s,
                         bool other = false) {
     const int nf = h->atom.n_freq;
-    const int last = nf - (s.ngroups - 1) * 2 * s.np;   // frequencies of the last group
+    const int last = (nf + 1) / 2 - (s.ngroups - 1) * s.np;   // slots of the last group
     PlaneArgs<T> a{};
     a.nx = L.nx;
     a.ny = L.ny;
@@ -374,61 +435,78 @@ PlaneArgs<T> plane_args(const mg3d_handle *h, const Level &L, const SweepShape &
     a.rows = s.rows;
     a.bands = s.bands;
     a.ngroups = s.ngroups;
-    a.nslot_last = (last + 1) / 2;
+    a.nslot_last = last;
     a.up_mask = h->up_mask;
     a.rmagic = band_magic(s.rows);
     a.xmagic = band_magic(L.nx);
     a.chi0 = (const T *)(other ? L.o_chi0 : L.chi0);
     a.S = (const T *)(other ? L.o_S : L.S);
     a.bbot = (const T *)(other ? L.o_bbot : L.bbot);
-    a.steps = (const PlaneStep<T> *)(other ? L.o_psteps : L.psteps);
+    a.steps = (const PlaneLerp<T> *)(other ? L.o_psteps : L.psteps);
     a.slots = (const PlaneSlot<T> *)(other ? h->o_pslot : h->d_pslot)[plane_np_index(s.np)];
     a.pj = (T *)(other ? h->o_pj : h->pj);
     a.pu = (T *)(other ? h->o_pu : h->pu);
-    a.exp_tab = h->d_exp_tab;
-    a.exp_l1 = h->exp_l1;
-    a.exp_l2 = h->exp_l2;
+    a.fx_tab = h->d_fx_tab;
     a.status = reinterpret_cast<unsigned *>(h->scal + kScalStatus);
     return a;
 }
 
 int dev_alloc(void **p, size_t bytes);
 
-// Slot tables of the shifted-plane sweep for every supported slot count:
-// group g takes the table positions [2 np g, 2 np (g + 1)) of mirror order 0
-// (x_0, x_{nf-1}, x_1, x_{nf-2}, ..., centre last), slot p of the group the
-// positions 2p and 2p + 1, so mirror pairs share a slot.
+// The tables of the FP64 exp and of the integer weights.
+int upload_tables(mg3d_handle *h) {
+    double tab[kExpTab + 2 * fx::kTab];
+    fx::u64 t[2 * fx::kTab];
+    exp_neg_constants(tab, &h->exp_l1, &h->exp_l2);
+    fx::build_tables(t);
+    std::memcpy(tab + kExpTab, t, sizeof(t));
+    MG_TRY(dev_alloc((void **)&h->d_exp_tab, sizeof(tab)));
+    MG_CUDA(cudaMemcpy(h->d_exp_tab, tab, sizeof(tab), cudaMemcpyHostToDevice));
+    h->d_fx_tab = reinterpret_cast<fx::u64 *>(h->d_exp_tab + kExpTab);
+    return MG3D_OK;
+}
+
+// The slots of a group as operands of the integer weights.
+void fixed_slots(PlaneSlot<double> *s, int np) {
+    long double sum = 0.0L;
+    for (int p = 0; p < np; ++p) {
+        s[p].fx = s[p].w > 0.0 && s[p].phi > std::ldexp(1.0, -fx::kSlotExp) &&
+                  s[p].phi < std::ldexp(1.0, fx::kSlotExp);
+        if (s[p].fx) sum += (long double)s[p].w / s[p].phi;
+    }
+    fx::u64 m;
+    int ea = 0;
+    if (sum > 0.0L) fx::split(sum * 1.0000001L, &m, &ea);   // sum < 2^ea
+    for (int p = 0; p < np; ++p) {
+        if (!s[p].fx) continue;
+        fx::split(s[p].phi, &s[p].pm, &s[p].pe);
+        fx::split(s[p].phi * 1.442695040888963407359924681L, &s[p].ym, &s[p].ye);
+        fx::split(1.0L / s[p].phi, &s[p].im, &s[p].ie);
+        s[p].aq = (fx::u64)std::ldexp((long double)s[p].w / s[p].phi, 64 - ea);
+        s[p].ea = ea;
+    }
+}
+
+// Slot tables of the shifted-plane sweep for every supported slot count: slot j
+// is the mirror pair (x_j, x_{nf-1-j}), the last one of an odd nf the line
+// centre alone; group g takes the slots [np g, np (g + 1)).
 template <typename T>
 int build_plane_slots(mg3d_handle *h, void **out) {
-    const int nf = h->atom.n_freq;
+    const int nf = h->atom.n_freq, nslots = (nf + 1) / 2;
     for (int i = 0; i < kPlaneNpCount; ++i) {
         const int np = kPlaneNp[i];
-        const int ngroups = (nf + 2 * np - 1) / (2 * np);
+        const int ngroups = (nslots + np - 1) / np;
         std::vector<PlaneSlot<T>> tab((size_t)ngroups * np);
-        for (int g = 0; g < ngroups; ++g)
-            for (int p = 0; p < np; ++p) {
-                PlaneSlot<T> &e = tab[(size_t)g * np + p];
-                e = PlaneSlot<T>{};
-                const int ja = 2 * np * g + 2 * p, jb = ja + 1;
-                if (ja >= nf) continue;   // inactive slot of the last group
-                const int ia = mirror_order(nf, 0, ja);
-                e.phi_a = (T)h->phi[ia];
-                e.iphi_a = (T)(1.0 / h->phi[ia]);
-                e.wphi_a = (T)(h->wphi[ia] / kRays);
-                e.wu_a = e.wphi_a;
-                if (jb < nf) {
-                    const int ib = mirror_order(nf, 0, jb);
-                    e.flags = plane::kHasB;
-                    e.phi_b = (T)h->phi[ib];
-                    e.iphi_b = (T)(1.0 / h->phi[ib]);
-                    e.wphi_b = (T)(h->wphi[ib] / kRays);
-                    e.wu_b = e.wphi_b;
-                    if (h->phi[ib] == h->phi[ia]) {
-                        e.flags |= plane::kShared;
-                        e.wu_a = (T)((h->wphi[ia] + h->wphi[ib]) / kRays);
-                    }
-                }
-            }
+        for (int j = 0; j < ngroups * np; ++j) {
+            tab[j] = PlaneSlot<T>{};
+            if (j >= nslots) continue;   // inactive slot of the last group
+            const int m = nf - 1 - j;
+            tab[j].phi = (T)h->phi[j];
+            tab[j].iphi = (T)(1.0 / h->phi[j]);
+            tab[j].w = (T)((h->wphi[j] + (m > j ? h->wphi[m] : 0.0)) / kRays);
+        }
+        if constexpr (sizeof(T) == 8)
+            for (int g = 0; g < ngroups; ++g) fixed_slots(&tab[(size_t)g * np], np);
         MG_TRY(dev_alloc(&out[i], tab.size() * sizeof(PlaneSlot<T>)));
         MG_CUDA(cudaMemcpy(out[i], tab.data(), tab.size() * sizeof(PlaneSlot<T>),
                            cudaMemcpyHostToDevice));
@@ -483,39 +561,56 @@ int shape_capacity(int prec, const SweepShape &s, int nx) {
 }
 
 // Default shifted-plane shape: the largest slot count that takes all
-// frequencies in one group (or groups of 16 beyond 16 frequencies), and the
-// most bands (up to 8) whose 24 x groups clusters the GPU holds in one wave.
-// Planes too large for that take fewer slots per group and up to 16 bands,
-// the first shape that fits.  mg3d_autotune replaces it by measurement.
+// frequencies in one group (or groups of 16 beyond 16 frequencies); fewer slots
+// only where no shape fits.  Of its shapes the ones whose 24 x groups clusters
+// the GPU holds in one wave, with the most bands up to 8 of at least 256
+// nodes (FP32) or 32 (FP64): a smaller band's step is all latency, which more
+// blocks only add to.  Where no shape fits in one wave, the fewest
+// waves (FP32: with the budget of two blocks per SM where that holds more
+// clusters), then the most bands up to 16.  mg3d_autotune replaces it by
+// measurement.
 SweepShape choose_plane_shape(int prec, int nx, int ny, int nfreq) {
     int np0 = plane_np_for(nfreq);
     if (np0 == 0) np0 = kPlaneNp[kPlaneNpCount - 1];
-    SweepShape fallback{};
+    const bool f64 = prec == MG3D_PREC_F64;
     for (int i = kPlaneNpCount - 1; i >= 0; --i) {
         const int np = kPlaneNp[i];
         if (np > np0) continue;
         const int ngroups = (nfreq + 2 * np - 1) / (2 * np);
         SweepShape best{};
-        for (int bands = 1; bands <= kMaxBands && bands <= ny; ++bands) {
-            const int rows = (ny + bands - 1) / bands;
-            if ((long)(bands - 1) * rows >= ny) continue;
-            if (plane_smem_bytes(prec, np, rows, nx) > kMaxPlaneSmem) continue;
-            // one thread per node up to 512 (1024 for FP32 with one or two slots)
-            const int cap = prec == MG3D_PREC_F32 && np <= 2 ? kPlaneMaxThreads : 512;
-            const int th = std::max(32, std::min(cap, ((rows * nx + 31) / 32) * 32));
-            if ((long)rows * nx > (long)plane_max_pass(np, prec == MG3D_PREC_F64) * th) continue;
-            SweepShape s{2 * np, ngroups, bands, rows, th};
-            s.stage = 0;
-            s.plane = 1;
-            s.np = np;
-            const int held = shape_capacity(prec, s, nx);
-            if (held < 1) continue;
-            if (fallback.ng == 0) fallback = s;
-            if (bands <= kPortableBands && held >= kRays * ngroups) best = s;
-        }
-        if (best.ng) return best;
+        int best_waves = 0;
+        for (int lean = 0; lean <= (f64 ? 0 : 1) && best_waves != 1; ++lean)
+            for (int bands = 1; bands <= kMaxBands && bands <= ny; ++bands) {
+                const int rows = (ny + bands - 1) / bands;
+                if ((long)(bands - 1) * rows >= ny) continue;
+                // one thread per node up to 512 (1024 for FP32 with one or two slots)
+                const int cap = !f64 && np <= 2 && !lean ? kPlaneMaxThreads : 512;
+                int th = std::max(32, std::min(cap, ((rows * nx + 31) / 32) * 32));
+                // FP64: a warp's arithmetic is most of a small plane's time, so
+                // the slots of its nodes go to several warps
+                if (f64 && rows * nx <= th) th *= std::max(1, std::min(cap / th, (np + 1) / 2));
+                if (plane_layout(prec, np, rows, nx, th).smem > plane_smem_max(f64)) continue;
+                if ((long)rows * nx > (long)plane_max_pass(np, f64) * th) continue;
+                SweepShape s{2 * np, ngroups, bands, rows, th};
+                s.lean = lean;
+                s.stage = 0;
+                s.plane = 1;
+                s.np = np;
+                const int held = shape_capacity(prec, s, nx);
+                if (held < 1) continue;
+                const int waves = (kRays * ngroups + held - 1) / held;
+                const bool fine = bands > kPortableBands || (long)rows * nx < (f64 ? 32 : 256);
+                if (waves == 1 && best_waves == 1 && fine) continue;
+                if (best_waves == 0 || waves <= best_waves) {
+                    if (waves < best_waves || best_waves == 0 || s.lean == best.lean ||
+                        waves != best_waves)
+                        best = s;
+                    best_waves = waves;
+                }
+            }
+        if (best_waves) return best;
     }
-    return fallback;
+    return SweepShape{};
 }
 
 // Grids the shifted-plane sweep's 32-bit node indices cover.
@@ -905,12 +1000,12 @@ int other_prec_fs(mg3d_handle *h, int k, int prec) {
         std::vector<StepGeom> g;
         build_geometry(h, L, g);
         if (prec == MG3D_PREC_F64) {
-            const auto ps = plane_steps<double>(L, g);
+            const auto ps = plane_lerps<double>(L, g);
             MG_TRY(dev_alloc(&L.o_psteps, ps.size() * sizeof(ps[0])));
             MG_CUDA(cudaMemcpy(L.o_psteps, ps.data(), ps.size() * sizeof(ps[0]),
                                cudaMemcpyHostToDevice));
         } else {
-            const auto ps = plane_steps<float>(L, g);
+            const auto ps = plane_lerps<float>(L, g);
             MG_TRY(dev_alloc(&L.o_psteps, ps.size() * sizeof(ps[0])));
             MG_CUDA(cudaMemcpy(L.o_psteps, ps.data(), ps.size() * sizeof(ps[0]),
                                cudaMemcpyHostToDevice));
@@ -1360,7 +1455,7 @@ static int plane_shape_from_args(const mg3d_handle *h, int level, int freq_per_b
     s.stage = 0;
     s.plane = kind;
     s.np = np;
-    if (plane_smem_bytes(h->prec, np, s.rows, L.nx) > kMaxPlaneSmem)
+    if (plane_layout(h->prec, np, s.rows, L.nx, threads).smem > plane_smem_max(h->prec == MG3D_PREC_F64))
         return fail(MG3D_E_ARG, "sweep shape exceeds shared memory");
     *out = s;
     return MG3D_OK;
@@ -1734,12 +1829,12 @@ int create_impl(const mg3d_atmosphere *atm, const mg3d_atom *atom, const mg3d_qu
         build_geometry(h, L, g);
         MG_CUDA(cudaMemcpy(L.geom, g.data(), g.size() * sizeof(StepGeom), cudaMemcpyHostToDevice));
         if (h->prec == MG3D_PREC_F64) {
-            const auto ps = plane_steps<double>(L, g);
+            const auto ps = plane_lerps<double>(L, g);
             MG_TRY(dev_alloc(&L.psteps, ps.size() * sizeof(ps[0])));
             MG_CUDA(cudaMemcpy(L.psteps, ps.data(), ps.size() * sizeof(ps[0]),
                                cudaMemcpyHostToDevice));
         } else {
-            const auto ps = plane_steps<float>(L, g);
+            const auto ps = plane_lerps<float>(L, g);
             MG_TRY(dev_alloc(&L.psteps, ps.size() * sizeof(ps[0])));
             MG_CUDA(cudaMemcpy(L.psteps, ps.data(), ps.size() * sizeof(ps[0]),
                                cudaMemcpyHostToDevice));
@@ -1818,12 +1913,7 @@ int create_impl(const mg3d_atmosphere *atm, const mg3d_atom *atom, const mg3d_qu
     if (h->prd) MG_TRY(setup_prd(h));
     if (h->prec == MG3D_PREC_F64) MG_TRY(build_plane_slots<double>(h, h->d_pslot));
     else MG_TRY(build_plane_slots<float>(h, h->d_pslot));
-    {
-        double tab[kExpTab];
-        exp_neg_constants(tab, &h->exp_l1, &h->exp_l2);
-        MG_TRY(dalloc(&h->d_exp_tab, kExpTab));
-        MG_CUDA(cudaMemcpy(h->d_exp_tab, tab, sizeof(tab), cudaMemcpyHostToDevice));
-    }
+    MG_TRY(upload_tables(h));
     MG_TRY(dev_alloc(&h->pj, h->partial_elems * es));
     MG_TRY(dev_alloc(&h->pu, h->partial_elems * es));
     MG_TRY(dalloc(&h->scal, kScalStatus + 1));
@@ -2469,12 +2559,7 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
                                             L.mib, h->stream),
                         "bottom intensity"));
     }
-    {
-        double tab[kExpTab];
-        exp_neg_constants(tab, &h->exp_l1, &h->exp_l2);
-        MG_TRY(dalloc(&h->d_exp_tab, kExpTab));
-        MG_CUDA(cudaMemcpy(h->d_exp_tab, tab, sizeof(tab), cudaMemcpyHostToDevice));
-    }
+    MG_TRY(upload_tables(h));
     if (atm->sigma_c) {
         for (long i = 0; i < F.nvox && !h->scatter; ++i) h->scatter = atm->sigma_c[i] > 0.0;
         for (long i = 0; i < F.nvox; ++i)
@@ -3841,8 +3926,8 @@ int mg3d_get_fs_occupancy(mg3d_handle *h, int level, int freq_per_block, int ban
     }
     if (max_clusters) *max_clusters = n;
     if (smem_bytes)
-        *smem_bytes = (long long)(s.plane ? plane_smem_bytes(h->prec, s.np, s.rows,
-                                                             h->lev[level].nx)
+        *smem_bytes = (long long)(s.plane ? plane_layout(h->prec, s.np, s.rows,
+                                                         h->lev[level].nx, s.threads).smem
                                           : sweep_smem_bytes(h->prec, s, h->lev[level].nx));
     return MG3D_OK;
 }

@@ -45,10 +45,10 @@ struct SweepShape {
     int np = 0;    //    frequencies per group (ng = 2 np table positions per group)
 };
 
-// Per (ray, step t) constants of the shifted-plane sweep (plane_sweep.cuh),
-// in the formal-solution precision: the bilinear weights of the upwind
-// corners and half the path length of step t (t >= 1), and the shift of the
-// plane written at step t, i.e. the corner offsets (ix0, iy0) of step t+1
+// Per (ray, step t) constants of the multi-level shifted-plane sweep
+// (ml_plane.cuh), in the formal-solution precision: the bilinear weights of the
+// upwind corners and half the path length of step t (t >= 1), and the shift of
+// the plane written at step t, i.e. the corner offsets (ix0, iy0) of step t+1
 // (t <= nz-2).
 template <typename T>
 struct alignas(16) PlaneStep {
@@ -57,35 +57,48 @@ struct alignas(16) PlaneStep {
     int sx, sy;   // (16-byte aligned and padded: loaded as whole vectors)
 };
 
-// Slot flags of the shifted-plane sweep.
-namespace plane {
-constexpr int kHasB = 1;    // the slot has a second frequency
-constexpr int kShared = 2;  // the second frequency has the first one's phi
-}  // namespace plane
+// The same for the two-level shifted-plane sweep (plane_sweep.cuh), whose
+// interpolation takes the two directions one after the other, scaled by the
+// larger weight of each: H = A + rx B, V = H + ry H', upwind value = c V.
+template <typename T>
+struct alignas(16) PlaneLerp {
+    T rx, ry, c, half_s;
+    int sx, sy;
+    int near;     // bit 0: the x + 1 column has the larger weight, bit 1: the y + 1 row
+};
 
-// One slot of the shifted-plane sweep: two frequencies (a, b) of a group.
+// One slot of the shifted-plane sweep: a mirror pair of frequencies, or the
+// line centre.
 template <typename T>
 struct PlaneSlot {
-    T phi_a, phi_b;      // profile values
-    T iphi_a, iphi_b;    // their inverses
-    T wphi_a, wphi_b;    // ray weight x frequency weight x profile (0: no frequency b)
-    T wu_a, wu_b;        // weight of u: wphi_a + wphi_b when a and b share phi, else own
-    int flags;           // bit 0: frequency b present; bit 1: b has a's phi
+    T phi, iphi;   // profile value and its inverse
+    T w;           // ray weight x sum of the frequencies' weights x profile (0: inactive)
+};
+
+// FP64: the same as operands of the integer weights (fixed_weights.cuh), a value
+// m 2^-64 2^e each.
+template <>
+struct PlaneSlot<double> {
+    double phi, iphi, w;
+    unsigned long long pm, ym, im;   // phi, phi log2(e), 1/phi
+    unsigned long long aq;           // w/phi in units of 2^(ea - 64); sum over a group < 2^64
+    int pe, ye, ie, ea;
+    int fx;                          // the exponents are within the integer weights' range
 };
 
 // Arguments of the shifted-plane sweep kernel (plane_sweep.cuh).
 template <typename T>
 struct PlaneArgs {
     int nx, ny, nz, rows, bands, ngroups;
-    int nslot_last;                      // active slots of the last group (0: all NP)
+    int nslot_last;                      // active slots of the last group
+    int ahead, chunks, ipad;             // of the launch's PlaneLayout (set by the launch)
     unsigned up_mask;                    // bit r set when ray r points up
     unsigned long long rmagic, xmagic;   // band_magic(rows), band_magic(nx)
     const T *chi0, *S, *bbot;            // [nvox], [nvox], [nx*ny]
-    const PlaneStep<T> *steps;           // [kRays][nz]
+    const PlaneLerp<T> *steps;           // [kRays][nz]
     const PlaneSlot<T> *slots;           // [ngroups][NP]
     T *pj, *pu;                          // [kRays*ngroups][nvox] partial Jeff and U
-    const double *exp_tab;               // FP64 exp table (FP64 sweeps)
-    double exp_l1, exp_l2;
+    const unsigned long long *fx_tab;    // tables of the integer weights (FP64 sweeps)
     unsigned *status;                    // kPlaneStatus* bits (async scheme), nullable
 };
 
@@ -93,19 +106,28 @@ struct PlaneArgs {
 // ran out (the launch's results are not valid).
 constexpr unsigned kPlaneStatusWait = 1u;
 
-// Slot counts (frequency pairs per group) the shifted-plane sweep is built for.
+// Slot counts (mirror pairs per group) the shifted-plane sweep is built for.
 constexpr int kPlaneNp[] = {1, 2, 3, 5, 8};
 constexpr int kPlaneNpCount = 5;
-constexpr size_t kMaxPlaneSmem = 224 * 1024;   // dynamic; static use stays below 3 KB
+// dynamic shared memory limit; static use stays below 6 KB (FP64) and 3 KB (FP32)
+__host__ __device__ constexpr size_t plane_smem_max(bool fp64) { return (fp64 ? 221 : 224) * 1024; }
 constexpr int kPlaneMaxThreads = 1024;
 // nodes a thread of the shifted-plane sweep takes per step (band <= this x
-// threads): the node loop is unrolled over them, which costs registers where
-// the compiler overlaps them (FP32 with more than two slots: two nodes)
+// threads)
 __host__ __device__ constexpr int plane_max_pass(int np, bool fp64) {
     return fp64 || np <= 2 ? 4 : 2;
 }
 bool plane_np_supported(int np);
-size_t plane_smem_bytes(int prec, int np, int rows, int nx);
+// How a block of `threads` threads works on its band of rows x nx nodes and
+// what it keeps in shared memory.
+struct PlaneLayout {
+    int item_rows;   // neighbouring rows a thread takes together (1 or 2)
+    int chunks;      // groups of threads that share the slots of a node
+    int ipad;        // threads of a group (whole warps)
+    int ahead;       // chi0 and S of the band are copied two steps ahead
+    size_t smem;     // dynamic shared memory, bytes
+};
+PlaneLayout plane_layout(int prec, int np, int rows, int nx, int threads);
 cudaError_t launch_plane_sweep_f64(const PlaneArgs<double> &a, const SweepShape &s,
                                    cudaStream_t st);
 cudaError_t launch_plane_sweep_f32(const PlaneArgs<float> &a, const SweepShape &s,

@@ -36,28 +36,52 @@
 // kernel records MG3D_STATUS_WAIT in the status word, stops waiting and runs
 // to the end, so the host reports an error instead of a hung launch.
 //
-// Channels: per stored node the intensities of the group's frequencies in
-// slot order, then chi0 and S of the node's plane (so the upwind chi0 and S
-// are interpolated with the intensities, from the same corners), padded to
-// whole 16-byte vectors; the node stride is an odd number of vectors, so the
-// 16-byte loads of a warp's consecutive nodes do not conflict in banks.
+// Slots: for the two-level atom in complete redistribution phi(x) = phi(-x)
+// and S does not depend on frequency, so in a static atmosphere the transfer
+// equation, its boundary values and its coefficients are the same at x and -x
+// and so is the intensity, bit for bit.  A slot stands for such a mirror pair
+// (or for the line centre): its intensity is solved once and enters the sums
+// with the weight of both frequencies.
 //
-// Slots: frequencies are taken in pairs.  For the two-level atom phi(x) =
-// phi(-x), so a pair of mirror frequencies shares the optical depth of every
-// short characteristic and hence the weights e^-x, w0, w_up, u (evaluated once
-// per slot); a slot whose two frequencies differ in phi evaluates them twice,
-// a slot of one frequency leaves its second channel unused.
+// Channels: per stored node chi0 and S of the node's plane (their upwind values
+// come from the same corners), then the intensities of the group's slots,
+// padded to whole 16-byte vectors.  Vector v of all nodes of a frame is
+// contiguous, so the 16-byte loads and stores of a warp's consecutive nodes do
+// not conflict in banks and a frame holds no padding between nodes.
 //
-// Per node the block accumulates, over its frequencies,
+// Interpolation.  The bilinear weights are the same for all nodes of a step, so
+// the two directions are taken one after the other and scaled by the larger
+// weight of each: H = A + rx B along x, V = H + ry H' along y, upwind value =
+// c V with c the product of the larger weights (0 <= rx, ry <= 1, 1/4 <= c <= 1).
+// A thread takes two nodes of neighbouring rows, which share the H of the row
+// between them: 2.5 fused multiply-adds and 3 corner loads per channel and node
+// instead of 4 and 4.
+//
+// What bounds it, and what it measured (GB300, one sweep, 9 frequencies; before:
+// the pairs solved twice, one row per thread, FP64 weights in FP64):
+//   FP64 64x64x129: 45 FP64 operations per node and ray (before 154) on a pipe
+//     that issues one warp instruction in 18 clocks; 5.01 -> 1.93 ms.  Small
+//     FP64 planes are the latency of one warp's slots, which the chunks below
+//     run side by side: 16x16x33 220 -> 110 us.
+//   FP32: issue slots and the wait for the slowest block of a plane; 64x64x129
+//     344 -> 300 us, 128x128x129 1527 -> 980 us.
+//
+// Per node the block accumulates, over its slots,
 //   Jeff = sum w phi (I - w0 S)   and   U = sum w phi (1 - w0)
 // (Sec. 2.1, the diagonal operator of MALI) into the partial slot of its
 // (ray, group); the rate kernel adds the slots in a fixed order.
+//
+// chi0 and S of the block's own nodes on the next plane are copied to shared
+// memory two steps ahead (cp.async), with the step's constants, so their latency
+// overlaps the steps before; where the shape
+// leaves no room for that they are read from global memory where used.
 #pragma once
 
 #include <cooperative_groups.h>
 
 #include <type_traits>
 
+#include "fixed_weights.cuh"
 #include "mg3d_internal.h"
 #include "sc_step.cuh"
 
@@ -67,15 +91,10 @@ namespace plane {
 
 template <typename T>
 __host__ __device__ constexpr int vec_width() { return 16 / (int)sizeof(T); }
-// channels per node: 2 NP intensities, chi0, S, padded to whole vectors
+// 16-byte vectors per node: chi0, S and NP intensities
 template <typename T, int NP>
-__host__ __device__ constexpr int channels() {
-    return (2 * NP + 2 + vec_width<T>() - 1) / vec_width<T>() * vec_width<T>();
-}
-// node stride in elements: an odd number of 16-byte vectors
-template <typename T, int NP>
-__host__ __device__ constexpr int node_stride() {
-    return ((channels<T, NP>() / vec_width<T>()) | 1) * vec_width<T>();
+__host__ __device__ constexpr int vectors() {
+    return (NP + 2 + vec_width<T>() - 1) / vec_width<T>();
 }
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) {
@@ -127,6 +146,15 @@ __device__ __forceinline__ void ld16(const double *p, double *o) {
     const double2 v = *reinterpret_cast<const double2 *>(p);
     o[0] = v.x;
     o[1] = v.y;
+}
+// The barrier in two halves: the release waits until the thread's earlier
+// stores are performed, so stores to global memory that no other block reads
+// go between the halves.
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait_acquire() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile(
@@ -203,6 +231,29 @@ static __device__ __noinline__ bool mbar_wait_bounded(unsigned bar, unsigned par
     }
 }
 
+// 4- or 8-byte copy from global to this block's shared memory
+__device__ __forceinline__ void cp_async(float *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async(double *dst, const double *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() {   // all of the thread's copies are done
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void cp_async_wait_but_last() {   // all but the last group
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
+
 __device__ __forceinline__ float ex2_approx(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -220,10 +271,7 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // Taylor series of w0 and w_up (e^-x = 1 - w0 - w_up) replace it.
 //   FP32: e^-x = 2^(-x log2 e) and 1/x by the hardware approximations (within
 //   2 ulp, ample for the FP32 formal solution); series below x = 0.1.
-//   FP64: Tang's table-driven e^-x (exp_neg) and 1/x from the caller
-//   (1/dtau0 times 1/phi); series below x ~ 1e-3, tested on the high word of x
-//   (a positive double orders like its bit pattern), which keeps the test off
-//   the FP64 pipe.
+//   FP64: 64-bit integer arithmetic (fixed_weights.cuh).
 struct Weights32 {
     static __device__ __forceinline__ void series(float x, float &ex, float &w0, float &wup,
                                                   float &u) {
@@ -234,85 +282,55 @@ struct Weights32 {
         u = 1.0f - w0;
         ex = u - wup;
     }
-    static __device__ __forceinline__ void closed(float x, float, const ExpNegTable &, float &ex,
-                                                  float &w0, float &wup, float &u) {
+    static __device__ __forceinline__ void closed(float x, float &ex, float &w0, float &wup,
+                                                  float &u) {
         ex = ex2_approx(x * -1.44269504088896341f);
         const float ix = rcp_approx(x);
         u = fmaf(-ex, ix, ix);
         w0 = 1.0f - u;
         wup = u - ex;
     }
-    static __device__ __forceinline__ void eval(float x, float ix, const ExpNegTable &et,
-                                                float &ex, float &w0, float &wup, float &u) {
+    static __device__ __forceinline__ void eval(float x, float &ex, float &w0, float &wup,
+                                                float &u) {
         if (x < 0.1f) series(x, ex, w0, wup, u);
-        else closed(x, ix, et, ex, w0, wup, u);
+        else closed(x, ex, w0, wup, u);
     }
 };
 
+// FP64 weights for the arguments the integer weights (fixed_weights.cuh) leave
+// out: optical paths that are zero, denormal, beyond 2^700, negative or NaN.  The
+// series (below 1e-3, tested on the high word of x) as products with rounded
+// reciprocals.
 struct Weights64 {
-    static __device__ __forceinline__ void series(double x, double &ex, double &w0, double &wup,
-                                                  double &u) {
-        // the coefficients as products with the rounded reciprocals: a division
-        // would cost an FP64 reciprocal iteration each
-        w0 = x * (0.5 - x * (1.0 / 6.0 - x * (1.0 / 24.0 - x * (1.0 / 120.0 - x * (1.0 / 720.0)))));
-        wup = x * (0.5 - x * (1.0 / 3.0 - x * (1.0 / 8.0 - x * (1.0 / 30.0 - x * (1.0 / 144.0)))));
-        u = 1.0 - w0;
-        ex = u - wup;
-    }
-    static __device__ __forceinline__ void closed(double x, double inv_x, const ExpNegTable &et,
-                                                  double &ex, double &w0, double &wup,
-                                                  double &u) {
-        ex = exp_neg_hi(x, et);
-        u = fma(-ex, inv_x, inv_x);
-        w0 = 1.0 - u;
-        wup = u - ex;
-    }
-    static __device__ __forceinline__ void eval(double x, double inv_x, const ExpNegTable &et,
-                                                double &ex, double &w0, double &wup, double &u) {
-        // 0x3F50624D is the high word of 1e-3: x below 1e-3 (up to the low word)
-        if (__double2hiint(x) < 0x3F50624D) series(x, ex, w0, wup, u);
-        else closed(x, inv_x, et, ex, w0, wup, u);
-    }
+    double ex, w0, wup, u;
 };
-
-template <typename T>
-struct WeightsOf;
-template <>
-struct WeightsOf<float> {
-    using W = Weights32;
-};
-template <>
-struct WeightsOf<double> {
-    using W = Weights64;
-};
-
-// 1/dtau0 for the FP64 weights (FP32 takes 1/x per slot instead): the
-// hardware approximation of the reciprocal (about 23 correct bits) refined by
-// two Newton-Raphson steps r <- r + r (1 - d r), each of which doubles the
-// correct bits, so the result is within about an ulp (the closed-form weights
-// only use it where x >= 1e-3, where dtau0 is far from 0 and from overflow).
-__device__ __forceinline__ double node_rcp(double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-d, r, 1.0);
-    return fma(r, e, r);
+static __device__ __noinline__ Weights64 weights64(double x) {
+    Weights64 w;
+    if (__double2hiint(x) < 0x3F50624D) {
+        w.w0 = x * (0.5 - x * (1.0 / 6.0 - x * (1.0 / 24.0 - x * (1.0 / 120.0 - x * (1.0 / 720.0)))));
+        w.wup = x * (0.5 - x * (1.0 / 3.0 - x * (1.0 / 8.0 - x * (1.0 / 30.0 - x * (1.0 / 144.0)))));
+        w.u = 1.0 - w.w0;
+        w.ex = w.u - w.wup;
+    } else {
+        const double ix = 1.0 / x;
+        w.ex = exp(-x);
+        w.u = fma(-w.ex, ix, ix);
+        w.w0 = 1.0 - w.u;
+        w.wup = w.u - w.ex;
+    }
+    return w;
 }
-__device__ __forceinline__ float node_rcp(float) { return 0.0f; }
 
 }  // namespace plane
 
 // The body of the kernel for ray blockIdx.z and frequency group blockIdx.y.
-template <typename T, int NP, bool AS>
+// R: rows of a thread's item.
+template <typename T, int NP, int R, bool AS>
 __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     using namespace plane;
     constexpr int VW = vec_width<T>();
-    constexpr int NCH = channels<T, NP>();
-    constexpr int NV = NCH / VW;
-    constexpr int CS = node_stride<T, NP>();
-    constexpr int CHI = 2 * NP, SRC = 2 * NP + 1;
-    using W = typename WeightsOf<T>::W;
+    constexpr int NV = vectors<T, NP>();
+    constexpr bool F64 = sizeof(T) == 8;
 
     const int r = blockIdx.z, g = blockIdx.y;
     const int nb = a.bands;
@@ -323,8 +341,9 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     const int y0 = rank * rows;
     const int myrows = min(rows, ny - y0);
     const int lastrows = ny - (nb - 1) * rows;   // rows of the last band
-    const int pitch = (nx + 1) * CS;             // one stored row, elements
-    const int plane_el = (rows + 1) * pitch;     // one stored plane, elements
+    const unsigned pitch = (unsigned)(nx + 1) * 16;      // one stored row of a vector, bytes
+    const unsigned vs = (unsigned)(rows + 1) * pitch;    // one vector of a frame
+    const unsigned frame = NV * vs;                      // one stored frame
     const int nplane = nx * ny;                  // the host keeps nvox below 2^31
     const bool up = (a.up_mask >> r) & 1u;
     const long slot = (long)r * a.ngroups + g;
@@ -333,10 +352,13 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     const PlaneSlot<T> *__restrict__ gs = a.slots + (long)g * NP;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *buf = reinterpret_cast<T *>(smem_raw);
-    const unsigned buf_addr = smem_addr(buf);
-    __shared__ double exp_tab[kExpTab];
+    const unsigned buf_addr = smem_addr(smem_raw);
+    // chi0 and S of the band's nodes two steps ahead: [3][2][rows * nx]
+    T *ahead = reinterpret_cast<T *>(smem_raw + 2 * (size_t)frame);
+    __shared__ fx::u64 fx_tab[F64 ? 2 * fx::kTab : 1];   // tables of the integer weights
     __shared__ PlaneSlot<T> stab[NP];
+    // step constants two steps ahead
+    __shared__ __align__(16) PlaneLerp<T> step_ring[4];
     // async scheme: one mbarrier per plane buffer, one phase per filling
     __shared__ __align__(8) unsigned long long full_bar[2];
     const unsigned bar_addr = smem_addr(full_bar);
@@ -345,140 +367,153 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
         mbar_init(bar_addr + 8, 1);
         mbar_init_fence();
     }
-    if (sizeof(T) == 8)
-        for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) exp_tab[i] = a.exp_tab[i];
+    if (F64)
+        for (int i = threadIdx.x; i < 2 * fx::kTab; i += blockDim.x) fx_tab[i] = a.fx_tab[i];
     for (int i = threadIdx.x; i < NP; i += blockDim.x) stab[i] = gs[i];
     __syncthreads();
-    const ExpNegTable et{exp_tab, a.exp_l1, a.exp_l2};
-    const int nslot = a.nslot_last > 0 && g == a.ngroups - 1 ? a.nslot_last : NP;
-
-    // Block-uniform slot facts.  The fast path covers groups whose NP slots
-    // are all active and mirror pairs (equal phi and w phi), except that the
-    // last slot may hold one frequency (the line centre); other groups take
-    // the general path with per-slot tests.
-    T wsum = 0, phimin = 0, phimax = 0;
-    bool fast = nslot == NP;
+    const int nslot = g == a.ngroups - 1 ? a.nslot_last : NP;
+    T wsum = 0;
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        const int fl = stab[p].flags;
-        wsum += stab[p].wphi_a + stab[p].wphi_b;
-        if (p < nslot) {
-            const T ph = stab[p].phi_a;
-            phimin = p == 0 ? ph : min(phimin, ph);
-            phimax = p == 0 ? ph : max(phimax, ph);
-            if (fl & kHasB) {
-                phimin = min(phimin, stab[p].phi_b);
-                phimax = max(phimax, stab[p].phi_b);
-            }
-        }
-        if (p < NP - 1 && fl != (kHasB | kShared)) fast = false;
-        if ((fl & kHasB) && (!(fl & kShared) || stab[p].wphi_a != stab[p].wphi_b)) fast = false;
-    }
-    const bool lastb = (stab[NP - 1].flags & kHasB) != 0;
+    for (int p = 0; p < NP; ++p) wsum += stab[p].w;
 
-    // FP32 keeps the slot tables in registers for the whole sweep; FP64 (bound
-    // by its FP64 pipe, not by issue) reads them from shared memory where used
-    constexpr bool kRegTabs = sizeof(T) == 4;
-    T r_phi[NP], r_wa[NP], r_wu[NP];
+    // FP32 keeps the slot tables in registers, an inactive slot as one of weight
+    // zero, and knows the dtau0 from which all slots take the closed form or
+    // below which all take the series (0.1 over the smallest and largest phi).
+    T r_phi[F64 ? 1 : NP], r_w[F64 ? 1 : NP], d_closed = 0, d_series = 0;
+    if constexpr (!F64) {
+        T lo = stab[0].phi, hi = stab[0].phi;
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        if (kRegTabs) {
-            r_phi[p] = stab[p].phi_a;
-            r_wa[p] = stab[p].wphi_a;
-            r_wu[p] = stab[p].wu_a;
+        for (int p = 0; p < NP; ++p) {
+            r_phi[p] = p < nslot ? stab[p].phi : stab[0].phi;
+            r_w[p] = stab[p].w;
+            lo = min(lo, r_phi[p]);
+            hi = max(hi, r_phi[p]);
         }
+        d_closed = T(0.1) / lo;
+        d_series = T(0.1) / hi;
     }
-    auto phi_a = [&](int p) { return kRegTabs ? r_phi[p] : stab[p].phi_a; };
-    auto wphi_a = [&](int p) { return kRegTabs ? r_wa[p] : stab[p].wphi_a; };
-    auto wu_a = [&](int p) { return kRegTabs ? r_wu[p] : stab[p].wu_a; };
 
-    // The nodes of this thread, the same at every step: q = tid + i*nth for
-    // i < MAXP (the host keeps the band within that many passes).
-    constexpr int MAXP = plane_max_pass(NP, sizeof(T) == 8);
-    const int band = myrows * nx;
+    // A thread's item is column x of rows yl0 .. yl0 + nr - 1 of the band.  With
+    // more than one chunk (small bands) `ipad` threads take the items of each
+    // chunk of the slots, so that the slots of a node run side by side; their
+    // sums meet in shared memory one step later.
     const int nth = blockDim.x;
-    bool valid[MAXP];
-    int xq[MAXP], yq[MAXP], nodeq[MAXP], corq[MAXP];
-#pragma unroll
-    for (int i = 0; i < MAXP; ++i) {
-        const int q = threadIdx.x + i * nth;
-        valid[i] = q < band;
-        const int yl = band_of(valid[i] ? q : 0, a.xmagic);
-        xq[i] = (valid[i] ? q : 0) - yl * nx;
-        yq[i] = y0 + yl;
-        nodeq[i] = yq[i] * nx + xq[i];
-        corq[i] = yl * pitch + xq[i] * CS;
-    }
+    const int items = (myrows + R - 1) / R * nx;
+    const int chunks = a.chunks;
+    const int ipad = a.ipad;
+    const int chunk = chunks > 1 ? (int)threadIdx.x / ipad : 0;
+    const int q0 = threadIdx.x - chunk * ipad;
+    const int qend = chunk < chunks ? items : 0;
+    // vectors 1 .. NV-1 of the chunk (the first chunk also takes vector 0)
+    const int v_begin = 1 + (NV - 1) * chunk / chunks;
+    const int v_end = 1 + (NV - 1) * (chunk + 1) / chunks;
+    T *red = ahead + (a.ahead ? 6 * rows * nx : 0);   // [2][chunks][rows * nx][2]
+    auto item_at = [&](int q, int &x, int &yl0, int &nr) {
+        const int gy = band_of(q, a.xmagic);
+        x = q - gy * nx;
+        yl0 = gy * R;
+        nr = min(R, myrows - yl0);
+    };
+    // Jeff and U of the plane of step t from the chunks' sums, in chunk order
+    auto flush_sums = [&](int t) {
+        const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
+        const T *src = red + (t & 1) * 2 * chunks * rows * nx;
+        for (int o = threadIdx.x; o < myrows * nx; o += nth) {
+            T j = src[2 * o], u = src[2 * o + 1];
+            for (int c = 1; c < chunks; ++c) {
+                j += src[2 * (c * rows * nx + o)];
+                u += src[2 * (c * rows * nx + o) + 1];
+            }
+            pj[kp + o] = j;
+            pu[kp + o] = u;
+        }
+    };
 
-    // Stores the channels of node (x, y) into the frame of the next step,
-    // shifted by (sx, sy), in buffer `par`, with its pad and halo copies
-    // (predicated stores: a node of column 0 also fills the pad column, a
-    // node of a band's first row also the halo row of the band before it).
-    auto store_node = [&](const T *ch, int x, int y, int sx, int sy, int par) {
-        int xs = x - sx;
-        xs += xs < 0 ? nx : 0;
-        int ys = y - sy;
+    // Where a node (x, yl) of the band goes in the frame of the next step,
+    // shifted by (sx, sy), in buffer `par`.  A node of column 0 also fills the
+    // pad column, a node of a band's first row also the halo row of the band
+    // before it; few nodes are either, so the copies are behind one branch.
+    struct Dest {
+        unsigned base;     // of vector 0 in the block that owns the row
+        int ob, lr, xs;    // that block, the row in its band, the column
+    };
+    const unsigned padoff = (unsigned)nx * 16;
+    auto dest_of = [&](int x, int yl, int sx, int sy, int par) {
+        Dest d;
+        d.xs = x - sx;
+        d.xs += d.xs < 0 ? nx : 0;
+        int ys = y0 + yl - sy;
         ys += ys < 0 ? ny : 0;
-        const int ob = band_of(ys, a.rmagic);
-        const int lr = ys - ob * rows;
-        const int hb = ob == 0 ? nb - 1 : ob - 1;   // the band whose halo row is ys
-        const int hr = hb == nb - 1 ? lastrows : rows;
-        const unsigned col = (unsigned)((par * plane_el + xs * CS) * (int)sizeof(T));
-        const unsigned base = cluster_addr(buf_addr, (unsigned)ob) +
-                              col + (unsigned)(lr * pitch * (int)sizeof(T));
-        const unsigned hbase = cluster_addr(buf_addr, (unsigned)hb) +
-                               col + (unsigned)(hr * pitch * (int)sizeof(T));
-        const unsigned padoff = (unsigned)(nx * CS * (int)sizeof(T));
-        const bool pad = xs == 0, halo = lr == 0;
+        d.ob = band_of(ys, a.rmagic);
+        d.lr = ys - d.ob * rows;
+        d.base = cluster_addr(buf_addr, (unsigned)d.ob) + par * frame + (unsigned)d.lr * pitch +
+                 (unsigned)d.xs * 16;
+        return d;
+    };
+    // one copy of vectors v0 .. v0+N-1 at byte offset `off` of block `ob`
+    auto store_to = [&](auto n_tag, unsigned addr, int ob, int par, int v0, const T *cv) {
+        constexpr int N = decltype(n_tag)::value;
         if constexpr (AS) {
-            if (as) {
-                // to another block: st.async counted on that block's mbarrier
-                // of buffer `par`; within the block: plain stores
+            // to another block: st.async counted on that block's mbarrier of
+            // the buffer; within the block: plain stores
+            if (as && ob != rank) {
                 const unsigned bar = cluster_addr(bar_addr + 8u * par, (unsigned)ob);
-                const unsigned hbar = cluster_addr(bar_addr + 8u * par, (unsigned)hb);
-                const bool rem = ob != rank, hrem = hb != rank;
 #pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    const T *cv = ch + v * VW;
-                    if (rem) {
-                        st16_async_if(true, base + v * 16, cv, bar);
-                        st16_async_if(pad, base + padoff + v * 16, cv, bar);
-                    } else {
-                        st16(base + v * 16, cv);
-                        st16_if(pad, base + padoff + v * 16, cv);
-                    }
-                    if (hrem) {
-                        st16_async_if(halo, hbase + v * 16, cv, hbar);
-                        st16_async_if(halo && pad, hbase + padoff + v * 16, cv, hbar);
-                    } else {
-                        st16_if(halo, hbase + v * 16, cv);
-                        st16_if(halo && pad, hbase + padoff + v * 16, cv);
-                    }
-                }
+                for (int v = 0; v < N; ++v)
+                    st16_async_if(true, addr + (v0 + v) * vs, cv + v * VW, bar);
                 return;
             }
         }
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            st16(base + v * 16, ch + v * VW);
-            st16_if(pad, base + padoff + v * 16, ch + v * VW);
-            st16_if(halo, hbase + v * 16, ch + v * VW);
-            st16_if(halo && pad, hbase + padoff + v * 16, ch + v * VW);
+        for (int v = 0; v < N; ++v) st16(addr + (v0 + v) * vs, cv + v * VW);
+    };
+    // vectors v0 .. v0+N-1 of the node's channels, with the copies
+    auto put = [&](auto n_tag, const Dest &d, int par, int v0, const T *cv) {
+        store_to(n_tag, d.base, d.ob, par, v0, cv);
+        if (d.xs == 0 || d.lr == 0) {
+            if (d.xs == 0) store_to(n_tag, d.base + padoff, d.ob, par, v0, cv);
+            if (d.lr == 0) {
+                const int hb = d.ob == 0 ? nb - 1 : d.ob - 1;   // the band before
+                const unsigned h = cluster_addr(buf_addr, (unsigned)hb) + par * frame +
+                                   (unsigned)(hb == nb - 1 ? lastrows : rows) * pitch +
+                                   (unsigned)d.xs * 16;
+                store_to(n_tag, h, hb, par, v0, cv);
+                if (d.xs == 0) store_to(n_tag, h + padoff, hb, par, v0, cv);
+            }
         }
     };
+    using One = std::integral_constant<int, 1>;
+    using All = std::integral_constant<int, NV>;
 
-    // chi0 and S of the thread's nodes on the next plane are loaded one step
-    // ahead into registers, so that the global-memory latency overlaps the
-    // current step and the barrier instead of opening each step.
-    T nchi[MAXP], nS[MAXP];
-    auto prefetch = [&](int t) {
-        const int kp = (up ? t : nz - 1 - t) * nplane;
-#pragma unroll
-        for (int i = 0; i < MAXP; ++i)
-            if (valid[i]) {
-                nchi[i] = a.chi0[kp + nodeq[i]];
-                nS[i] = a.S[kp + nodeq[i]];
+    // chi0 and S of step t's plane into part t mod 3 of the ring, and the
+    // constants of step t
+    auto prefetch = [&](int t, int part) {
+        constexpr int NC = sizeof(PlaneLerp<T>) / 16;
+        if (threadIdx.x < NC)
+            cp_async16(reinterpret_cast<unsigned char *>(&step_ring[t & 3]) + 16 * threadIdx.x,
+                       reinterpret_cast<const unsigned char *>(&a.steps[(long)r * nz + t]) +
+                           16 * threadIdx.x);
+        if (a.ahead) {
+            const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
+            T *dst = ahead + part * 2 * rows * nx;
+            for (int o = threadIdx.x; o < myrows * nx; o += nth) {
+                cp_async(dst + o, a.chi0 + kp + o);
+                cp_async(dst + rows * nx + o, a.S + kp + o);
             }
+        }
+        cp_async_commit();
+    };
+    // chi0 and S of node o of the band on the plane of step t, part t mod 3
+    auto local = [&](int t, int part, int o, T &chi, T &S) {
+        if (a.ahead) {
+            const T *src = ahead + part * 2 * rows * nx;
+            chi = src[o];
+            S = src[rows * nx + o];
+        } else {
+            const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
+            chi = a.chi0[kp + o];
+            S = a.S[kp + o];
+        }
     };
 
     // Async scheme: the bytes buffer `par` of this block receives from other
@@ -516,230 +551,310 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
 
     // ---- entering boundary plane: I prescribed (bottom: Planck at the local
     // temperature, top: zero), so w0 = 0 and 1 - w0 = 1
-    prefetch(0);
+    if (nz > 1) prefetch(1, 1);
+    if (nz > 2) prefetch(2, 2);
     {
-        const int k0 = (up ? 0 : nz - 1) * nplane;
-        const PlaneStep<T> sp = a.steps[(long)r * nz];
+        const int k0 = (up ? 0 : nz - 1) * nplane + y0 * nx;
+        const PlaneLerp<T> sp = a.steps[(long)r * nz];
+        for (int q = threadIdx.x; q < items; q += nth) {
+            int x, yl0, nr;
+            item_at(q, x, yl0, nr);
+            for (int j = 0; j < nr; ++j) {
+                const int o = (yl0 + j) * nx + x;
+                const T Ib = up ? a.bbot[y0 * nx + o] : T(0);
+                pj[k0 + o] = Ib * wsum;
+                pu[k0 + o] = wsum;
+                if (nz > 1) {
+                    const Dest d = dest_of(x, yl0 + j, sp.sx, sp.sy, 0);
+                    T cv[NV * VW];
 #pragma unroll
-        for (int i = 0; i < MAXP; ++i) {
-            if (!valid[i]) continue;
-            const T Ib = up ? a.bbot[nodeq[i]] : T(0);
-            T ch[NCH];
-#pragma unroll
-            for (int c = 0; c < NCH; ++c) ch[c] = c < 2 * NP ? Ib : T(0);
-            ch[CHI] = nchi[i];
-            ch[SRC] = nS[i];
-            pj[k0 + nodeq[i]] = Ib * wsum;
-            pu[k0 + nodeq[i]] = wsum;
-            if (nz > 1) store_node(ch, xq[i], yq[i], sp.sx, sp.sy, 0);
+                    for (int e = 0; e < NV * VW; ++e) cv[e] = Ib;
+                    cv[0] = a.chi0[k0 + o];
+                    cv[1] = a.S[k0 + o];
+                    put(All{}, d, 0, 0, cv);
+                }
+            }
         }
     }
-    if (nz > 1) prefetch(1);
+    cp_async_wait();
     if (cl && !as) cluster_barrier();
     else __syncthreads();
 
-    // Regime of a node's weights: every slot in closed form, every slot by
-    // series, or a per-slot choice.  FP32 compares dtau0 with the thresholds
-    // 0.1/phi_min and 0.1/phi_max; FP64 compares the high words of dtau0 and
-    // of 1e-3/phi (integer compares, off the FP64 pipe), a conservative test
-    // whose border cases take the per-slot choice.
-    const T thr = sizeof(T) == 8 ? T(1e-3) : T(0.1);
-    const T d_all_closed = thr / phimin, d_all_series = thr / phimax;
-    const int hi_closed = sizeof(T) == 8 ? __double2hiint((double)d_all_closed) : 0;
-    const int hi_series = sizeof(T) == 8 ? __double2hiint((double)d_all_series) : 0;
-    auto regime = [&](T dtau0) {   // 0 closed, 1 series, 2 mixed
-        if constexpr (sizeof(T) == 8) {
-            const int hd = __double2hiint((double)dtau0);
-            return hd > hi_closed ? 0 : (hd < hi_series ? 1 : 2);
-        } else {
-            return dtau0 >= d_all_closed ? 0 : (dtau0 < d_all_series ? 1 : 2);
+    int part = 1;   // t mod 3
+    for (int t = 1; t < nz; ++t) {
+        const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
+        const unsigned char *prev = smem_raw + ((t - 1) & 1) * (size_t)frame;
+        const PlaneLerp<T> sp = step_ring[t & 3];
+        const bool write = t + 1 < nz;
+        // part (t + 2) mod 3 was last read at step t - 1
+        if (t + 2 < nz) prefetch(t + 2, part == 0 ? 2 : part - 1);
+        if (chunks > 1 && t > 1) flush_sums(t - 1);
+        if (as) {
+            // the other blocks' part of the plane stored at step t - 1
+            wait_fill(t - 1);
+            if (write) {
+                expect_fill(sp.sy, t & 1);
+                // every block's reads of this buffer (step t - 1) are over
+                if (t >= 2) cluster_wait();
+            }
         }
-    };
-
-    auto run = [&](auto fast_tag) {
-        constexpr bool FAST = decltype(fast_tag)::value;
-        // channel c is interpolated when it carries a frequency of an active
-        // slot, or chi0 or S; the others (the second channel of a
-        // one-frequency slot, slots past the last group's end, padding) hold 0
-        auto live = [&](int c) {
-            if (c == CHI || c == SRC) return true;
-            if (c >= 2 * NP) return false;
-            if (FAST) return c != 2 * NP - 1 || lastb;
-            const int p = c >> 1;
-            return p < nslot && ((c & 1) == 0 || (stab[p].flags & kHasB));
-        };
-        // the step constants are loaded one step ahead as well
-        PlaneStep<T> sp_next = a.steps[(long)r * nz + (nz > 1 ? 1 : 0)];
-        for (int t = 1; t < nz; ++t) {
-            const int kp = (up ? t : nz - 1 - t) * nplane;
-            const T *prev = buf + ((t - 1) & 1) * plane_el;
-            const PlaneStep<T> sp = sp_next;
-            const bool write = t + 1 < nz;
-            if (write) sp_next = a.steps[(long)r * nz + t + 1];
-            T cchi[MAXP], cS[MAXP];
+        // the nearer column and row first: H = A + rx B, V = H + ry H'
+        const unsigned near_x = (sp.near & 1) ? 16u : 0u, far_x = 16u - near_x;
+        const bool down = sp.near & 2;   // the nearer row is the higher one
+        fx::u64 cm = 0;   // FP64: c = (cm, ce)
+        int ce = 0;
+        if constexpr (F64) fx::unpack(sp.c, &cm, &ce);
+        // Jeff and U of the thread's first item, stored after the barrier's first half
+        T kj[R], ku[R];
+        int ko[R], nk = 0;
+        for (int q = q0; q < qend; q += nth) {
+            int x, yl0, nr;
+            item_at(q, x, yl0, nr);
+            // rows in the order they are needed: node j of the item lies
+            // between row j (nearer) and row j + 1 of the walk
+            const unsigned char *row0 =
+                prev + (unsigned)(down ? yl0 + nr : yl0) * pitch + (unsigned)x * 16;
+            const int dpitch = down ? -(int)pitch : (int)pitch;
+            auto row_h = [&](int v, int k, T *h) {
+                const unsigned char *p = row0 + k * dpitch + v * vs;
+                T A[VW], B[VW];
+                ld16(reinterpret_cast<const T *>(p + near_x), A);
+                ld16(reinterpret_cast<const T *>(p + far_x), B);
 #pragma unroll
-            for (int i = 0; i < MAXP; ++i) {
-                cchi[i] = nchi[i];
-                cS[i] = nS[i];
-            }
-            if (write) prefetch(t + 1);
-            if (as) {
-                // the other blocks' part of the plane stored at step t - 1
-                wait_fill(t - 1);
-                if (write) {
-                    expect_fill(sp.sy, t & 1);
-                    // every block's reads of this buffer (step t - 1) are over
-                    if (t >= 2) cluster_wait();
-                }
-            }
+                for (int e = 0; e < VW; ++e) h[e] = fma(sp.rx, B[e], A[e]);
+            };
+            if constexpr (!F64) {
+                // FP32: all channels of a node at once, the slots unrolled
+                T h0[NV * VW], h1[NV * VW];
 #pragma unroll
-            for (int i = 0; i < MAXP; ++i) {
-                // FP64 takes its nodes one after the other (its pipe, not
-                // latency, bounds it, and overlapping two nodes would spill)
-                if (sizeof(T) == 8 && i > 0) asm volatile("" ::: "memory");
-                if (!valid[i]) continue;
-                const int v = kp + nodeq[i];
-                const T chi_loc = cchi[i];
-                const T S_loc = cS[i];
-                // the four upwind corners, interpolated channel by channel
-                const T *c00 = prev + corq[i];
-                const T *c10 = c00 + CS, *c01 = c00 + pitch, *c11 = c01 + CS;
-                T ch[NCH];
+                for (int v = 0; v < NV; ++v) row_h(v, 0, h0 + v * VW);
 #pragma unroll
-                for (int vv = 0; vv < NV; ++vv) {
-                    T A[VW], B[VW], C[VW], D[VW];
-                    ld16(c00 + vv * VW, A);
-                    ld16(c10 + vv * VW, B);
-                    ld16(c01 + vv * VW, C);
-                    ld16(c11 + vv * VW, D);
+                for (int j = 0; j < R; ++j) {
+                    if (j >= nr) break;
 #pragma unroll
-                    for (int e = 0; e < VW; ++e)
-                        ch[vv * VW + e] = live(vv * VW + e) ? sp.w00 * A[e] + sp.w10 * B[e] +
-                                                                  sp.w01 * C[e] + sp.w11 * D[e]
-                                                            : T(0);
-                }
-                const T chi_up = ch[CHI], S_up = ch[SRC];
-                const T dtau0 = (chi_up + chi_loc) * sp.half_s;
-                const T inv_dtau0 = node_rcp(dtau0);
-                T cj = 0, cu = 0;
-                // new intensities of slot p's frequencies from its weights
-                auto apply = [&](int p, bool two, T ex, T w0, T wup, T u) {
-                    cu = fma(wu_a(p), u, cu);
-                    const T wupS = wup * S_up;
-                    const T pa = fma(ch[2 * p], ex, wupS);
-                    if (two) {
-                        const T pb = fma(ch[2 * p + 1], ex, wupS);
-                        cj = fma(wphi_a(p), pa + pb, cj);
-                        ch[2 * p + 1] = fma(w0, S_loc, pb);
-                    } else {
-                        cj = fma(wphi_a(p), pa, cj);
+                    for (int v = 0; v < NV; ++v) row_h(v, j + 1, h1 + v * VW);
+                    T ch[NV * VW];
+#pragma unroll
+                    for (int c = 0; c < NV * VW; ++c) {
+                        ch[c] = c < NP + 2 ? fma(sp.ry, h1[c], h0[c]) : T(0);
+                        h0[c] = h1[c];
                     }
-                    ch[2 * p] = fma(w0, S_loc, pa);
-                };
-                if constexpr (FAST) {
-                    // every slot a mirror pair except possibly the last
+                    const int yl = down ? yl0 + nr - 1 - j : yl0 + j;
+                    T chi_loc, S_loc;
+                    local(t, part, yl * nx + x, chi_loc, S_loc);
+                    const T dtau0 = fma(sp.c, ch[0], chi_loc) * sp.half_s;
+                    const T S_up = ch[1] * sp.c;
+                    T cj = 0, cu = 0;
+                    // every slot in closed form (0), by series (1), or each its own
                     auto slots = [&](auto mode_tag) {
                         constexpr int MODE = decltype(mode_tag)::value;
 #pragma unroll
                         for (int p = 0; p < NP; ++p) {
-                            const T x = dtau0 * phi_a(p);
-                            const T ix = sizeof(T) == 8 ? inv_dtau0 * stab[p].iphi_a : T(0);
                             T ex, w0, wup, u;
-                            if (MODE == 0) W::closed(x, ix, et, ex, w0, wup, u);
-                            else if (MODE == 1) W::series(x, ex, w0, wup, u);
-                            else W::eval(x, ix, et, ex, w0, wup, u);
-                            apply(p, p < NP - 1 || lastb, ex, w0, wup, u);
+                            const T xt = dtau0 * r_phi[p];
+                            if (MODE == 0) Weights32::closed(xt, ex, w0, wup, u);
+                            else if (MODE == 1) Weights32::series(xt, ex, w0, wup, u);
+                            else Weights32::eval(xt, ex, w0, wup, u);
+                            cu = fma(r_w[p], u, cu);
+                            const T part = fma(ch[2 + p], sp.c * ex, wup * S_up);   // I - w0 S
+                            cj = fma(r_w[p], part, cj);
+                            ch[2 + p] = fma(w0, S_loc, part);
                         }
                     };
-                    const int rg = regime(dtau0);
-                    if (rg == 0) slots(std::integral_constant<int, 0>{});
-                    else if (rg == 1) slots(std::integral_constant<int, 1>{});
+                    if (dtau0 >= d_closed) slots(std::integral_constant<int, 0>{});
+                    else if (dtau0 < d_series) slots(std::integral_constant<int, 1>{});
                     else slots(std::integral_constant<int, 2>{});
-                } else {
+                    const int o = yl * nx + x;
+                    if (q == q0) {
+                        kj[j] = cj;
+                        ku[j] = cu;
+                        ko[j] = kp + o;
+                        nk = j + 1;
+                    } else {
+                        pj[kp + o] = cj;
+                        pu[kp + o] = cu;
+                    }
+                    if (write) {
+                        ch[0] = chi_loc;
+                        ch[1] = S_loc;
+                        put(All{}, dest_of(x, yl, sp.sx, sp.sy, t & 1), t & 1, 0, ch);
+                    }
+                }
+            } else {
+            // vector v interpolated at the item's nodes (without the factor c)
+            auto upwind = [&](int v, T (*o)[VW]) {
+                T h0[VW], h1[VW];
+                row_h(v, 0, h0);
 #pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        if (p >= nslot) continue;
-                        const int fl = stab[p].flags;
-                        T ex, w0, wup, u;
-                        W::eval(dtau0 * phi_a(p), sizeof(T) == 8 ? inv_dtau0 * stab[p].iphi_a : T(0),
-                                et, ex, w0, wup, u);
-                        cu = fma(wu_a(p), u, cu);
-                        T wupS = wup * S_up;
-                        T part = fma(ch[2 * p], ex, wupS);
-                        cj = fma(wphi_a(p), part, cj);
-                        ch[2 * p] = fma(w0, S_loc, part);
-                        if (fl & kHasB) {
-                            if (!(fl & kShared)) {
-                                W::eval(dtau0 * stab[p].phi_b,
-                                        sizeof(T) == 8 ? inv_dtau0 * stab[p].iphi_b : T(0), et,
-                                        ex, w0, wup, u);
-                                cu = fma(stab[p].wu_b, u, cu);
-                                wupS = wup * S_up;
-                            }
-                            part = fma(ch[2 * p + 1], ex, wupS);
-                            cj = fma(stab[p].wphi_b, part, cj);
-                            ch[2 * p + 1] = fma(w0, S_loc, part);
+                for (int j = 0; j < R; ++j) {
+                    if (j < nr) {
+                        row_h(v, j + 1, h1);
+#pragma unroll
+                        for (int e = 0; e < VW; ++e) {
+                            o[j][e] = fma(sp.ry, h1[e], h0[e]);
+                            h0[e] = h1[e];
                         }
                     }
                 }
-                pj[v] = cj;
-                pu[v] = cu;
-                if (write) {
-                    ch[CHI] = chi_loc;
-                    ch[SRC] = S_loc;
-                    store_node(ch, xq[i], yq[i], sp.sx, sp.sy, t & 1);
+            };
+            T V0[R][VW];
+            upwind(0, V0);
+            T S_up[R], S_loc[R], chi_loc[R], dtau0[R], cj[R], cu[R];
+            // FP64: dtau0 = (dm, de), 1/dtau0 = (dr, 1 - de), the sum of the
+            // slots' (w/phi)(1 - e^-x) in units of 2^(ea - 64)
+            fx::u64 dm[R], dr[R], ud[R];
+            int de[R];
+            bool dok[R];
+            Dest dst[R];
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (j < nr) {
+                    const int yl = down ? yl0 + nr - 1 - j : yl0 + j;
+                    local(t, part, yl * nx + x, chi_loc[j], S_loc[j]);
+                    S_up[j] = V0[j][1] * sp.c;
+                    dtau0[j] = fma(sp.c, V0[j][0], chi_loc[j]) * sp.half_s;
+                    dok[j] = fx::in_range(dtau0[j]);
+                    fx::unpack(dtau0[j], &dm[j], &de[j]);
+                    dr[j] = fx::recip(dm[j]);
+                    ud[j] = 0;
+                    cj[j] = cu[j] = T(0);
+                    if (write) dst[j] = dest_of(x, yl, sp.sx, sp.sy, t & 1);
                 }
             }
-            if (write) {
-                if (as) {
-                    __syncthreads();
-                    if (t + 2 < nz) cluster_arrive_relaxed();
-                } else if (cl) {
-                    cluster_barrier();
+            // slot p's new intensity at node j from the upwind sum i (without c)
+            auto step = [&](int j, int p, T i) {
+                const PlaneSlot<T> &sl = stab[p];
+                T cex, w0, wup;   // c e^-x, w0, w_up
+                if (dok[j] && sl.fx) {
+                    const int ex = de[j] + sl.pe;
+                    fx::Weights w;
+                    if (ex <= fx::kThinExp) {
+                        w = fx::thin(fx::mulhi(dm[j], sl.pm), ex);
+                        cu[j] = fma(sl.w, fx::pack(w.u, 0), cu[j]);
+                    } else {
+                        w = fx::closed(fx::mulhi(dm[j], sl.ym), de[j] + sl.ye,
+                                       fx::mulhi(dr[j], sl.im), 1 - de[j] + sl.ie,
+                                       fx::Tables{fx_tab, fx_tab + fx::kTab});
+                        ud[j] += fx::mulhi(sl.aq, w.D);
+                    }
+                    cex = w.E ? fx::pack62(fx::mulhi(w.E, cm), ce - w.n) : 0.0;
+                    w0 = w.w0;
+                    wup = w.wup;
                 } else {
-                    __syncthreads();
+                    const Weights64 w = weights64(dtau0[j] * sl.phi);
+                    cu[j] = fma(sl.w, w.u, cu[j]);
+                    cex = sp.c * w.ex;
+                    w0 = w.w0;
+                    wup = w.wup;
+                }
+                const T part = fma(i, cex, wup * S_up[j]);   // I - w0 S
+                cj[j] = fma(sl.w, part, cj[j]);
+                return fma(w0, S_loc[j], part);
+            };
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                if (j < nr && chunk == 0) {
+                    V0[j][0] = chi_loc[j];
+                    V0[j][1] = S_loc[j];
+                    if (write) put(One{}, dst[j], t & 1, 0, V0[j]);
+                }
+#pragma unroll 1
+            for (int v = v_begin; v < v_end; ++v) {
+                T V[R][VW];
+                upwind(v, V);
+#pragma unroll
+                for (int j = 0; j < R; ++j)
+                    if (j < nr) {
+#pragma unroll
+                        for (int e = 0; e < VW; ++e) {
+                            const int p = v * VW + e - 2;
+                            V[j][e] = p < nslot ? step(j, p, V[j][e]) : T(0);
+                        }
+                        if (write) put(One{}, dst[j], t & 1, v, V[j]);
+                    }
+            }
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                if (j < nr) {
+                    const int o = (down ? yl0 + nr - 1 - j : yl0 + j) * nx + x;
+                    // + (sum of (w/phi)(1 - e^-x)) / dtau0
+                    if (ud[j] >> 32)
+                        cu[j] = fma(fx::pack(dr[j], 1 - de[j] + stab[0].ea),
+                                    fx::pack32(ud[j], 0), cu[j]);
+                    if (chunks > 1) {
+                        T *dr = red + 2 * (((t & 1) * chunks + chunk) * rows * nx + o);
+                        dr[0] = cj[j];
+                        dr[1] = cu[j];
+                    } else if (q == q0) {
+                        kj[j] = cj[j];
+                        ku[j] = cu[j];
+                        ko[j] = kp + o;
+                        nk = j + 1;
+                    } else {
+                        pj[kp + o] = cj[j];
+                        pu[kp + o] = cu[j];
+                    }
                 }
             }
         }
-    };
-    if (fast) run(std::true_type{});
-    else run(std::false_type{});
+        // before the barrier, since any thread may read the next plane's values:
+        // the copies for step t + 1 are done
+        if (t + 2 < nz) cp_async_wait_but_last();
+        else cp_async_wait();
+        if (write) {
+            if (as) {
+                __syncthreads();
+                if (t + 2 < nz) cluster_arrive_relaxed();
+            } else if (cl) {
+                cluster_arrive();
+            } else {
+                __syncthreads();
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+            if (j < nk) {
+                pj[ko[j]] = kj[j];
+                pu[ko[j]] = ku[j];
+            }
+        if (write && cl && !as) cluster_wait_acquire();
+        part = part == 2 ? 0 : part + 1;
+    }
+    if (chunks > 1 && nz > 1) {
+        __syncthreads();
+        flush_sums(nz - 1);
+    }
     // no block leaves while another may still address its shared memory
     if (as && nz > 1) cluster_barrier();
 }
 
 // MAXT: block-size bound the kernel is compiled for; MINB: resident blocks
-// per SM it must fit (the register budget).
-template <typename T, int NP, int MAXT, int MINB, bool AS>
+// per SM it must fit (the register budget); R: rows of a thread's item.
+template <typename T, int NP, int MAXT, int MINB, int R, bool AS>
 __global__ void __launch_bounds__(MAXT, MINB) plane_sweep_kernel(const PlaneArgs<T> a) {
-    plane_sweep_body<T, NP, AS>(a);
+    plane_sweep_body<T, NP, R, AS>(a);
 }
 
 // ------------------------------------------------------------- launching
 
-template <typename T, int NP>
-inline size_t plane_smem_t(int rows, int nx) {
-    return 2ull * (rows + 1) * (nx + 1) * plane::node_stride<T, NP>() * sizeof(T);
-}
-
 // Kernel attributes and the launch configuration of shape s (dynamic shared
-// memory, clusters of `bands` blocks); a is used by the launch only.
-template <typename T, int NP, int MAXT, int MINB, bool AS>
-static cudaError_t plane_config(const SweepShape &s, int nx, cudaStream_t st,
+// memory, clusters of `bands` blocks).
+template <typename T, int NP, int MAXT, int MINB, int R, bool AS>
+static cudaError_t plane_config(const SweepShape &s, size_t smem, cudaStream_t st,
                                 cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr) {
     // the limit is the same for every launch, so a CUDA graph that captured a
     // launch needing more shared memory than a later one still replays
-    cudaError_t e = cudaFuncSetAttribute(plane_sweep_kernel<T, NP, MAXT, MINB, AS>,
+    cudaError_t e = cudaFuncSetAttribute(plane_sweep_kernel<T, NP, MAXT, MINB, R, AS>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kMaxPlaneSmem);
+                                         (int)plane_smem_max(sizeof(T) == 8));
     if (e == cudaSuccess && s.bands > kPortableBands)
-        e = cudaFuncSetAttribute(plane_sweep_kernel<T, NP, MAXT, MINB, AS>,
+        e = cudaFuncSetAttribute(plane_sweep_kernel<T, NP, MAXT, MINB, R, AS>,
                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     *cfg = cudaLaunchConfig_t{};
     cfg->gridDim = dim3(s.bands, s.ngroups, kRays);
     cfg->blockDim = dim3(s.threads, 1, 1);
-    cfg->dynamicSmemBytes = plane_smem_t<T, NP>(s.rows, nx);
+    cfg->dynamicSmemBytes = smem;
     cfg->stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = s.bands;
@@ -752,18 +867,33 @@ static cudaError_t plane_config(const SweepShape &s, int nx, cudaStream_t st,
 
 // launch (a non-null) or occupancy query (a null: *n = clusters, or blocks
 // per SM for one band, the GPU holds at once)
+template <typename T, int NP, int MAXT, int MINB, int R, bool AS>
+static cudaError_t plane_go_r(const PlaneArgs<T> *a, const SweepShape &s, const PlaneLayout &lay,
+                              cudaStream_t st, int *n) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    cudaError_t e = plane_config<T, NP, MAXT, MINB, R, AS>(s, lay.smem, st, &cfg, attr);
+    if (e != cudaSuccess) return e;
+    if (a) {
+        PlaneArgs<T> b = *a;
+        b.ahead = lay.ahead;
+        b.chunks = lay.chunks;
+        b.ipad = lay.ipad;
+        return cudaLaunchKernelEx(&cfg, plane_sweep_kernel<T, NP, MAXT, MINB, R, AS>, b);
+    }
+    if (s.bands == 1)
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            n, plane_sweep_kernel<T, NP, MAXT, MINB, R, AS>, s.threads, cfg.dynamicSmemBytes);
+    return cudaOccupancyMaxActiveClusters(n, plane_sweep_kernel<T, NP, MAXT, MINB, R, AS>, &cfg);
+}
+
 template <typename T, int NP, int MAXT, int MINB, bool AS>
 static cudaError_t plane_go(const PlaneArgs<T> *a, const SweepShape &s, int nx, cudaStream_t st,
                             int *n) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    cudaError_t e = plane_config<T, NP, MAXT, MINB, AS>(s, nx, st, &cfg, attr);
-    if (e != cudaSuccess) return e;
-    if (a) return cudaLaunchKernelEx(&cfg, plane_sweep_kernel<T, NP, MAXT, MINB, AS>, *a);
-    if (s.bands == 1)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            n, plane_sweep_kernel<T, NP, MAXT, MINB, AS>, s.threads, cfg.dynamicSmemBytes);
-    return cudaOccupancyMaxActiveClusters(n, plane_sweep_kernel<T, NP, MAXT, MINB, AS>, &cfg);
+    const PlaneLayout lay =
+        plane_layout(sizeof(T) == 8 ? 0 : 1, NP, s.rows, nx, s.threads);
+    return lay.item_rows == 2 ? plane_go_r<T, NP, MAXT, MINB, 2, AS>(a, s, lay, st, n)
+                              : plane_go_r<T, NP, MAXT, MINB, 1, AS>(a, s, lay, st, n);
 }
 
 // register budget: lean 0 the full budget of MAXT threads (one block per SM),
@@ -786,12 +916,10 @@ static cudaError_t plane_go_np(const PlaneArgs<T> *a, const SweepShape &s, int n
         return s.threads <= 256 ? plane_go<T, NP, 256, 1, AS>(a, s, nx, st, n)
                                 : plane_go<T, NP, 512, 1, AS>(a, s, nx, st, n);
     } else {
-        // the FP64 body does not fit 64 registers without spilling: no lean
-        // variant; 448 threads leave it up to 146 registers
+        // the FP64 body does not fit 64 registers without spilling: no lean variant
         if (s.lean != 0 || s.threads > 512) return cudaErrorInvalidValue;
-        if (s.threads <= 256) return plane_go<T, NP, 256, 1, AS>(a, s, nx, st, n);
-        if (s.threads <= 448) return plane_go<T, NP, 448, 1, AS>(a, s, nx, st, n);
-        return plane_go<T, NP, 512, 1, AS>(a, s, nx, st, n);
+        return s.threads <= 256 ? plane_go<T, NP, 256, 1, AS>(a, s, nx, st, n)
+                                : plane_go<T, NP, 512, 1, AS>(a, s, nx, st, n);
     }
 }
 
