@@ -841,7 +841,7 @@ int ml_prd_prepare(mg3d_handle *h, int k) {
     return launched(h, launch_ml_prd_rho(a, h->stream), "partial redistribution ratios");
 }
 
-int formal_solution(mg3d_handle *h, int k);
+int formal_solution(mg3d_handle *h, int k, bool fresh = false);
 
 // One Lambda-iteration of the lagged field of grid k (background field, or
 // the mean intensity of partial redistribution): a formal solution with the
@@ -938,12 +938,15 @@ cudaError_t launch_level_sweep(const mg3d_handle *h, const Level &L, const Sweep
 }
 
 // Formal solution on level k with its populations: partial sums into pj/pu.
-int formal_solution(mg3d_handle *h, int k) {
+// fresh: chi0 and S already belong to the populations (two-level handles; the
+// sweep or formal solution just before left them).
+int formal_solution(mg3d_handle *h, int k, bool fresh) {
     if (h->kind == 1) return ml_formal_solution(h, k);
     Level &L = h->lev[k];
-    MG_TRY(launched(h, launch_opacity(h->prec, L.nvox, h->atom.g_ratio, h->atom.kappa, L.n,
-                                      L.chi0, L.S, h->stream),
-                    "opacity"));
+    if (!fresh)
+        MG_TRY(launched(h, launch_opacity(h->prec, L.nvox, h->atom.g_ratio, h->atom.kappa, L.n,
+                                          L.chi0, L.S, h->stream),
+                        "opacity"));
     if (h->params.sc_interp)
         MG_TRY(launched(h, launch_xslopes(h->prec, L.nx, L.nvox, L.chi0, L.S, L.dchi0, L.dS,
                                           h->stream),
@@ -1086,13 +1089,21 @@ RateArgs rate_args(mg3d_handle *h, int k, int mode) {
     return a;
 }
 
-int sweep(mg3d_handle *h, int k) {
-    MG_TRY(formal_solution(h, k));
+// One MALI sweep.  fresh: as for formal_solution.  next: a formal solution of
+// the new populations follows, so the rate kernel leaves their chi0 and S
+// (which saves that solution's opacity launch).
+int sweep(mg3d_handle *h, int k, bool fresh, bool next) {
+    MG_TRY(formal_solution(h, k, fresh));
     if (h->kind == 1) {
         MlRateArgs a = ml_rate_args(h, k, kRateSolve);
         MG_TRY(launched(h, launch_ml_rates(a, h->stream), "multi-level rates"));
     } else {
         RateArgs a = rate_args(h, k, kRateSolve);
+        if (next) {
+            a.kappa = h->atom.kappa;
+            a.chi0 = h->lev[k].chi0;
+            a.S = h->lev[k].S;
+        }
         MG_TRY(launched(h, launch_rates(a, h->stream), "rates"));
     }
     ++h->sweeps[k];
@@ -1169,8 +1180,8 @@ int zero_radiation(mg3d_handle *h, int k) {
 }
 
 // out <- f - W(n) (mode residual) or out += W(n) (mode add), one extra FS.
-int apply_W(mg3d_handle *h, int k, int mode, double *out) {
-    MG_TRY(formal_solution(h, k));
+int apply_W(mg3d_handle *h, int k, int mode, double *out, bool fresh = false) {
+    MG_TRY(formal_solution(h, k, fresh));
     if (h->kind == 1) {
         MlRateArgs a = ml_rate_args(h, k, mode);
         a.out = out;
@@ -1185,13 +1196,14 @@ int apply_W(mg3d_handle *h, int k, int mode, double *out) {
     return MG3D_OK;
 }
 
-int vcycle(mg3d_handle *h, int k, bool first) {
+// fresh: chi0 and S of grid k belong to its populations.
+int vcycle(mg3d_handle *h, int k, bool first, bool fresh) {
     Level &F = h->lev[k];
     Level &C = h->lev[k - 1];
     const int nu_pre = (first && k == h->L) ? h->params.nu0 : h->params.nu1;
-    for (int i = 0; i < nu_pre; ++i) MG_TRY(sweep(h, k));
+    for (int i = 0; i < nu_pre; ++i) MG_TRY(sweep(h, k, fresh || i > 0, true));
     // residual with an extra formal solution (Eq. 5)
-    MG_TRY(apply_W(h, k, kRateResidual, F.r));
+    MG_TRY(apply_W(h, k, kRateResidual, F.r, fresh || nu_pre > 0));
     // coarse-grid equation (Eq. 9)
     MG_TRY(launched(h, launch_restrict(h->N, F.nx, F.ny, F.nz, F.n, C.n, h->stream,
                                        h->params.restriction),
@@ -1220,18 +1232,20 @@ int vcycle(mg3d_handle *h, int k, bool first) {
                     "restrict r"));
     C.f_default = false;
     MG_TRY(apply_W(h, k - 1, kRateAddW, C.f));
+    // the populations are still those of the coarse operator just applied
     if (k - 1 == 1) {
-        for (int i = 0; i < h->params.nu3; ++i) MG_TRY(sweep(h, 1));
+        for (int i = 0; i < h->params.nu3; ++i)
+            MG_TRY(sweep(h, 1, true, i + 1 < h->params.nu3));
     } else {
-        MG_TRY(vcycle(h, k - 1, false));
+        MG_TRY(vcycle(h, k - 1, false, true));
     }
     // relative correction, interpolated (Eqs. 10-11), 10 % rule (Sec. 4.10)
     MG_TRY(launched(h, launch_prolong_correct(h->params.interpolation, h->N, C.nx, C.ny, C.nz,
                                               F.tz, F.zf, C.n, C.n_before, F.n, h->scal,
                                               h->stream),
                     "prolong correction"));
-    if (h->params.interpolation) ++h->launches;  // the Hermite correction is two kernels
-    for (int i = 0; i < h->params.nu2; ++i) MG_TRY(sweep(h, k));
+    ++h->launches;  // the correction is two kernels
+    for (int i = 0; i < h->params.nu2; ++i) MG_TRY(sweep(h, k, i > 0, i + 1 < h->params.nu2));
     return MG3D_OK;
 }
 
@@ -1245,7 +1259,7 @@ int cycle_work(mg3d_handle *h, bool first) {
                             cudaMemcpyDeviceToDevice, h->stream));
     F.f_default = true;
     MG_TRY(reset_scalars(h));
-    MG_TRY(vcycle(h, h->L, first));
+    MG_TRY(vcycle(h, h->L, first, false));
     MG_TRY(launched(h, launch_max_rel_change((long)h->N * F.nvox, F.n, h->scratch, h->scal + 4,
                                              h->stream),
                     "max rel change"));
@@ -2658,15 +2672,17 @@ int ml_chunks(const mg3d_handle *h) { return (h->nfreq_ml + h->ml_chunk - 1) / h
 // Formal solution of level k for every member: per-member opacity, then one
 // batched sweep launch per atom kind (per frequency chunk for multi-level
 // members, each chunk followed by the members' radiative sums).
-int batch_fs(mg3d_batch *b, int k) {
+int batch_fs(mg3d_batch *b, int k, bool fresh) {
     for (mg3d_handle *h : b->m) {
         Level &L = h->lev[k];
         if (h->kind == 1) {
             b->fs_units += (double)L.nvox * kRays * h->nfreq_ml;
         } else {
-            MG_TRY(batch_launched(b, launch_opacity(h->prec, L.nvox, h->atom.g_ratio,
-                                                    h->atom.kappa, L.n, L.chi0, L.S, b->stream),
-                                  "batch opacity"));
+            if (!fresh)
+                MG_TRY(batch_launched(b, launch_opacity(h->prec, L.nvox, h->atom.g_ratio,
+                                                        h->atom.kappa, L.n, L.chi0, L.S,
+                                                        b->stream),
+                                      "batch opacity"));
             b->fs_units += (double)L.nvox * kRays * h->atom.n_freq;
         }
         ++h->fss[k];
@@ -2703,8 +2719,9 @@ int batch_fs(mg3d_batch *b, int k) {
     return MG3D_OK;
 }
 
+// next (kRateSolve): a formal solution of the new populations follows.
 int member_rates(mg3d_batch *b, mg3d_handle *h, int k, int mode, double *out, bool zero_rad,
-                 unsigned long long *scal) {
+                 unsigned long long *scal, bool next = false) {
     if (h->kind == 1) {
         if (zero_rad) MG_TRY(batch_ml_sums(b, h, k, 0, h->nfreq_ml, true, true));
         MlRateArgs a = ml_rate_args(h, k, mode);
@@ -2716,22 +2733,27 @@ int member_rates(mg3d_batch *b, mg3d_handle *h, int k, int mode, double *out, bo
     a.out = out;
     a.zero_radiation = zero_rad;
     a.scal = scal;
+    if (next) {
+        a.kappa = h->atom.kappa;
+        a.chi0 = h->lev[k].chi0;
+        a.S = h->lev[k].S;
+    }
     return batch_launched(b, launch_rates(a, b->stream), "batch rates");
 }
 
-int batch_sweep(mg3d_batch *b, int k) {
-    MG_TRY(batch_fs(b, k));
+int batch_sweep(mg3d_batch *b, int k, bool fresh, bool next) {
+    MG_TRY(batch_fs(b, k, fresh));
     for (mg3d_handle *h : b->m) {
-        MG_TRY(member_rates(b, h, k, kRateSolve, nullptr, false, h->scal));
+        MG_TRY(member_rates(b, h, k, kRateSolve, nullptr, false, h->scal, next));
         ++h->sweeps[k];
     }
     return MG3D_OK;
 }
 
-int batch_vcycle(mg3d_batch *b, int k, bool first) {
+int batch_vcycle(mg3d_batch *b, int k, bool first, bool fresh) {
     const int nu_pre = (first && k == b->L) ? b->params.nu0 : b->params.nu1;
-    for (int i = 0; i < nu_pre; ++i) MG_TRY(batch_sweep(b, k));
-    MG_TRY(batch_fs(b, k));
+    for (int i = 0; i < nu_pre; ++i) MG_TRY(batch_sweep(b, k, fresh || i > 0, true));
+    MG_TRY(batch_fs(b, k, fresh || nu_pre > 0));
     for (mg3d_handle *h : b->m)
         MG_TRY(member_rates(b, h, k, kRateResidual, h->lev[k].r, false, nullptr));
     for (mg3d_handle *h : b->m) {
@@ -2747,13 +2769,14 @@ int batch_vcycle(mg3d_batch *b, int k, bool first) {
                               "restrict r"));
         C.f_default = false;
     }
-    MG_TRY(batch_fs(b, k - 1));
+    MG_TRY(batch_fs(b, k - 1, false));
     for (mg3d_handle *h : b->m)
         MG_TRY(member_rates(b, h, k - 1, kRateAddW, h->lev[k - 1].f, false, nullptr));
     if (k - 1 == 1) {
-        for (int i = 0; i < b->params.nu3; ++i) MG_TRY(batch_sweep(b, 1));
+        for (int i = 0; i < b->params.nu3; ++i)
+            MG_TRY(batch_sweep(b, 1, true, i + 1 < b->params.nu3));
     } else {
-        MG_TRY(batch_vcycle(b, k - 1, false));
+        MG_TRY(batch_vcycle(b, k - 1, false, true));
     }
     for (mg3d_handle *h : b->m) {
         Level &F = h->lev[k];
@@ -2762,9 +2785,10 @@ int batch_vcycle(mg3d_batch *b, int k, bool first) {
                                                         C.nz, F.tz, F.zf, C.n, C.n_before, F.n,
                                                         h->scal, b->stream),
                               "prolong correction"));
-        if (h->params.interpolation) ++b->launches;
+        ++b->launches;
     }
-    for (int i = 0; i < b->params.nu2; ++i) MG_TRY(batch_sweep(b, k));
+    for (int i = 0; i < b->params.nu2; ++i)
+        MG_TRY(batch_sweep(b, k, i > 0, i + 1 < b->params.nu2));
     return MG3D_OK;
 }
 
@@ -2776,7 +2800,7 @@ int batch_cycle_work(mg3d_batch *b, bool first) {
         F.f_default = true;
         MG_CUDA(cudaMemsetAsync(h->scal, 0, 8 * sizeof(unsigned long long), b->stream));
     }
-    MG_TRY(batch_vcycle(b, b->L, first));
+    MG_TRY(batch_vcycle(b, b->L, first, false));
     for (mg3d_handle *h : b->m) {
         Level &F = h->lev[h->L];
         MG_TRY(batch_launched(b, launch_max_rel_change((long)h->N * F.nvox, F.n, h->scratch,
@@ -3502,7 +3526,7 @@ int mg3d_batch_fmg_solve(mg3d_batch *b, double tol, int max_cycles, mg3d_stats *
         begin_stats(h);
         MG_TRY(zero_radiation(h, 1));
     }
-    for (int i = 0; i < b->params.nu_fmg; ++i) MG_TRY(batch_sweep(b, 1));
+    for (int i = 0; i < b->params.nu_fmg; ++i) MG_TRY(batch_sweep(b, 1, i > 0, i + 1 < b->params.nu_fmg));
     for (int k = 2; k <= b->L; ++k) {
         for (mg3d_handle *h : b->m) {
             Level &Fk = h->lev[k];
@@ -3512,7 +3536,7 @@ int mg3d_batch_fmg_solve(mg3d_batch *b, double tol, int max_cycles, mg3d_stats *
                                   "prolong full approximation"));
             Fk.f_default = true;
         }
-        if (k < b->L) MG_TRY(batch_vcycle(b, k, false));
+        if (k < b->L) MG_TRY(batch_vcycle(b, k, false, false));
     }
     std::vector<double> C(b->n, 1.0);
     std::vector<int> done_at(b->n, 0);
@@ -3717,7 +3741,7 @@ int mg3d_mali_sweep(mg3d_handle *h, int level, int n_sweeps, double *max_rel_cha
     long long bad = 0;
     for (int i = 0; i < n_sweeps; ++i) {
         if (i == n_sweeps - 1) MG_TRY(reset_scalars(h));
-        MG_TRY(sweep(h, level));
+        MG_TRY(sweep(h, level, i > 0, i + 1 < n_sweeps));
     }
     if (n_sweeps > 0) MG_TRY(read_scalars(h, &C, nullptr, &bad));
     if (max_rel_change) *max_rel_change = C;
@@ -3752,7 +3776,7 @@ int mg3d_mali_solve(mg3d_handle *h, double tol, int max_sweeps, mg3d_stats *stat
     int it = 0;
     while (it < max_sweeps) {
         MG_TRY(reset_scalars(h));
-        MG_TRY(sweep(h, h->L));
+        MG_TRY(sweep(h, h->L, it > 0, it + 1 < max_sweeps));
         ++it;
         long long bad = 0;
         MG_TRY(read_scalars(h, &C, nullptr, &bad));
@@ -3794,7 +3818,8 @@ int fmg_stage(mg3d_handle *h, int k) {
     h->top = k;  // each stage solves on its own grid
     if (k == 1) {
         MG_TRY(zero_radiation(h, 1));
-        for (int i = 0; i < h->params.nu_fmg; ++i) MG_TRY(sweep(h, 1));
+        for (int i = 0; i < h->params.nu_fmg; ++i)
+            MG_TRY(sweep(h, 1, i > 0, i + 1 < h->params.nu_fmg));
         return MG3D_OK;
     }
     Level &Fk = h->lev[k];
@@ -3815,7 +3840,7 @@ int fmg_stage(mg3d_handle *h, int k) {
     Fk.f_default = true;
     if (k < h->L) {
         MG_TRY(reset_scalars(h));
-        MG_TRY(vcycle(h, k, false));
+        MG_TRY(vcycle(h, k, false, false));
         long long neg = 0;
         MG_TRY(read_scalars(h, nullptr, &neg, nullptr));
         h->negatives += neg;

