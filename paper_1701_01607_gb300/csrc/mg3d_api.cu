@@ -83,8 +83,7 @@ struct Level {
     // intensity [kRays][nf][nvox]
     void *jnu = nullptr, *jnu_new = nullptr, *rho = nullptr, *rhoS = nullptr;
     StepGeom *geom = nullptr;    // [kRays][nz]
-    void *psteps = nullptr;      // [kRays][nz] PlaneLerp<T> (two-level) or PlaneStep<T>
-                                 // (multi-level) of the shifted-plane sweep
+    void *psteps = nullptr;      // [kRays][nz] PlaneLerp<T> of the shifted-plane sweeps
     SweepShape shape{};
     // formal solutions in the precision other than the handle's (built on the
     // first request, two-level static CRD handles): chi0, S, the bottom
@@ -336,61 +335,45 @@ void build_geometry(const mg3d_handle *h, const Level &L, std::vector<StepGeom> 
     }
 }
 
-// Per-step constants of the multi-level shifted-plane sweep from the upwind
-// geometry: the bilinear weights and half path of step t, and the corner
-// offsets of step t+1 as the shift of the plane written at step t.
-template <typename T>
-std::vector<PlaneStep<T>> plane_steps(const Level &L, const std::vector<StepGeom> &g) {
-    std::vector<PlaneStep<T>> out((size_t)kRays * L.nz);
-    for (int r = 0; r < kRays; ++r)
-        for (int t = 0; t < L.nz; ++t) {
-            const StepGeom &e = g[(size_t)r * L.nz + t];
-            PlaneStep<T> &p = out[(size_t)r * L.nz + t];
-            p.w00 = (T)((1.0 - e.tx) * (1.0 - e.ty));
-            p.w10 = (T)(e.tx * (1.0 - e.ty));
-            p.w01 = (T)((1.0 - e.tx) * e.ty);
-            p.w11 = (T)(e.tx * e.ty);
-            p.half_s = (T)(0.5 * e.s);
-            const bool last = t + 1 >= L.nz;
-            p.sx = last ? 0 : g[(size_t)r * L.nz + t + 1].ix0;
-            p.sy = last ? 0 : g[(size_t)r * L.nz + t + 1].iy0;
-        }
-    return out;
+// The weights of one step from the offsets (tx, ty) of the crossing.
+void round_lerp(PlaneLerp<double> &p, double tx, double ty) {
+    const double bx = std::max(tx, 1.0 - tx), by = std::max(ty, 1.0 - ty);
+    p.rx = std::min(tx, 1.0 - tx) / bx;
+    p.ry = std::min(ty, 1.0 - ty) / by;
+    p.c = 1.0 / ((1.0 + p.rx) * (1.0 + p.ry));
+    p.near = (tx > 0.5 ? 1 : 0) | (ty > 0.5 ? 2 : 0);
 }
-
-// The rounded ratios and scale of the shifted-plane sweep's interpolation.  The
-// weights are the same for every node of a step, and for every step of evenly
-// spaced planes, so a sum c (1 + rx)(1 + ry) that is off 1 by a rounding shifts
-// the intensities of a thin ray by it at every step.  FP32: of the ratios within
-// 4 units in the last place (an offset of the crossing by less than 3e-7
-// cells) the pair whose sum is nearest to 1 (within 1e-9 as a rule).
-template <typename T>
-void round_lerp(PlaneLerp<T> &p, double rx, double ry) {
-    p.rx = (T)rx;
-    p.ry = (T)ry;
-    p.c = (T)(1.0 / ((1.0 + rx) * (1.0 + ry)));
-    if (sizeof(T) == 8) return;
-    const T ulp = (T)std::ldexp(1.0, -24);
+// FP32: the weights are the same for every node of a step, and for every step
+// of evenly spaced planes, so a sum (1 + rx)(wy0 + wy1) that is off 1 by a
+// rounding shifts the intensities of a thin ray by it at every step.  Of the
+// values within 4 units of 2^-24 (an offset of the crossing by less than 3e-7
+// cells) the ones whose sum is nearest to 1 (within 1e-9 as a rule).
+void round_lerp(PlaneLerp<float> &p, double tx, double ty) {
+    const double bx = std::max(tx, 1.0 - tx), rx = std::min(tx, 1.0 - tx) / bx;
+    const double ulp = std::ldexp(1.0, -24);
     double best = 2.0;
-    const T rx0 = p.rx, ry0 = p.ry;
     for (int i = -4; i <= 4; ++i)
         for (int j = -4; j <= 4; ++j) {
-            const T x = (T)((double)rx0 + i * ulp), y = (T)((double)ry0 + j * ulp);
-            if (x < T(0) || x > T(1) || y < T(0) || y > T(1)) continue;
-            const double sum = (1.0 + (double)x) * (1.0 + (double)y);
-            const T c = (T)(1.0 / sum);
-            const double off = std::fabs((double)c * sum - 1.0) + 1e-12 * (std::abs(i) + std::abs(j));
+            const float x = (float)(rx + i * ulp), y1 = (float)(bx * ty + j * ulp);
+            if (x < 0.0f || x > 1.0f || y1 < 0.0f) continue;
+            const float y0 = (float)(1.0 / (1.0 + (double)x) - (double)y1);
+            if (y0 < 0.0f) continue;
+            const double sum = (1.0 + (double)x) * ((double)y0 + (double)y1);
+            const double off = std::fabs(sum - 1.0) + 1e-12 * (std::abs(i) + std::abs(j));
             if (off < best) {
                 best = off;
                 p.rx = x;
-                p.ry = y;
-                p.c = c;
+                p.wy0 = y0;
+                p.wy1 = y1;
             }
         }
+    p.near = tx > 0.5 ? 1 : 0;
 }
 
-// The same for the two-level shifted-plane sweep: the weights of each
-// direction as their ratio (at most 1) and the product of the larger ones.
+// Per-step constants of the shifted-plane sweeps from the upwind geometry: the
+// weights of each direction as their ratio (at most 1) and the product of the
+// larger ones, the half path of step t, and the corner offsets of step t+1 as
+// the shift of the plane written at step t.
 template <typename T>
 std::vector<PlaneLerp<T>> plane_lerps(const Level &L, const std::vector<StepGeom> &g) {
     std::vector<PlaneLerp<T>> out((size_t)kRays * L.nz);
@@ -398,20 +381,13 @@ std::vector<PlaneLerp<T>> plane_lerps(const Level &L, const std::vector<StepGeom
         for (int t = 0; t < L.nz; ++t) {
             const StepGeom &e = g[(size_t)r * L.nz + t];
             PlaneLerp<T> &p = out[(size_t)r * L.nz + t];
-            const double bx = std::max(e.tx, 1.0 - e.tx), by = std::max(e.ty, 1.0 - e.ty);
             const StepGeom &e1 = g[(size_t)r * L.nz + std::max(t - 1, 0)];
-            if (t > 1 && e1.tx == e.tx && e1.ty == e.ty) {
-                p.rx = out[(size_t)r * L.nz + t - 1].rx;
-                p.ry = out[(size_t)r * L.nz + t - 1].ry;
-                p.c = out[(size_t)r * L.nz + t - 1].c;
-            } else {
-                round_lerp(p, std::min(e.tx, 1.0 - e.tx) / bx, std::min(e.ty, 1.0 - e.ty) / by);
-            }
+            if (t > 1 && e1.tx == e.tx && e1.ty == e.ty) p = out[(size_t)r * L.nz + t - 1];
+            else round_lerp(p, e.tx, e.ty);
             p.half_s = (T)(0.5 * e.s);
             const bool last = t + 1 >= L.nz;
             p.sx = last ? 0 : g[(size_t)r * L.nz + t + 1].ix0;
             p.sy = last ? 0 : g[(size_t)r * L.nz + t + 1].iy0;
-            p.near = (e.tx > 0.5 ? 1 : 0) | (e.ty > 0.5 ? 2 : 0);
         }
     return out;
 }
@@ -741,17 +717,15 @@ cudaError_t launch_ml_level_plane(const mg3d_handle *h, const Level &L, int nc, 
         MlPlaneArgs<double> a{L.nx, L.ny, L.nz, nc, rows, bands, rpb, band_magic(rows),
                               band_magic(L.nx), (const double *)L.mchi, (const double *)L.mS,
                               (const double *)L.msc, (const double *)L.moc, (const double *)ib,
-                              (const PlaneStep<double> *)L.psteps, (double *)h->ml_jx,
-                              (double *)h->ml_ux, (double *)h->ml_jm, h->d_exp_tab, h->exp_l1,
-                              h->exp_l2};
+                              (const PlaneLerp<double> *)L.psteps, (double *)h->ml_jx,
+                              (double *)h->ml_ux, (double *)h->ml_jm, h->d_fx_tab};
         return launch_ml_plane_f64(a, nf, threads, h->stream);
     }
     MlPlaneArgs<float> a{L.nx, L.ny, L.nz, nc, rows, bands, rpb, band_magic(rows),
                          band_magic(L.nx), (const float *)L.mchi, (const float *)L.mS,
                          (const float *)L.msc, (const float *)L.moc, (const float *)ib,
-                         (const PlaneStep<float> *)L.psteps, (float *)h->ml_jx,
-                         (float *)h->ml_ux, (float *)h->ml_jm, h->d_exp_tab, h->exp_l1,
-                         h->exp_l2};
+                         (const PlaneLerp<float> *)L.psteps, (float *)h->ml_jx,
+                         (float *)h->ml_ux, (float *)h->ml_jm, h->d_fx_tab};
     return launch_ml_plane_f32(a, nf, threads, h->stream);
 }
 
@@ -2376,6 +2350,34 @@ int setup_ml_prd(mg3d_handle *h, const mg3d_ml_atom *atom) {
     return MG3D_OK;
 }
 
+// Default shape of the FP64 multi-level sweep: the shifted-plane form with two
+// blocks of at most 256 threads per SM (its 128 registers and half the shared
+// memory), the fewest bands of at most 512 nodes and the most rays that fit.
+// Measured (32x32x65, 120 frequencies): 2 bands x 3 rays 7.2 ms, the other form
+// at its former default, 2 x 12, 17.6 ms.  False where no such shape fits.
+bool choose_ml_plane(Level &L) {
+    constexpr size_t kHalfSmem = 103 * 1024;
+    if (!plane_grid_ok(L.nx, L.ny, L.nz)) return false;
+    for (int b = 1; b <= kPortableBands && b <= L.ny; ++b) {
+        const int rows = (L.ny + b - 1) / b;
+        if ((long)(b - 1) * rows >= L.ny) continue;
+        if ((long)rows * L.nx > 512 && !(b == kPortableBands || rows == 1)) continue;
+        const int th = std::min(256, ((rows + 1) / 2 * L.nx + 31) / 32 * 32);
+        if ((long)rows * L.nx > (long)ml_plane_max_pass(1) * th) continue;
+        for (int rpb : {12, 6, 4, 3, 2, 1}) {
+            if (ml_plane_smem_bytes(MG3D_PREC_F64, 1, rows, L.nx, rpb) > kHalfSmem) continue;
+            L.ml_bands = b;
+            L.ml_rows = rows;
+            L.ml_rpb = rpb;
+            L.ml_threads = th;
+            L.ml_plane = 1;
+            L.ml_nf = 1;
+            return true;
+        }
+    }
+    return false;
+}
+
 int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
                    const mg3d_quadrature *quad, const mg3d_params *params, mg3d_handle *h) {
     h->kind = 1;
@@ -2472,12 +2474,12 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
         // per-step constants of the shifted-plane form (static, linear upwind)
         if (!atm->vel && !params->sc_interp) {
             if (h->prec == MG3D_PREC_F64) {
-                const auto ps = plane_steps<double>(L, g);
+                const auto ps = plane_lerps<double>(L, g);
                 MG_TRY(dev_alloc(&L.psteps, ps.size() * sizeof(ps[0])));
                 MG_CUDA(cudaMemcpy(L.psteps, ps.data(), ps.size() * sizeof(ps[0]),
                                    cudaMemcpyHostToDevice));
             } else {
-                const auto ps = plane_steps<float>(L, g);
+                const auto ps = plane_lerps<float>(L, g);
                 MG_TRY(dev_alloc(&L.psteps, ps.size() * sizeof(ps[0])));
                 MG_CUDA(cudaMemcpy(L.psteps, ps.data(), ps.size() * sizeof(ps[0]),
                                    cudaMemcpyHostToDevice));
@@ -2486,23 +2488,34 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
         // rays per block: all 12 of a hemisphere if some band count fits in
         // shared memory, else the largest divisor of 12 that does; bands: the
         // fewest that fit and give >= 300 blocks, else the most that fit
-        int pick = 0;
-        for (int rpb : {12, 6, 4, 3, 2, 1}) {
-            for (int b = 1; b <= kPortableBands && b <= L.ny; ++b) {
-                const int rows = (L.ny + b - 1) / b;
-                if ((long)(b - 1) * rows >= L.ny) continue;
-                if (ml_sweep_smem_bytes(h->prec, rows, L.nx, rpb, params->sc_interp,
-                                        atm->vel ? 1 : 0) > kMaxSweepSmem)
-                    continue;
-                pick = b;
-                if (2L * (12 / rpb) * nf * b >= 300) break;
-            }
-            if (pick) {
-                L.ml_rpb = rpb;
-                h->ml_slots = std::max(h->ml_slots, 2 * (12 / rpb));
-                break;
-            }
+        const bool plain = !atm->vel && !params->sc_interp;
+        if (plain && h->prec == MG3D_PREC_F64 && choose_ml_plane(L)) {
+            h->ml_slots = std::max(h->ml_slots, 2 * (12 / L.ml_rpb));
+            continue;
         }
+        int pick = 0;
+        // static linear sweeps: four blocks of 256 threads per SM where at least
+        // three rays leave room for them (FP32 64x64x129, 120 frequencies: 8
+        // bands x 12 rays 7.6 ms, the fewest bands that fit, 3 x 12, 15.6 ms)
+        for (int pass = plain ? 0 : 1; pass < 2 && !pick; ++pass)
+            for (int rpb : {12, 6, 4, 3, 2, 1}) {
+                if (pass == 0 && rpb < 3) break;
+                for (int b = 1; b <= kPortableBands && b <= L.ny; ++b) {
+                    const int rows = (L.ny + b - 1) / b;
+                    if ((long)(b - 1) * rows >= L.ny) continue;
+                    if (ml_sweep_smem_bytes(h->prec, rows, L.nx, rpb, params->sc_interp,
+                                            atm->vel ? 1 : 0) >
+                        (pass == 0 ? kMlQuarterSmem : kMaxSweepSmem))
+                        continue;
+                    pick = b;
+                    if (pass == 0 || 2L * (12 / rpb) * nf * b >= 300) break;
+                }
+                if (pick) {
+                    L.ml_rpb = rpb;
+                    h->ml_slots = std::max(h->ml_slots, 2 * (12 / rpb));
+                    break;
+                }
+            }
         if (pick == 0) return fail(MG3D_E_ARG, "plane too large for the multi-level sweep");
         L.ml_bands = pick;
         L.ml_rows = (L.ny + pick - 1) / pick;
@@ -2975,6 +2988,8 @@ int batch_build_level(mg3d_batch *b, int k) {
             L.ml_bands = bands;
             L.ml_rows = rows;
             L.ml_threads = std::min(256, threads_for_band(rows * L.nx));
+            L.ml_plane = 0;   // batches run the other form
+            L.ml_nf = 1;
             threads = std::max(threads, L.ml_threads);
             smem = std::max(smem, ml_sweep_smem_bytes(h->prec, rows, L.nx, L.ml_rpb));
             chunks = std::max(chunks, ml_chunks(h));

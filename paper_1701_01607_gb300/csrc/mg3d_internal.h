@@ -45,26 +45,28 @@ struct SweepShape {
     int np = 0;    //    frequencies per group (ng = 2 np table positions per group)
 };
 
-// Per (ray, step t) constants of the multi-level shifted-plane sweep
-// (ml_plane.cuh), in the formal-solution precision: the bilinear weights of the
-// upwind corners and half the path length of step t (t >= 1), and the shift of
-// the plane written at step t, i.e. the corner offsets (ix0, iy0) of step t+1
-// (t <= nz-2).
+// Per (ray, step t) constants of the shifted-plane sweeps (plane_sweep.cuh,
+// ml_plane.cuh), in the formal-solution precision: the bilinear weights of the
+// upwind corners, taken one direction after the other, half the path length of
+// step t (t >= 1), and the shift of the plane written at step t, i.e. the corner
+// offsets (ix0, iy0) of step t+1 (t <= nz-2).  Along x both precisions take H =
+// A + rx B, A the corner of the larger weight.  Along y FP64 takes V = H + ry H'
+// the same way, with the upwind value c V (the factor c goes where no FP64
+// operation is needed for it); FP32 takes V = wy0 H + wy1 H' of rows y and y + 1
+// with all factors in, which is one operation more here and one less there.
 template <typename T>
-struct alignas(16) PlaneStep {
-    T w00, w10, w01, w11;
-    T half_s;
-    int sx, sy;   // (16-byte aligned and padded: loaded as whole vectors)
-};
-
-// The same for the two-level shifted-plane sweep (plane_sweep.cuh), whose
-// interpolation takes the two directions one after the other, scaled by the
-// larger weight of each: H = A + rx B, V = H + ry H', upwind value = c V.
-template <typename T>
-struct alignas(16) PlaneLerp {
-    T rx, ry, c, half_s;
+struct alignas(16) PlaneLerp;
+template <>
+struct alignas(16) PlaneLerp<double> {
+    double rx, ry, c, half_s;
     int sx, sy;
     int near;     // bit 0: the x + 1 column has the larger weight, bit 1: the y + 1 row
+};
+template <>
+struct alignas(16) PlaneLerp<float> {
+    float rx, wy0, wy1, half_s;
+    int sx, sy;
+    int near;     // 1: the x + 1 column has the larger weight
 };
 
 // One slot of the shifted-plane sweep: a mirror pair of frequencies, or the
@@ -329,10 +331,9 @@ struct MlPlaneArgs {
     unsigned long long rmagic, xmagic;   // band_magic(rows), band_magic(nx)
     const T *chi, *S, *sc, *oc;          // [nfreq][nvox]
     const T *ib;                         // [nfreq][nx*ny] intensity entering at the bottom
-    const PlaneStep<T> *steps;           // [kRays][nz]
+    const PlaneLerp<T> *steps;           // [kRays][nz]
     T *jx, *ux, *jm;                     // [2 * 12 / rpb slots][nfreq][nvox]; jm nullable
-    const double *exp_tab;
-    double exp_l1, exp_l2;
+    const unsigned long long *fx_tab;    // tables of the integer weights (FP64 sweeps)
 };
 
 // Frequencies per block the multi-level shifted-plane sweep is built for,
@@ -341,6 +342,8 @@ constexpr int kMlPlaneNf[] = {1, 2, 4};
 // dynamic shared memory limit of the multi-level shifted-plane sweep: its
 // static part (the FP64 exp table and the rays' step constants, 3.2 KB) and
 // this stay within the 227 KB a block may take
+// a quarter of an SM's shared memory: four blocks of the multi-level sweep
+constexpr size_t kMlQuarterSmem = 52 * 1024;
 constexpr size_t kMlPlaneMaxSmem = 220 * 1024;
 constexpr int kMlPlaneNfCount = 3;
 __host__ __device__ constexpr int ml_plane_max_pass(int nf) { return nf <= 2 ? 4 : 2; }

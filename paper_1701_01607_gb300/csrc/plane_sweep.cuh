@@ -50,9 +50,9 @@
 // not conflict in banks and a frame holds no padding between nodes.
 //
 // Interpolation.  The bilinear weights are the same for all nodes of a step, so
-// the two directions are taken one after the other and scaled by the larger
-// weight of each: H = A + rx B along x, V = H + ry H' along y, upwind value =
-// c V with c the product of the larger weights (0 <= rx, ry <= 1, 1/4 <= c <= 1).
+// the two directions are taken one after the other: H = A + rx B along x, scaled
+// by the larger weight, and in FP64 V = H + ry H' along y the same way, upwind
+// value = c V (0 <= rx, ry <= 1, 1/4 <= c <= 1); FP32 takes V = wy0 H + wy1 H'.
 // A thread takes two nodes of neighbouring rows, which share the H of the row
 // between them: 2.5 fused multiply-adds and 3 corner loads per channel and node
 // instead of 4 and 4.
@@ -133,6 +133,15 @@ __device__ __forceinline__ void st16_if(bool c, unsigned a, const double *v) {
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t"
         "@p st.shared::cluster.v2.f64 [%1], {%2, %3};\n\t}" ::"r"((int)c),
         "r"(a), "d"(v[0]), "d"(v[1]));
+}
+// one 16-byte vector at an address of this block's shared memory
+__device__ __forceinline__ void lds16(unsigned a, float *o) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3])
+                 : "r"(a));
+}
+__device__ __forceinline__ void lds16(unsigned a, double *o) {
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(o[0]), "=d"(o[1]) : "r"(a));
 }
 // one 16-byte vector of shared memory into registers
 __device__ __forceinline__ void ld16(const float *p, float *o) {
@@ -268,18 +277,18 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // Short-characteristics weights of optical path x (>= 0) for the linear
 // step I = I_up e^-x + w_up S_up + w0 S0:  u = (1 - e^-x)/x, w0 = 1 - u,
 // w_up = u - e^-x.  Below a threshold the closed form cancels, and the
-// Taylor series of w0 and w_up (e^-x = 1 - w0 - w_up) replace it.
+// Taylor series of w0 and w_up (FP32: w_up = x u - w0) replace it.
 //   FP32: e^-x = 2^(-x log2 e) and 1/x by the hardware approximations (within
 //   2 ulp, ample for the FP32 formal solution); series below x = 0.1.
 //   FP64: 64-bit integer arithmetic (fixed_weights.cuh).
 struct Weights32 {
     static __device__ __forceinline__ void series(float x, float &ex, float &w0, float &wup,
                                                   float &u) {
+        // w0 + w_up = 1 - e^-x = x u
         w0 = x * (0.5f - x * (1.0f / 6.0f - x * (1.0f / 24.0f -
                                                  x * (1.0f / 120.0f - x * (1.0f / 720.0f)))));
-        wup = x * (0.5f - x * (1.0f / 3.0f - x * (1.0f / 8.0f -
-                                                  x * (1.0f / 30.0f - x * (1.0f / 144.0f)))));
         u = 1.0f - w0;
+        wup = fmaf(x, u, -w0);
         ex = u - wup;
     }
     static __device__ __forceinline__ void closed(float x, float &ex, float &w0, float &wup,
@@ -600,10 +609,13 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
         }
         // the nearer column and row first: H = A + rx B, V = H + ry H'
         const unsigned near_x = (sp.near & 1) ? 16u : 0u, far_x = 16u - near_x;
-        const bool down = sp.near & 2;   // the nearer row is the higher one
-        fx::u64 cm = 0;   // FP64: c = (cm, ce)
+        bool down = false;   // FP64: the nearer row is the higher one
+        fx::u64 cm = 0;      // FP64: c = (cm, ce)
         int ce = 0;
-        if constexpr (F64) fx::unpack(sp.c, &cm, &ce);
+        if constexpr (F64) {
+            down = sp.near & 2;
+            fx::unpack(sp.c, &cm, &ce);
+        }
         // Jeff and U of the thread's first item, stored after the barrier's first half
         T kj[R], ku[R];
         int ko[R], nk = 0;
@@ -636,14 +648,14 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                     T ch[NV * VW];
 #pragma unroll
                     for (int c = 0; c < NV * VW; ++c) {
-                        ch[c] = c < NP + 2 ? fma(sp.ry, h1[c], h0[c]) : T(0);
+                        ch[c] = c < NP + 2 ? fma(sp.wy1, h1[c], sp.wy0 * h0[c]) : T(0);
                         h0[c] = h1[c];
                     }
-                    const int yl = down ? yl0 + nr - 1 - j : yl0 + j;
+                    const int yl = yl0 + j;
                     T chi_loc, S_loc;
                     local(t, part, yl * nx + x, chi_loc, S_loc);
-                    const T dtau0 = fma(sp.c, ch[0], chi_loc) * sp.half_s;
-                    const T S_up = ch[1] * sp.c;
+                    const T dtau0 = (ch[0] + chi_loc) * sp.half_s;
+                    const T S_up = ch[1];
                     T cj = 0, cu = 0;
                     // every slot in closed form (0), by series (1), or each its own
                     auto slots = [&](auto mode_tag) {
@@ -656,7 +668,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                             else if (MODE == 1) Weights32::series(xt, ex, w0, wup, u);
                             else Weights32::eval(xt, ex, w0, wup, u);
                             cu = fma(r_w[p], u, cu);
-                            const T part = fma(ch[2 + p], sp.c * ex, wup * S_up);   // I - w0 S
+                            const T part = fma(ch[2 + p], ex, wup * S_up);   // I - w0 S
                             cj = fma(r_w[p], part, cj);
                             ch[2 + p] = fma(w0, S_loc, part);
                         }
