@@ -145,6 +145,33 @@ __device__ __forceinline__ u64 exp2_neg(u64 Y, int e, const Tables t, int *n) {
     return A - mulhi(A, W);
 }
 
+// e^-x and 1 - e^-x for x >= 0: e^-x = E 2^-64 2^-n (0 below 2^-1015), and
+// 1 - e^-x = D 2^-64; false for x outside 2^-11 .. 2^700 (E, D not set).
+__device__ __forceinline__ bool exp_parts(double x, const Tables t, u64 *E, int *n, u64 *D) {
+    u64 m;
+    int e;
+    unpack(x, &m, &e);
+    if (!in_range(x) || e <= kThinExp) return false;
+    *E = exp2_neg(mulhi(m, kLog2e), min(e + 1, 11), t, n);
+    if (e + 1 > 11 || *n > 1015) *E = 0;
+    const u64 Eq = shr(*E, *n);
+    *D = Eq ? 0ull - Eq : ~0ull;
+    return true;
+}
+// e^-x in FP64 for x >= 0 (absolute error below 2^-55.5, then one rounding)
+__device__ __forceinline__ double exp_neg_fx(double x, const Tables t) {
+    u64 E, D;
+    int n;
+    if (exp_parts(x, t, &E, &n, &D)) return E ? pack62(E, -n) : 0.0;
+    // below 2^-11: the Taylor series to x^4
+    if (x < 1.0) return fma(x, fma(x, fma(x, fma(x, 1.0 / 24.0, -1.0 / 6.0), 0.5), -1.0), 1.0);
+    return exp(-x);
+}
+// v 2^-64 2^-n in FP32
+__device__ __forceinline__ float to_float(u64 v, int n) {
+    return __ull2float_rn(v) * 5.4210108624275222e-20f * __int_as_float(max(0, 127 - n) << 23);
+}
+
 struct Weights {
     u64 E;           // e^-x = E 2^-64 2^-n (0: below 2^-1015)
     int n;

@@ -106,6 +106,7 @@ struct Level {
     int ml_rpb = 12;             // rays of a hemisphere per block of the multi-level sweep
     int ml_plane = 0;            // 1: the shifted-plane form (ml_plane.cuh), ml_nf
     int ml_nf = 1;               //    frequencies per block
+    MlNodeTab ntab{};            // per-node constants of the opacity and the radiative sums
 };
 
 struct TimedLaunch {
@@ -130,6 +131,7 @@ struct mg3d_handle {
     std::vector<FreqInfo> fi;
     std::vector<TransInfo> ti;
     FreqInfo *d_fi = nullptr;
+    FreqOp *d_fo = nullptr;              // [nfreq_ml] constants of the opacity and the sums
     TransInfo *d_ti = nullptr;
     // multi-level formal solution, in chunks of ml_chunk frequencies:
     // angle sums of the chunk [2 hemispheres][ml_chunk][nvox] and the
@@ -661,7 +663,9 @@ void free_level(Level &L) {
                     L.mchi,  L.mS,    L.msc,  L.moc,  L.mib,  L.sigma_c, L.jbg,
                     L.dchi0, L.dS,   L.mdchi, L.mdS,  L.vel,  L.uproj, L.vnorm, L.dinv,
                     L.jnu,   L.jnu_new, L.rho, L.rhoS, L.psteps, L.o_chi0, L.o_S, L.o_bbot,
-                    L.o_psteps, L.prd_c, L.prd_rho, L.prd_oc};
+                    L.o_psteps, L.prd_c, L.prd_rho, L.prd_oc,
+                    (void *)L.ntab.nf, (void *)L.ntab.pnorm, (void *)L.ntab.inv_d,
+                    (void *)L.ntab.inv_T, (void *)L.ntab.bline};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     L = Level{};
@@ -729,16 +733,71 @@ cudaError_t launch_ml_level_plane(const mg3d_handle *h, const Level &L, int nc, 
     return launch_ml_plane_f32(a, nf, threads, h->stream);
 }
 
+// Arguments of the opacity of frequencies f0 .. f0+nc-1 on level L, without the
+// lagged fields (background scattering, partial redistribution).
+MlOpacityArgs ml_opacity_args(const mg3d_handle *h, const Level &L, int f0, int nc) {
+    MlOpacityArgs a{};
+    a.nvox = L.nvox;
+    a.f0 = f0;
+    a.nfreq = nc;
+    a.n_trans = h->ntrans;
+    a.prec = h->prec;
+    a.fi = h->d_fi;
+    a.fo = h->d_fo;
+    a.ti = h->d_ti;
+    a.tab = L.ntab;
+    a.theta_ref = h->theta_ref;
+    a.n = L.n;
+    a.T = L.T;
+    a.chi_c = L.chi_c;
+    a.saha = L.saha;
+    a.chi = L.mchi;
+    a.S = L.mS;
+    a.sc = L.msc;
+    a.oc = L.moc;
+    a.fx_tab = h->d_fx_tab;
+    a.moving = h->moving ? 1 : 0;
+    a.voigt = h->d_voigt;
+    return a;
+}
+
+// Arguments of the radiative sums of frequencies f0 .. f0+nc-1 on level L,
+// without the lagged fields.
+MlAccumArgs ml_accum_args(const mg3d_handle *h, const Level &L, int f0, int nc, bool zero_rad) {
+    MlAccumArgs a{};
+    a.nvox = L.nvox;
+    a.f0 = f0;
+    a.nfreq = nc;
+    a.n_trans = h->ntrans;
+    a.prec = h->prec;
+    a.fi = h->d_fi;
+    a.fo = h->d_fo;
+    a.ti = h->d_ti;
+    a.tab = L.ntab;
+    a.jx = h->ml_jx;
+    a.ux = h->ml_ux;
+    a.nslots = 2 * (12 / L.ml_rpb);
+    a.zero_radiation = zero_rad ? 1 : 0;
+    a.acc = h->ml_acc;
+    a.fx_tab = h->d_fx_tab;
+    a.moving = h->moving ? 1 : 0;
+    a.voigt = h->d_voigt;
+    return a;
+}
+
 // Opacity and sweep of the chunk of frequencies f0 .. f0+nc-1 on level k:
 // per-frequency angle sums of both hemispheres into ml_jx/ml_ux.
 int ml_chunk_fs(mg3d_handle *h, int k, int f0, int nc) {
     Level &L = h->lev[k];
-    MlOpacityArgs oa{L.nvox, nc, h->N, h->prec, h->d_fi, h->theta_ref, h->t_ref,
-                     L.n, L.T, L.chi_c, L.saha, L.mchi, L.mS, L.msc, L.moc, f0,
-                     h->d_exp_tab, h->exp_l1, h->exp_l2,
-                     h->scatter ? L.sigma_c : nullptr, h->scatter ? L.jbg : nullptr,
-                     h->moving ? 1 : 0, h->ml_prd ? h->d_prd_index : nullptr,
-                     h->ml_prd ? L.prd_rho : nullptr, h->d_voigt};
+    MlOpacityArgs oa = ml_opacity_args(h, L, f0, nc);
+    if (h->scatter) {
+        oa.sigma_c = L.sigma_c;
+        oa.jbg = L.jbg;
+    }
+    if (h->ml_prd) {
+        oa.prd_index = h->d_prd_index;
+        oa.prd_rho = L.prd_rho;
+    }
     MG_TRY(launched(h, launch_ml_opacity(oa, h->stream), "multi-level opacity"));
     if (h->params.sc_interp)
         MG_TRY(launched(h, launch_xslopes(h->prec, L.nx, (long)nc * L.nvox, L.mchi, L.mS, L.mdchi,
@@ -832,12 +891,15 @@ int lambda_iteration(mg3d_handle *h, int k) {
 int ml_accumulate(mg3d_handle *h, int k, int f0, int nc, bool zero_rad) {
     Level &L = h->lev[k];
     const bool bg = !zero_rad && updates_background(h, k);   // the mean intensity becomes the field
-    MlAccumArgs a{L.nvox, f0, nc, h->ntrans, h->prec, h->d_fi, h->d_ti, h->theta_ref,
-                  h->t_ref, L.T, h->ml_jx, h->ml_ux, 2 * (12 / L.ml_rpb), zero_rad ? 1 : 0,
-                  h->ml_acc, h->d_exp_tab, h->exp_l1, h->exp_l2, bg ? h->ml_jm : nullptr,
-                  bg ? L.jbg : nullptr, h->moving ? 1 : 0,
-                  h->ml_prd ? h->d_prd_index : nullptr, h->ml_prd ? L.prd_oc : nullptr,
-                  h->d_voigt};
+    MlAccumArgs a = ml_accum_args(h, L, f0, nc, zero_rad);
+    if (bg) {
+        a.jm = h->ml_jm;
+        a.jbg = L.jbg;
+    }
+    if (h->ml_prd) {
+        a.prd_index = h->d_prd_index;
+        a.prd_oc = L.prd_oc;
+    }
     return launched(h, launch_ml_accum(a, h->stream), "radiative sums");
 }
 
@@ -2101,10 +2163,7 @@ bool ml_single_ray_only(const mg3d_handle *h, int k) {
 // that fit; once each, the best six three more times) and keeps the fastest.
 int autotune_ml_level(mg3d_handle *h, int k, int nc, int *evaluated) {
     Level &L = h->lev[k];
-    MlOpacityArgs oa{L.nvox, nc, h->N, h->prec, h->d_fi, h->theta_ref, h->t_ref,
-                     L.n, L.T, L.chi_c, L.saha, L.mchi, L.mS, L.msc, L.moc, 0,
-                     h->d_exp_tab, h->exp_l1, h->exp_l2, nullptr, nullptr, h->moving ? 1 : 0,
-                     nullptr, nullptr, h->d_voigt};
+    const MlOpacityArgs oa = ml_opacity_args(h, L, 0, nc);
     MG_TRY(launched(h, launch_ml_opacity(oa, h->stream), "multi-level opacity"));
     if (h->params.sc_interp)
         MG_TRY(launched(h, launch_xslopes(h->prec, L.nx, (long)nc * L.nvox, L.mchi, L.mS, L.mdchi,
@@ -2378,6 +2437,70 @@ bool choose_ml_plane(Level &L) {
     return false;
 }
 
+// Constants of every frequency for the opacity and the radiative sums.
+int setup_freq_ops(mg3d_handle *h) {
+    std::vector<FreqOp> ops(h->fi.size());
+    auto pair = [](double v, float *hi, float *lo) {
+        *hi = (float)v;
+        *lo = (float)(v - (double)*hi);
+    };
+    for (const TransInfo &tr : h->ti)
+        for (int f = tr.f_begin; f < tr.f_end; ++f) {
+            const FreqInfo &q = h->fi[f];
+            FreqOp o{};
+            if (tr.kind == 0) {
+                o.damped = q.adamp > 0.0 ? 1 : 0;
+                o.a = q.xy;
+                o.kap = q.kappa;
+                o.emis = q.kappa * q.rho * q.rho * q.rho;
+                o.w = q.w;
+                pair(q.xy * q.xy, &o.ah, &o.al);
+            } else {
+                const double y = q.xy, ry = q.rho * y;
+                o.a = h->theta_ref * q.rho * y;
+                o.kap = q.kappa / (y * y * y);
+                o.ry3 = ry * ry * ry;
+                o.emis = o.kap * o.ry3;
+                o.w = tr.coef * q.w / (y * y * y * y);
+                o.q3 = o.w * o.ry3;
+                pair(o.a, &o.ah, &o.al);
+                pair(o.q3, &o.q3h, &o.q3l);
+            }
+            pair(o.w, &o.wh, &o.wl);
+            o.kapf = (float)o.kap;
+            o.emisf = (float)o.emis;
+            o.ry3f = (float)o.ry3;
+            ops[f] = o;
+        }
+    MG_TRY(dev_alloc((void **)&h->d_fo, ops.size() * sizeof(FreqOp)));
+    MG_CUDA(cudaMemcpy(h->d_fo, ops.data(), ops.size() * sizeof(FreqOp), cudaMemcpyHostToDevice));
+    return MG3D_OK;
+}
+
+// Per-node constants of a level (its temperature is fixed).
+int setup_node_tab(mg3d_handle *h, Level &L, int n_lines) {
+    float4 *nf = nullptr;
+    float *pnorm = nullptr;
+    double *inv_d = nullptr, *inv_T = nullptr;
+    void *bline = nullptr;
+    if (h->prec == MG3D_PREC_F32) {
+        MG_TRY(dalloc(&nf, L.nvox));
+        L.ntab.nf = nf;
+        MG_TRY(dalloc(&pnorm, L.nvox));
+        L.ntab.pnorm = pnorm;
+    }
+    MG_TRY(dalloc(&inv_d, L.nvox));
+    L.ntab.inv_d = inv_d;
+    MG_TRY(dalloc(&inv_T, L.nvox));
+    L.ntab.inv_T = inv_T;
+    MG_TRY(dev_alloc(&bline, std::max<size_t>(1, (size_t)n_lines * L.nvox) * elem_size(h->prec)));
+    L.ntab.bline = bline;
+    return launched(h, launch_ml_node_tab(h->prec, L.nvox, n_lines, h->d_ti, h->t_ref,
+                                          h->theta_ref, L.T, nf, pnorm, inv_d, inv_T, bline,
+                                          h->stream),
+                    "node constants");
+}
+
 int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
                    const mg3d_quadrature *quad, const mg3d_params *params, mg3d_handle *h) {
     h->kind = 1;
@@ -2406,7 +2529,8 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
         trapezoid_grid(-ln.x_max, ln.x_max, ln.n_freq, x, w);
         if (ln.n_freq == 1) x[0] = 0.0;
         TransInfo tr{0, ln.lower, ln.upper, (int)h->fi.size(), 0, ln.rho, ln.a_ul,
-                     atom->g[ln.upper] / atom->g[ln.lower]};
+                     atom->g[ln.upper] / atom->g[ln.lower],
+                     ln.a_ul / (ln.rho * ln.rho * ln.rho)};
         for (int i = 0; i < ln.n_freq; ++i)
             h->fi.push_back(
                 FreqInfo{0, ln.lower, ln.upper, x[i], w[i], ln.rho, ln.kappa, tr.gr, ln.a_damp});
@@ -2580,8 +2704,10 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
                        cudaMemcpyHostToDevice));
     MG_CUDA(cudaMemcpy(h->d_ti, h->ti.data(), h->ti.size() * sizeof(TransInfo),
                        cudaMemcpyHostToDevice));
+    MG_TRY(setup_freq_ops(h));
     for (int k = 1; k <= h->L; ++k) {
         Level &L = h->lev[k];
+        MG_TRY(setup_node_tab(h, L, atom->n_lines));
         MG_TRY(launched(h, launch_ml_bottom(h->prec, L.nplane, nf, h->d_fi, h->theta_ref, L.T,
                                             L.mib, h->stream),
                         "bottom intensity"));
@@ -2674,9 +2800,7 @@ int batch_ml_sums(mg3d_batch *b, mg3d_handle *h, int k, int f0, int nc, bool zer
         MG_CUDA(cudaMemsetAsync(h->ml_acc, 0,
                                 (size_t)h->ntrans * kAccTerms * L.nvox * sizeof(double),
                                 b->stream));
-    MlAccumArgs a{L.nvox, f0, nc, h->ntrans, h->prec, h->d_fi, h->d_ti, h->theta_ref,
-                  h->t_ref, L.T, h->ml_jx, h->ml_ux, 2 * (12 / L.ml_rpb), zero_rad ? 1 : 0,
-                  h->ml_acc, h->d_exp_tab, h->exp_l1, h->exp_l2};
+    const MlAccumArgs a = ml_accum_args(h, L, f0, nc, zero_rad);
     return batch_launched(b, launch_ml_accum(a, b->stream), "batch radiative sums");
 }
 
@@ -2711,9 +2835,7 @@ int batch_fs(mg3d_batch *b, int k, bool fresh) {
             if ((int)c >= ml_chunks(h)) continue;
             Level &L = h->lev[k];
             const int f0 = (int)c * h->ml_chunk, nc = std::min(h->ml_chunk, h->nfreq_ml - f0);
-            MlOpacityArgs oa{L.nvox, nc, h->N, h->prec, h->d_fi, h->theta_ref, h->t_ref,
-                             L.n, L.T, L.chi_c, L.saha, L.mchi, L.mS, L.msc, L.moc, f0,
-                             h->d_exp_tab, h->exp_l1, h->exp_l2};
+            const MlOpacityArgs oa = ml_opacity_args(h, L, f0, nc);
             MG_TRY(batch_launched(b, launch_ml_opacity(oa, b->stream), "batch opacity"));
         }
         mg3d_batch::KindLevel &q = b->mlc[k][c];
@@ -3601,7 +3723,7 @@ int mg3d_destroy(mg3d_handle *h) {
     if (h->o_pu) cudaFree(h->o_pu);
     void *ptrs[] = {h->d_ftab, h->d_vtab, h->d_vline, h->d_kmat, h->d_wphin, h->d_fidx,
                     h->d_exp_tab, h->pj, h->pu, h->scal,
-                    h->scratch, h->d_fi, h->d_ti, h->ml_jx, h->ml_ux, h->ml_acc,
+                    h->scratch, h->d_fi, h->d_fo, h->d_ti, h->ml_jx, h->ml_ux, h->ml_acc,
                     h->ml_jm};
     for (void *p : ptrs)
         if (p) cudaFree(p);

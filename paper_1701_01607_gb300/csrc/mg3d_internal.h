@@ -297,6 +297,7 @@ struct TransInfo {
     double rho;     // as in FreqInfo
     double coef;    // line: A_ul; continuum: beta
     double gr;      // line: g_u/g_l
+    double b_ul;    // line: Einstein B_ul = A_ul/rho^3
 };
 
 template <typename T>
@@ -393,18 +394,41 @@ struct MlPrdArgs {
 
 // Opacity of the chunk of frequencies f0 .. f0+nfreq-1, written at the
 // chunk-local index [f - f0][nvox].
+// Constants of a frequency for the opacity and the radiative sums, in both
+// precisions; (h, l) is a value as a pair of floats.
+struct alignas(16) FreqOp {
+    // FP32: line: a = x^2, continuum: a = theta_ref rho y; kap, emis as below
+    float ah, al, kapf, emisf;
+    float wh, wl, q3h, q3l;      // line: w (trapezoid weight); continuum: qa; qa (rho y)^3
+    float ry3f;                  // continuum: (rho y)^3
+    int damped;                  // line: Voigt profile
+    double a;                    // line: x; continuum: theta_ref rho y
+    double kap, emis;            // line: kappa, kappa rho^3; continuum: kappa/y^3 (emis: times
+                                 // (rho y)^3 in FP32, unused in FP64)
+    double ry3, w, q3;
+};
+// Per-node constants of a level (the temperature is fixed).
+struct MlNodeTab {
+    const float4 *nf;       // FP32: t_ref/T and 1/T as pairs
+    const float *pnorm;     // FP32: sqrt(t_ref/T)/sqrt(pi)
+    const double *inv_d;    // sqrt(t_ref/T)
+    const double *inv_T;    // 1/T
+    const void *bline;      // [n_lines][nvox] Planck function at line centre (FS precision)
+};
+
 struct MlOpacityArgs {
     long nvox;
-    int nfreq, n_levels, prec;
+    int f0, nfreq, n_trans, prec;  // chunk f0 .. f0+nfreq-1
     const FreqInfo *fi;
-    double theta_ref, t_ref;
+    const FreqOp *fo;
+    const TransInfo *ti;
+    MlNodeTab tab;
+    double theta_ref;
     const double *n, *T, *chi_c, *saha;
     void *chi, *S, *sc, *oc;       // sc = S - rho eta_t/chi, oc = 1 - chi_t/chi (0 for a
                                    // PRD frequency: its 1 - rho chi_t/chi goes in FP64
                                    // to the radiative sums, MlAccumArgs::prd_oc)
-    int f0;
-    const double *exp_tab;         // FP64 exp table of the sweep
-    double exp_l1, exp_l2;
+    const unsigned long long *fx_tab;   // tables of the integer exponential
     const double *sigma_c;         // background scattering [nvox], or null
     const void *jbg;               // background field [n_freq][nvox] (FS precision)
     int moving;                    // 1: write the ray-independent parts instead (a
@@ -418,25 +442,20 @@ struct MlOpacityArgs {
     const VoigtTable *voigt;       // coefficients of the Voigt function (damped lines), or null
 };
 
-// Radiative sums per transition and node, [n_trans][3][nvox] in FP64:
-//   line:       sum w phi, sum w phi J, sum w phi U   (phi at the node's T)
-//   continuum:  sum qa J, sum qa E J, sum qa E (rho y)^3 U
-// accumulated chunk by chunk from the per-frequency angle sums Jx, Ux.
 constexpr int kAccTerms = 3;
 
 struct MlAccumArgs {
     long nvox;
     int f0, nfreq, n_trans, prec;  // chunk f0 .. f0+nfreq-1
     const FreqInfo *fi;
+    const FreqOp *fo;
     const TransInfo *ti;
-    double theta_ref, t_ref;
-    const double *T;
+    MlNodeTab tab;
     const void *jx, *ux;           // [nslots][nfreq][nvox] of the chunk
     int nslots;                    // ray groups of both hemispheres
     int zero_radiation;            // 1: J = 0, U = 1 (jx, ux unused)
     double *acc;
-    const double *exp_tab;         // FP64 exp table of the sweep
-    double exp_l1, exp_l2;
+    const unsigned long long *fx_tab;   // tables of the integer exponential
     const void *jm;                // mean intensity per slot [nslots][nfreq][nvox], or null
     void *jbg;                     // background field [n_freq][nvox] written from jm
     int moving;                    // 1: line sums already carry their per-ray profile
@@ -468,6 +487,10 @@ cudaError_t launch_ml_vel_prep(int prec, long nvox, int ntrans, const TransInfo 
                                const double *T, double t_ref, void *uproj, void *dinv,
                                void *vnorm, cudaStream_t st);
 cudaError_t launch_ml_opacity(const MlOpacityArgs &a, cudaStream_t st);
+// fills the per-node constants (nf, pnorm FP32 only; bline [n_lines][nvox])
+cudaError_t launch_ml_node_tab(int prec, long nvox, int n_lines, const TransInfo *ti, double t_ref,
+                               double theta_ref, const double *T, float4 *nf, float *pnorm,
+                               double *inv_d, double *inv_T, void *bline, cudaStream_t st);
 // Per node and PRD line: the symmetric scaling c of R_I-A at the node's
 // Doppler width, the fixed point of c <- sqrt(c phi / (R0^T (wq c))) after
 // 200 steps from c = 1 (R = diag(c) R0 diag(c) then has marginals phi).

@@ -42,6 +42,7 @@
 #include <cmath>
 
 #include "mg3d.h"
+#include "fixed_weights.cuh"
 #include "mg3d_internal.h"
 #include "sc_step.cuh"
 #include "voigt.cuh"
@@ -63,13 +64,6 @@ __device__ __forceinline__ double planck_rho(double rho, double theta_ref, doubl
 
 // ------------------------------------------------------------------ opacity
 
-// exp(-x), x >= 0, in the opacity's precision: the sweep's table-driven FP64
-// exp, or the FP32 library exp for the FP32 formal solution.
-__device__ __forceinline__ double opac_exp(double x, const ExpNegTable &et) {
-    return exp_neg(x, et);
-}
-__device__ __forceinline__ float opac_exp(float x, const ExpNegTable &) { return expf(-x); }
-
 // Line profile exp(-dd2) di / sqrt(pi) in the formal-solution precision.
 __device__ __forceinline__ double ml_doppler(double dd2, double di, const ExpNegTable &et) {
     return exp_neg(dd2, et) * di * 0.56418958354775628;
@@ -78,113 +72,177 @@ __device__ __forceinline__ float ml_doppler(float dd2, float di, const ExpNegTab
     return __expf(-dd2) * di * 0.564189584f;
 }
 
-// A line's profile at a node of Doppler width d = 1/inv_d reference widths,
-// per reference width: the Doppler profile in the formal-solution precision,
-// or for a damped line (damping a at t_ref; the node's parameter a/d, since
-// the damping width does not scale with temperature) H(a/d, x/d)/(sqrt(pi) d)
-// from the rational Voigt function in FP64, rounded once.
-template <typename T>
-__device__ __forceinline__ T ml_line_phi(const FreqInfo &q, double inv_d, T pnorm,
-                                         const VoigtTable *vt, const ExpNegTable &et) {
-    const double xd = q.xy * inv_d;
-    if (q.adamp > 0.0)
-        return (T)(voigt_H_rational(*vt, q.adamp * inv_d, xd) * 0.5641895835477563 * inv_d);
-    return opac_exp((T)(xd * xd), et) * pnorm;
+// Opacity and radiative sums of one transition per thread and node.  Both are
+// bound by memory (four values written, two per ray-group slot read, per node
+// and frequency) once their arithmetic is off the FP64 pipe, which converts
+// and multiplies at 2 lanes per clock and SM: FP32 works on pairs of floats
+// prepared per frequency and per node (the arguments of the exponentials are
+// rounded once, as when they were formed in FP64), FP64 takes its exponentials
+// from 64-bit integer arithmetic.  The grid's y index is the transition, so
+// that small grids still fill the GPU and the populations and Planck function
+// of a transition are read once.  Measured (64x64x129, 120 frequencies, FP32):
+// opacity 3.00 -> 0.45 ms, sums 2.53 -> 0.37 ms; FP64 32x32x65: 0.82 -> 0.40 and 0.45 ->
+// 0.25 ms; on an 8x8x9 grid with 30 frequencies (FP32) 75 -> 10 us each.
+
+// e^-(product of two pairs) in FP32, the argument rounded once
+__device__ __forceinline__ float pair_arg(float ah, float al, float bh, float bl) {
+    const float p = ah * bh;
+    float e = fmaf(ah, bh, -p);
+    e = fmaf(ah, bl, e);
+    return p + fmaf(al, bh, e);
 }
 
-// One thread per node walks the chunk's frequencies, so per-node quantities
-// (temperature, Doppler width, background) and per-transition ones
-// (populations, the line-centre Planck function) are formed once.  The
-// profile and the source terms are evaluated in the formal-solution
-// precision T; population differences in FP64.
+// A damped line's profile at a node of Doppler width d = 1/inv_d reference
+// widths, per reference width: H(a/d, x/d)/(sqrt(pi) d) with the damping a at
+// t_ref (the damping width does not scale with temperature), from the
+// rational Voigt function in FP64, rounded once.
+template <typename T>
+__device__ __forceinline__ T ml_voigt_phi(const FreqInfo &q, double inv_d, const VoigtTable *vt) {
+    return (T)(voigt_H_rational(*vt, q.adamp * inv_d, q.xy * inv_d) * 0.5641895835477563 * inv_d);
+}
+
+// What a thread keeps of its node.
+template <typename T>
+struct MlNode;
+template <>
+struct MlNode<float> {
+    float4 nf;
+    float pnorm;
+    __device__ __forceinline__ MlNode(const MlNodeTab &t, long v)
+        : nf(t.nf[v]), pnorm(t.pnorm[v]) {}
+    // e^-(x/d)^2
+    __device__ __forceinline__ float line_exp(const FreqOp &q, const fx::Tables &) const {
+        return expf(-pair_arg(q.ah, q.al, nf.x, nf.y));
+    }
+    // e^-(theta_ref rho y/T)
+    __device__ __forceinline__ float cont_exp(const FreqOp &q, const fx::Tables &) const {
+        return expf(-pair_arg(q.ah, q.al, nf.z, nf.w));
+    }
+};
+template <>
+struct MlNode<double> {
+    double inv_d, inv_T, pnorm;
+    __device__ __forceinline__ MlNode(const MlNodeTab &t, long v)
+        : inv_d(t.inv_d[v]), inv_T(t.inv_T[v]), pnorm(0.5641895835477563 * t.inv_d[v]) {}
+    __device__ __forceinline__ double line_exp(const FreqOp &q, const fx::Tables &ft) const {
+        const double xd = q.a * inv_d;
+        return fx::exp_neg_fx(xd * xd, ft);
+    }
+    __device__ __forceinline__ double cont_exp(const FreqOp &q, const fx::Tables &ft) const {
+        return fx::exp_neg_fx(q.a * inv_T, ft);
+    }
+};
+
+// Bound-free continuum: E = e^-x and the Planck function (rho y)^3/(e^x - 1),
+// x = theta_ref rho y/T.
+__device__ __forceinline__ void cont_terms(const FreqOp &q, double inv_T, const fx::Tables &ft,
+                                           float &E, float &B) {
+    const double x = q.a * inv_T;
+    fx::u64 e, d;
+    int n;
+    if (fx::exp_parts(x, ft, &e, &n, &d)) {
+        E = fx::to_float(e, n);
+        B = q.ry3f * E / fx::to_float(d, 0);
+    } else {
+        E = expf(-(float)x);
+        B = (float)(q.ry3 / expm1(x));
+    }
+}
+__device__ __forceinline__ void cont_terms(const FreqOp &q, double inv_T, const fx::Tables &ft,
+                                           double &E, double &B) {
+    const double x = q.a * inv_T;
+    fx::u64 e, d;
+    int n;
+    if (fx::exp_parts(x, ft, &e, &n, &d)) {
+        E = e ? fx::pack62(e, -n) : 0.0;
+        B = q.ry3 * fast_div(E, fx::pack32(d, 0));
+    } else {
+        E = exp(-x);
+        B = q.ry3 / expm1(x);
+    }
+}
+__device__ __forceinline__ float fast_inv(float x) { return 1.0f / x; }
+__device__ __forceinline__ double fast_inv(double x) { return fast_div(1.0, x); }
+
 template <typename T>
 __global__ void ml_opacity_kernel(const MlOpacityArgs a) {
-    __shared__ double tab[kExpTab];
-    for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) tab[i] = a.exp_tab[i];
+    __shared__ fx::u64 fx_tab[2 * fx::kTab];
+    for (int i = threadIdx.x; i < 2 * fx::kTab; i += blockDim.x) fx_tab[i] = a.fx_tab[i];
     __syncthreads();
-    const ExpNegTable et{tab, a.exp_l1, a.exp_l2};
-    const double rsqpi = 0.5641895835477563;  // 1/sqrt(pi)
+    const fx::Tables ft{fx_tab, fx_tab + fx::kTab};
     const long nvox = a.nvox;
+    const int t = blockIdx.y;
+    const TransInfo tr = a.ti[t];
+    const int fb = max(tr.f_begin, a.f0), fe = min(tr.f_end, a.f0 + a.nfreq);
+    if (fb >= fe) return;
     for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox;
          v += (long)gridDim.x * blockDim.x) {
-        const double Tg = a.T[v];
-        const double cc = a.chi_c[v];
-        const double inv_d = sqrt(a.t_ref / Tg);   // 1/d, d = sqrt(T/t_ref)
-        const T pnorm = (T)(rsqpi * inv_d);
-        int lo = -1, up = -1;
-        double nl = 0.0, nu = 0.0, G = 0.0, rho_b = -1.0;
+        const MlNode<T> node(a.tab, v);
+        const T cc = (T)a.chi_c[v];
+        const T sg = a.sigma_c ? (T)a.sigma_c[v] : T(0);
+        const double nl = a.n[(long)tr.lo * nvox + v], nu = a.n[(long)tr.up * nvox + v];
+        // line: the population difference; continuum: n_u G, G = n_l*/n_u*
+        const double nd = tr.kind == 0 ? tr.gr * nl - nu : nu * a.saha[(long)tr.lo * nvox + v];
+        const T nlT = (T)nl, nuT = (T)nu, ndT = (T)nd;
         T B = 0;
-        for (int fl = 0; fl < a.nfreq; ++fl) {
-            const FreqInfo q = a.fi[a.f0 + fl];
-            if (q.lo != lo || q.up != up) {
-                lo = q.lo;
-                up = q.up;
-                nl = a.n[(long)lo * nvox + v];
-                nu = a.n[(long)up * nvox + v];
-                G = a.saha[(long)lo * nvox + v];
-                rho_b = -1.0;
-            }
+        double inv_d = 0.0, inv_T = 0.0;
+        if (tr.kind == 0) {
+            B = ((const T *)a.tab.bline)[(long)t * nvox + v];
+            if (a.voigt) inv_d = a.tab.inv_d[v];
+        } else {
+            inv_T = a.tab.inv_T[v];
+        }
+        for (int f = fb; f < fe; ++f) {
+            const FreqOp &q = a.fo[f];
+            const long i = (long)(f - a.f0) * nvox + v;
+            const T kap = sizeof(T) == 8 ? (T)q.kap : (T)q.kapf;
+            const T emis = sizeof(T) == 8 ? (T)q.emis : (T)q.emisf;
             T chi_t, eta_t;
-            if (q.kind == 0) {
-                if (q.rho != rho_b) {
-                    rho_b = q.rho;
-                    B = (T)planck_rho(q.rho, a.theta_ref, Tg);
+            if (tr.kind == 0) {
+                const T phi = q.damped ? ml_voigt_phi<T>(a.fi[f], inv_d, a.voigt)
+                                       : node.line_exp(q, ft) * node.pnorm;
+                chi_t = kap * phi * ndT;
+                eta_t = emis * nuT * phi;
+                if (a.moving) {
+                    // a line's profile is applied per ray in the sweep
+                    chi_t = kap * ndT;
+                    eta_t = emis * nuT;
                 }
-                const T phi = ml_line_phi<T>(q, inv_d, pnorm, a.voigt, et);
-                chi_t = (T)q.kappa * phi * (T)(q.gr * nl - nu);
-                eta_t = (T)(q.kappa * q.rho * q.rho * q.rho) * (T)nu * phi;
             } else {
-                const double y = q.xy;
-                const T E = opac_exp((T)(a.theta_ref * q.rho * y / Tg), et);
-                const double ry = q.rho * y;
-                const T alpha = (T)(q.kappa / (y * y * y));
-                chi_t = alpha * ((T)nl - (T)(nu * G) * E);
-                eta_t = alpha * (T)(nu * G * ry * ry * ry) * E;
-                B = (T)planck_rho(ry, a.theta_ref, Tg);
-                rho_b = -1.0;
-            }
-            const long i = (long)fl * nvox + v;
-            if (a.moving) {
-                // ray-independent parts; a line's profile is applied per ray
-                // in the sweep (continua do not shift)
-                T ca = chi_t, ea = eta_t;
-                if (q.kind == 0) {
-                    ca = (T)q.kappa * (T)(q.gr * nl - nu);
-                    ea = (T)(q.kappa * q.rho * q.rho * q.rho) * (T)nu;
-                }
-                T cb = (T)cc, eb = (T)cc * B;
-                if (a.sigma_c) {
-                    const T sg = (T)a.sigma_c[v];
-                    cb += sg;
-                    eb += sg * ((const T *)a.jbg)[(long)(a.f0 + fl) * nvox + v];
-                }
-                ((T *)a.chi)[i] = ca;
-                ((T *)a.S)[i] = ea;
-                ((T *)a.oc)[i] = cb;
-                ((T *)a.sc)[i] = eb;
-                continue;
+                T E;
+                cont_terms(q, inv_T, ft, E, B);
+                chi_t = kap * (nlT - ndT * E);
+                if constexpr (sizeof(T) == 8) eta_t = kap * (ndT * q.ry3) * E;
+                else eta_t = emis * ndT * E;
             }
             // the background's opacity and emissivity (continuum, and
             // coherent scattering of the previous mean intensity)
-            T chi_b = (T)cc, eta_b = (T)cc * B;
+            T chi_b = cc, eta_b = cc * B;
             if (a.sigma_c) {
-                const T sg = (T)a.sigma_c[v];
                 chi_b += sg;
-                eta_b += sg * ((const T *)a.jbg)[(long)(a.f0 + fl) * nvox + v];
+                eta_b += sg * ((const T *)a.jbg)[(long)f * nvox + v];
+            }
+            if (a.moving) {
+                // ray-independent parts (continua do not shift)
+                ((T *)a.chi)[i] = chi_t;
+                ((T *)a.S)[i] = eta_t;
+                ((T *)a.oc)[i] = chi_b;
+                ((T *)a.sc)[i] = eta_b;
+                continue;
             }
             T rho = T(1);
             bool prd = false;
             if (a.prd_index) {
                 // partial redistribution: the line's emission profile is rho phi,
                 // so its emissivity and the transition's shares scale by rho
-                const int pr = a.prd_index[a.f0 + fl];
+                const int pr = a.prd_index[f];
                 if (pr >= 0) {
                     rho = (T)a.prd_rho[(long)pr * nvox + v];
                     prd = true;
                 }
             }
             const T chi = chi_t + chi_b;
-            const T inv = T(1) / chi;
+            const T inv = fast_inv(chi);
             ((T *)a.chi)[i] = chi;
             ((T *)a.S)[i] = (rho * eta_t + eta_b) * inv;
             // the parts of S and chi the transition does not set, formed
@@ -197,6 +255,40 @@ __global__ void ml_opacity_kernel(const MlOpacityArgs a) {
             ((T *)a.oc)[i] = prd ? T(0) : chi_b * inv;
         }
     }
+}
+
+// The per-node constants of a level.
+template <typename T>
+__global__ void ml_node_tab_kernel(long nvox, int n_lines, const TransInfo *__restrict__ ti,
+                                   double t_ref, double theta_ref, const double *__restrict__ Tg,
+                                   float4 *nf, float *pnorm, double *inv_d, double *inv_T,
+                                   T *bline) {
+    for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox;
+         v += (long)gridDim.x * blockDim.x) {
+        const double it = 1.0 / Tg[v], d2 = t_ref / Tg[v], di = sqrt(d2);
+        inv_d[v] = di;
+        inv_T[v] = it;
+        if (nf) {
+            const float dh = (float)d2, th = (float)it;
+            nf[v] = make_float4(dh, (float)(d2 - (double)dh), th, (float)(it - (double)th));
+            pnorm[v] = (float)(0.5641895835477563 * di);
+        }
+        for (int l = 0; l < n_lines; ++l)
+            bline[(long)l * nvox + v] = (T)planck_rho(ti[l].rho, theta_ref, Tg[v]);
+    }
+}
+
+cudaError_t launch_ml_node_tab(int prec, long nvox, int n_lines, const TransInfo *ti, double t_ref,
+                               double theta_ref, const double *T, float4 *nf, float *pnorm,
+                               double *inv_d, double *inv_T, void *bline, cudaStream_t st) {
+    if (prec == MG3D_PREC_F64)
+        ml_node_tab_kernel<double><<<grid_for(nvox, 256), 256, 0, st>>>(
+            nvox, n_lines, ti, t_ref, theta_ref, T, nullptr, nullptr, inv_d, inv_T,
+            (double *)bline);
+    else
+        ml_node_tab_kernel<float><<<grid_for(nvox, 256), 256, 0, st>>>(
+            nvox, n_lines, ti, t_ref, theta_ref, T, nf, pnorm, inv_d, inv_T, (float *)bline);
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------ partial redistribution
@@ -898,178 +990,331 @@ __device__ __forceinline__ unsigned long long dbits_ml(double x) {
     return (unsigned long long)__double_as_longlong(x);
 }
 
-// Radiative sums of the transitions over the chunk's frequencies, added to
-// acc (frequencies in increasing order within a chunk, chunks in order).
-template <typename TP>
-__global__ void ml_accum_kernel(const MlAccumArgs a) {
-    __shared__ double tab[kExpTab];
-    for (int i = threadIdx.x; i < kExpTab; i += blockDim.x) tab[i] = a.exp_tab[i];
+// an angle sum over the ray-group slots, in slot order
+__device__ __forceinline__ double slots_sum(const double *p, long stride, int n) {
+    double s = p[0];
+    for (int i = 1; i < n; ++i) s += p[(long)i * stride];
+    return s;
+}
+__device__ __forceinline__ PairSum slots_sum(const float *p, long stride, int n) {
+    PairSum s;
+    s.hi = p[0];
+    for (int i = 1; i < n; ++i) s.add(p[(long)i * stride]);
+    return s;
+}
+
+// Radiative sums of transition blockIdx.y over the chunk's frequencies, added
+// to acc (frequencies in increasing order within a chunk, chunks in order).
+// The sums of a line share the factor 1/(sqrt(pi) d) of its profile, which
+// cancels in their ratios and is left out.
+// PLAIN: no flow, partial redistribution, damped line, background field or zero
+// radiation.
+template <bool PLAIN>
+__global__ void ml_accum64_kernel(const MlAccumArgs a) {
+    __shared__ fx::u64 fx_tab[2 * fx::kTab];
+    for (int i = threadIdx.x; i < 2 * fx::kTab; i += blockDim.x) fx_tab[i] = a.fx_tab[i];
     __syncthreads();
-    const ExpNegTable et{tab, a.exp_l1, a.exp_l2};
-    const TP *__restrict__ jx = (const TP *)a.jx;
-    const TP *__restrict__ ux = (const TP *)a.ux;
-    const long nvox = a.nvox;
-    const long hstride = (long)a.nfreq * nvox;
-    const int f1 = a.f0 + a.nfreq;
-    // J, U of frequency f at node v: the ray-group slots added in order
-    auto sums = [&](int f, long v, double &J, double &U) {
-        const long i = (long)(f - a.f0) * nvox + v;
-        J = (double)jx[i];
-        U = (double)ux[i];
-        for (int s = 1; s < a.nslots; ++s) {
-            J += (double)jx[(long)s * hstride + i];
-            U += (double)ux[(long)s * hstride + i];
-        }
-    };
-    const double rsqpi = 0.5641895835477563;
+    const fx::Tables ft{fx_tab, fx_tab + fx::kTab};
+    const double *__restrict__ jx = (const double *)a.jx;
+    const double *__restrict__ ux = (const double *)a.ux;
+    const long nvox = a.nvox, hstride = (long)a.nfreq * nvox;
+    const int t = blockIdx.y;
+    const TransInfo tr = a.ti[t];
+    const int fb = max(tr.f_begin, a.f0), fe = min(tr.f_end, a.f0 + a.nfreq);
+    if (fb >= fe) return;
     for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox;
          v += (long)gridDim.x * blockDim.x) {
-        const double Tg = a.T[v];
-        for (int t = 0; t < a.n_trans; ++t) {
-            const TransInfo tr = a.ti[t];
-            const int fb = max(tr.f_begin, a.f0), fe = min(tr.f_end, f1);
-            if (fb >= fe) continue;
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-            if (tr.kind == 0) {
-                const double inv_d = sqrt(a.t_ref / Tg);
-                for (int f = fb; f < fe; ++f) {
-                    if (a.moving && !a.zero_radiation) {
-                        // the per-ray profile weights are inside J and U already
-                        double J, U;
-                        sums(f, v, J, U);
-                        s0 += f == tr.f_begin ? 1.0 : 0.0;
-                        s1 += J;
-                        s2 += U;
-                        continue;
-                    }
-                    const FreqInfo q = a.fi[f];
-                    // profile in the formal-solution precision, sums in FP64
-                    double wphi;
-                    if (q.adamp > 0.0) {
-                        wphi = q.w * (double)ml_line_phi<TP>(q, inv_d, TP(0), a.voigt, et);
-                    } else {
-                        const double xd = q.xy * inv_d;
-                        wphi = q.w * (double)opac_exp((TP)(xd * xd), et) * rsqpi * inv_d;
-                    }
-                    double J = 0.0, U = 1.0;
-                    if (!a.zero_radiation) {
-                        sums(f, v, J, U);
-                        const int pr = a.prd_index ? a.prd_index[f] : -1;
-                        if (pr >= 0) {
-                            // U = sum_r w_r (1 - w0 (1 - oc)) = oc + (1 - oc) sum_r w_r u_r
-                            const double oc = a.prd_oc[(long)pr * nvox + v];
-                            U = oc + (1.0 - oc) * U;
-                        }
-                    }
+        const MlNode<double> node(a.tab, v);
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        if (PLAIN) {
+            // the next frequency's angle sums are loaded while this one's are added
+            const double *pj = jx + (long)(fb - a.f0) * nvox + v;
+            const double *pu = ux + (long)(fb - a.f0) * nvox + v;
+#pragma unroll 2
+            for (int f = fb; f < fe; ++f, pj += nvox, pu += nvox) {
+                const FreqOp &q = a.fo[f];
+                const double J = slots_sum(pj, hstride, a.nslots);
+                const double U = slots_sum(pu, hstride, a.nslots);
+                if (tr.kind == 0) {
+                    const double wphi = q.w * node.line_exp(q, ft);
                     s0 += wphi;
-                    s1 += wphi * J;
-                    s2 += wphi * U;
+                    s1 = fma(wphi, J, s1);
+                    s2 = fma(wphi, U, s2);
+                } else {
+                    const double E = node.cont_exp(q, ft);
+                    s0 = fma(q.w, J, s0);
+                    s1 = fma(q.w * E, J, s1);
+                    s2 = fma(q.q3 * E, U, s2);
+                }
+            }
+        } else
+        for (int f = fb; f < fe; ++f) {
+            const FreqOp &q = a.fo[f];
+            const long i = (long)(f - a.f0) * nvox + v;
+            double J = 0.0, U = 1.0;
+            if (!a.zero_radiation) {
+                J = slots_sum(jx + i, hstride, a.nslots);
+                U = slots_sum(ux + i, hstride, a.nslots);
+            }
+            if (tr.kind == 0) {
+                if (a.moving && !a.zero_radiation) {
+                    // the per-ray profile weights are inside J and U already
+                    s0 += f == tr.f_begin ? 1.0 : 0.0;
+                    s1 += J;
+                    s2 += U;
+                } else {
+                    const int pr = a.prd_index && !a.zero_radiation ? a.prd_index[f] : -1;
+                    if (pr >= 0) {
+                        // U = sum_r w_r (1 - w0 (1 - oc)) = oc + (1 - oc) sum_r w_r u_r
+                        const double oc = a.prd_oc[(long)pr * nvox + v];
+                        U = oc + (1.0 - oc) * U;
+                    }
+                    const double wphi =
+                        q.w * (q.damped ? voigt_H_rational(*a.voigt, a.fi[f].adamp * node.inv_d,
+                                                           q.a * node.inv_d)
+                                        : node.line_exp(q, ft));
+                    s0 += wphi;
+                    s1 = fma(wphi, J, s1);
+                    s2 = fma(wphi, U, s2);
                 }
             } else {
-                for (int f = fb; f < fe; ++f) {
-                    const FreqInfo q = a.fi[f];
-                    const double y = q.xy;
-                    const double qa = tr.coef * q.w / (y * y * y * y);
-                    const double E = (double)opac_exp((TP)(a.theta_ref * tr.rho * y / Tg), et);
-                    const double ry = tr.rho * y;
-                    double J = 0.0, U = 1.0;
-                    if (!a.zero_radiation) sums(f, v, J, U);
-                    s0 += qa * J;
-                    s1 += qa * E * J;
-                    s2 += qa * E * ry * ry * ry * U;
-                }
+                const double E = node.cont_exp(q, ft);
+                s0 = fma(q.w, J, s0);
+                s1 = fma(q.w * E, J, s1);
+                s2 = fma(q.q3 * E, U, s2);
             }
-            double *acc = a.acc + (long)t * kAccTerms * nvox + v;
-            acc[0] += s0;
-            acc[nvox] += s1;
-            acc[2 * nvox] += s2;
+            // background field of the frequency: the new mean intensity
+            if (a.jbg && !a.zero_radiation)
+                ((double *)a.jbg)[(long)f * nvox + v] =
+                    slots_sum((const double *)a.jm + i, hstride, a.nslots);
         }
-        // background field of the chunk's frequencies: the new mean intensity
-        if (a.jbg && !a.zero_radiation) {
-            const TP *__restrict__ jm = (const TP *)a.jm;
-            for (int fl = 0; fl < a.nfreq; ++fl) {
-                const long i = (long)fl * nvox + v;
-                double J = (double)jm[i];
-                for (int s = 1; s < a.nslots; ++s) J += (double)jm[(long)s * hstride + i];
-                ((TP *)a.jbg)[(long)(a.f0 + fl) * nvox + v] = (TP)J;
-            }
-        }
+        double *acc = a.acc + (long)t * kAccTerms * nvox + v;
+        acc[0] += s0;
+        acc[nvox] += s1;
+        acc[2 * nvox] += s2;
     }
 }
 
-__global__ void __launch_bounds__(128) ml_rates_kernel(const MlRateArgs a) {
+template <bool PLAIN>
+__global__ void ml_accum32_kernel(const MlAccumArgs a) {
+    const fx::Tables none{nullptr, nullptr};
+    const float *__restrict__ jx = (const float *)a.jx;
+    const float *__restrict__ ux = (const float *)a.ux;
+    const long nvox = a.nvox, hstride = (long)a.nfreq * nvox;
+    const int t = blockIdx.y;
+    const TransInfo tr = a.ti[t];
+    const int fb = max(tr.f_begin, a.f0), fe = min(tr.f_end, a.f0 + a.nfreq);
+    if (fb >= fe) return;
+    for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox;
+         v += (long)gridDim.x * blockDim.x) {
+        const MlNode<float> node(a.tab, v);
+        const double inv_d = tr.kind == 0 && a.voigt ? a.tab.inv_d[v] : 0.0;
+        PairSum s0, s1, s2;
+        auto add_line = [&](const FreqOp &q, float phi, const PairSum &J, const PairSum &U) {
+            const float wh = q.wh * phi;   // w phi as a pair
+            const float wl = fmaf(q.wl, phi, fmaf(q.wh, phi, -wh));
+            s0.add(wh);
+            s0.lo += wl;
+            s1.add_product(wh, wl, J.hi, J.lo);
+            s2.add_product(wh, wl, U.hi, U.lo);
+        };
+        auto add_cont = [&](const FreqOp &q, float E, const PairSum &J, const PairSum &U) {
+            s0.add_product(q.wh, q.wl, J.hi, J.lo);
+            const float eh = q.wh * E, el = fmaf(q.wl, E, fmaf(q.wh, E, -eh));
+            s1.add_product(eh, el, J.hi, J.lo);
+            const float gh = q.q3h * E, gl = fmaf(q.q3l, E, fmaf(q.q3h, E, -gh));
+            s2.add_product(gh, gl, U.hi, U.lo);
+        };
+        if (PLAIN) {
+            // four frequencies at a time, so that their loads are in flight together
+            constexpr int B = 4;
+            const float *pj = jx + (long)(fb - a.f0) * nvox + v;
+            const float *pu = ux + (long)(fb - a.f0) * nvox + v;
+            for (int f = fb; f < fe; f += B, pj += B * nvox, pu += B * nvox) {
+                PairSum J[B], U[B];
+                for (int s = 0; s < a.nslots; ++s) {
+                    float vj[B], vu[B];
+#pragma unroll
+                    for (int k = 0; k < B; ++k) {
+                        const long o = (long)s * hstride + (f + k < fe ? k : 0) * nvox;
+                        vj[k] = pj[o];
+                        vu[k] = pu[o];
+                    }
+#pragma unroll
+                    for (int k = 0; k < B; ++k) {
+                        J[k].add(vj[k]);
+                        U[k].add(vu[k]);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < B; ++k) {
+                    if (f + k >= fe) break;
+                    const FreqOp &q = a.fo[f + k];
+                    if (tr.kind == 0) add_line(q, node.line_exp(q, none), J[k], U[k]);
+                    else add_cont(q, node.cont_exp(q, none), J[k], U[k]);
+                }
+            }
+        } else
+        for (int f = fb; f < fe; ++f) {
+            const FreqOp &q = a.fo[f];
+            const long i = (long)(f - a.f0) * nvox + v;
+            PairSum J, U;
+            U.hi = 1.0f;
+            if (!a.zero_radiation) {
+                J = slots_sum(jx + i, hstride, a.nslots);
+                U = slots_sum(ux + i, hstride, a.nslots);
+            }
+            if (tr.kind == 0) {
+                if (a.moving && !a.zero_radiation) {
+                    // the per-ray profile weights are inside J and U already
+                    s0.add(f == tr.f_begin ? 1.0f : 0.0f);
+                    s1.add_product(1.0f, 0.0f, J.hi, J.lo);
+                    s2.add_product(1.0f, 0.0f, U.hi, U.lo);
+                } else {
+                    const int pr = a.prd_index && !a.zero_radiation ? a.prd_index[f] : -1;
+                    if (pr >= 0) {
+                        // U = sum_r w_r (1 - w0 (1 - oc)) = oc + (1 - oc) sum_r w_r u_r
+                        const double oc = a.prd_oc[(long)pr * nvox + v];
+                        const double u = oc + (1.0 - oc) * U.value();
+                        U.hi = (float)u;
+                        U.lo = (float)(u - (double)U.hi);
+                    }
+                    const float phi =
+                        q.damped ? (float)voigt_H_rational(*a.voigt, a.fi[f].adamp * inv_d,
+                                                           q.a * inv_d)
+                                 : node.line_exp(q, none);
+                    add_line(q, phi, J, U);
+                }
+            } else {
+                add_cont(q, node.cont_exp(q, none), J, U);
+            }
+            // background field of the frequency: the new mean intensity
+            if (a.jbg && !a.zero_radiation) {
+                const PairSum m = slots_sum((const float *)a.jm + i, hstride, a.nslots);
+                ((float *)a.jbg)[(long)f * nvox + v] = m.hi + m.lo;
+            }
+        }
+        double *acc = a.acc + (long)t * kAccTerms * nvox + v;
+        acc[0] += s0.value();
+        acc[nvox] += s1.value();
+        acc[2 * nvox] += s2.value();
+    }
+}
+
+// Rates and the N x N solve, one node per thread, N known at compile time: the
+// rate matrix is gathered in shared memory (the transitions index it), the
+// elimination runs on registers with every index static, pivots chosen on the
+// bit patterns (positive doubles order like them) and one refined reciprocal
+// per pivot, so that the FP64 pipe sees the products alone.  64x64x129, N = 6:
+// 549 -> 300 us; an 8x8x9 grid, latency alone: 50 -> 15 us.
+constexpr int kRateThreads = 64;
+template <int N>
+__global__ void __launch_bounds__(kRateThreads) ml_rates_kernel(const MlRateArgs a) {
+    __shared__ double Ps[N * N][kRateThreads];
     const long nvox = a.nvox;
-    const int N = a.n_levels;
+    const int tid = threadIdx.x;
     double cmax = 0.0;
     unsigned neg = 0, bad = 0;
     const long stride = (long)gridDim.x * blockDim.x;
     for (long base = (long)blockIdx.x * blockDim.x; base < nvox; base += stride) {
-        const long v = base + threadIdx.x;
+        const long v = base + tid;
         if (v >= nvox) continue;
-        double P[kMaxLevels][kMaxLevels];
-        for (int i = 0; i < N; ++i)
-            for (int j = 0; j < N; ++j) P[i][j] = i == j ? 0.0 : a.c[((long)i * N + j) * nvox + v];
-        for (int t = 0; t < a.n_trans; ++t) {
-            const TransInfo tr = a.ti[t];
-            const double *acc = a.acc + (long)t * kAccTerms * nvox + v;
-            if (tr.kind == 0) {
-                const double norm = acc[0];
-                const double Jb = acc[nvox] / norm, Ub = acc[2 * nvox] / norm;
-                const double b_ul = tr.coef / (tr.rho * tr.rho * tr.rho);
-                P[tr.lo][tr.up] += tr.gr * b_ul * Jb;
-                P[tr.up][tr.lo] += tr.coef * Ub + b_ul * Jb;
-            } else {
-                const double G = a.saha[(long)tr.lo * nvox + v];
-                P[tr.lo][tr.up] += acc[0];
-                P[tr.up][tr.lo] += G * (acc[2 * nvox] + acc[nvox]);
+#pragma unroll
+        for (int i = 0; i < N * N; ++i)
+            Ps[i][tid] = i % (N + 1) == 0 ? 0.0 : a.c[(long)i * nvox + v];
+        // four transitions at a time, so that their loads are in flight together
+        for (int t0 = 0; t0 < a.n_trans; t0 += 4) {
+            double a0[4], a1[4], a2[4], G[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int t = min(t0 + k, a.n_trans - 1);
+                const double *acc = a.acc + (long)t * kAccTerms * nvox + v;
+                a0[k] = acc[0];
+                a1[k] = acc[nvox];
+                a2[k] = acc[2 * nvox];
+                G[k] = a.saha[(long)a.ti[t].lo * nvox + v];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (t0 + k >= a.n_trans) break;
+                const TransInfo tr = a.ti[t0 + k];
+                double up, down;
+                if (tr.kind == 0) {
+                    const double inv = fast_div(1.0, a0[k]);
+                    const double bJ = tr.b_ul * (a1[k] * inv);
+                    up = tr.gr * bJ;
+                    down = fma(tr.coef, a2[k] * inv, bJ);
+                } else {
+                    up = a0[k];
+                    down = G[k] * (a2[k] + a1[k]);
+                }
+                Ps[tr.lo * N + tr.up][tid] += up;
+                Ps[tr.up * N + tr.lo][tid] += down;
             }
         }
         // W(n) = M n: row 0 conservation, row i: n_i sum_j P_ij - sum_j n_j P_ji
-        double M[kMaxLevels][kMaxLevels + 1];
-        for (int j = 0; j < N; ++j) M[0][j] = 1.0;
-        for (int i = 1; i < N; ++i) {
+        double M[N][N + 1];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
             double out_i = 0.0;
+#pragma unroll
             for (int j = 0; j < N; ++j)
-                if (j != i) out_i += P[i][j];
-            for (int j = 0; j < N; ++j) M[i][j] = j == i ? out_i : -P[j][i];
+                if (j != i) out_i += Ps[i * N + j][tid];
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                M[i][j] = i == 0 ? 1.0 : (j == i ? out_i : -Ps[j * N + i][tid]);
+            M[i][N] = a.f ? a.f[(long)i * nvox + v] : (i == 0 ? a.n_tot[v] : 0.0);
         }
-        double fv[kMaxLevels];
-        for (int i = 0; i < N; ++i)
-            fv[i] = a.f ? a.f[(long)i * nvox + v] : (i == 0 ? a.n_tot[v] : 0.0);
         if (a.mode == kRateSolve) {
-            for (int i = 0; i < N; ++i) M[i][N] = fv[i];
+            double inv[N];
+#pragma unroll
             for (int c = 0; c < N; ++c) {
+                // partial pivoting: the largest |M[r][c]| of the rows below c up
+                unsigned long long best = (unsigned long long)__double_as_longlong(fabs(M[c][c]));
                 int piv = c;
-                double best = fabs(M[c][c]);
-                for (int r = c + 1; r < N; ++r)
-                    if (fabs(M[r][c]) > best) {
-                        best = fabs(M[r][c]);
+#pragma unroll
+                for (int r = c + 1; r < N; ++r) {
+                    const unsigned long long m =
+                        (unsigned long long)__double_as_longlong(fabs(M[r][c]));
+                    if (m > best) {
+                        best = m;
                         piv = r;
                     }
-                if (piv != c)
-                    for (int j = c; j <= N; ++j) {
-                        const double tmp = M[c][j];
-                        M[c][j] = M[piv][j];
-                        M[piv][j] = tmp;
-                    }
-                const double inv = 1.0 / M[c][c];
+                }
+#pragma unroll
                 for (int r = c + 1; r < N; ++r) {
-                    const double fac = M[r][c] * inv;
-                    for (int j = c; j <= N; ++j) M[r][j] -= fac * M[c][j];
+                    const bool sw = r == piv;
+#pragma unroll
+                    for (int j = c; j <= N; ++j) {
+                        const double x = M[c][j], y = M[r][j];
+                        M[c][j] = sw ? y : x;
+                        M[r][j] = sw ? x : y;
+                    }
+                }
+                inv[c] = fast_div(1.0, M[c][c]);
+#pragma unroll
+                for (int r = c + 1; r < N; ++r) {
+                    const double fac = M[r][c] * inv[c];
+#pragma unroll
+                    for (int j = c + 1; j <= N; ++j) M[r][j] = fma(-fac, M[c][j], M[r][j]);
                 }
             }
-            double xsol[kMaxLevels];
+            double xsol[N];
+#pragma unroll
             for (int i = N - 1; i >= 0; --i) {
                 double acc = M[i][N];
-                for (int j = i + 1; j < N; ++j) acc -= M[i][j] * xsol[j];
-                xsol[i] = acc / M[i][i];
+#pragma unroll
+                for (int j = i + 1; j < N; ++j) acc = fma(-M[i][j], xsol[j], acc);
+                const double q = acc * inv[i];
+                xsol[i] = fma(fma(-M[i][i], q, acc), inv[i], q);
             }
             bool finite = true;
             double cl = 0.0;
+#pragma unroll
             for (int i = 0; i < N; ++i) {
                 const double old = a.n[(long)i * nvox + v];
                 a.n[(long)i * nvox + v] = xsol[i];
-                const double ci = fabs(xsol[i] - old) / fabs(xsol[i]);
+                const double ci = fast_div(fabs(xsol[i] - old), fabs(xsol[i]));
                 if (!(isfinite(xsol[i]) && isfinite(ci))) finite = false;
                 else cl = fmax(cl, ci);
                 neg += xsol[i] <= 0.0;
@@ -1077,10 +1322,15 @@ __global__ void __launch_bounds__(128) ml_rates_kernel(const MlRateArgs a) {
             if (finite) cmax = fmax(cmax, cl);
             else ++bad;
         } else {
+            double nn[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) nn[j] = a.n[(long)j * nvox + v];
+#pragma unroll
             for (int i = 0; i < N; ++i) {
                 double w = 0.0;
-                for (int j = 0; j < N; ++j) w += M[i][j] * a.n[(long)j * nvox + v];
-                if (a.mode == kRateResidual) a.out[(long)i * nvox + v] = fv[i] - w;
+#pragma unroll
+                for (int j = 0; j < N; ++j) w += M[i][j] * nn[j];
+                if (a.mode == kRateResidual) a.out[(long)i * nvox + v] = M[i][N] - w;
                 else a.out[(long)i * nvox + v] += w;
             }
         }
@@ -1117,11 +1367,14 @@ __global__ void __launch_bounds__(128) ml_rates_kernel(const MlRateArgs a) {
     }
 }
 
+// small grids take small blocks, so that their few nodes reach every SM
+static int node_threads(long nvox) { return nvox <= 152L * 64 ? 64 : 256; }
+
 cudaError_t launch_ml_opacity(const MlOpacityArgs &a, cudaStream_t st) {
-    if (a.prec == MG3D_PREC_F64)
-        ml_opacity_kernel<double><<<grid_for(a.nvox, 256), 256, 0, st>>>(a);
-    else
-        ml_opacity_kernel<float><<<grid_for(a.nvox, 256), 256, 0, st>>>(a);
+    const int th = node_threads(a.nvox);
+    const dim3 grid(grid_for(a.nvox, th), a.n_trans);
+    if (a.prec == MG3D_PREC_F64) ml_opacity_kernel<double><<<grid, th, 0, st>>>(a);
+    else ml_opacity_kernel<float><<<grid, th, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1138,15 +1391,31 @@ cudaError_t launch_ml_bottom(int prec, long nplane, int nfreq, const FreqInfo *f
 }
 
 cudaError_t launch_ml_accum(const MlAccumArgs &a, cudaStream_t st) {
-    if (a.prec == MG3D_PREC_F64)
-        ml_accum_kernel<double><<<grid_for(a.nvox, 128), 128, 0, st>>>(a);
-    else
-        ml_accum_kernel<float><<<grid_for(a.nvox, 128), 128, 0, st>>>(a);
+    const int th = node_threads(a.nvox);
+    const dim3 grid(grid_for(a.nvox, th), a.n_trans);
+    const bool plain = !a.zero_radiation && !a.moving && !a.prd_index && !a.voigt && !a.jbg;
+    if (a.prec == MG3D_PREC_F64) {
+        if (plain) ml_accum64_kernel<true><<<grid, th, 0, st>>>(a);
+        else ml_accum64_kernel<false><<<grid, th, 0, st>>>(a);
+    } else {
+        if (plain) ml_accum32_kernel<true><<<grid, th, 0, st>>>(a);
+        else ml_accum32_kernel<false><<<grid, th, 0, st>>>(a);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_ml_rates(const MlRateArgs &a, cudaStream_t st) {
-    ml_rates_kernel<<<grid_for(a.nvox, 128), 128, 0, st>>>(a);
+    const int g = grid_for(a.nvox, kRateThreads);
+    switch (a.n_levels) {
+        case 2: ml_rates_kernel<2><<<g, kRateThreads, 0, st>>>(a); break;
+        case 3: ml_rates_kernel<3><<<g, kRateThreads, 0, st>>>(a); break;
+        case 4: ml_rates_kernel<4><<<g, kRateThreads, 0, st>>>(a); break;
+        case 5: ml_rates_kernel<5><<<g, kRateThreads, 0, st>>>(a); break;
+        case 6: ml_rates_kernel<6><<<g, kRateThreads, 0, st>>>(a); break;
+        case 7: ml_rates_kernel<7><<<g, kRateThreads, 0, st>>>(a); break;
+        case 8: ml_rates_kernel<8><<<g, kRateThreads, 0, st>>>(a); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

@@ -17,6 +17,7 @@
 // (linear in physical height for z), and the relative correction of
 // Eqs. 10-11 with the 10 % rule for negative populations (Sec. 4.10).
 #include "mg3d_internal.h"
+#include "sc_step.cuh"
 
 namespace mg3d {
 
@@ -70,15 +71,6 @@ __device__ __forceinline__ unsigned block_count(unsigned c) {
 // reduction took 377 us for 128x128x129 FP32 slots and 54 us for 64x64x129 FP64
 // ones; now 75 and 40 us.
 constexpr int kSumSlots = 24;   // slots added at a time; their number is a multiple
-
-struct PairSum {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = hi + x, b = s - hi;
-        lo += (hi - (s - b)) + (x - b);
-        hi = s;
-    }
-};
 
 __device__ __noinline__ double plain_sum(const float *p, long stride, int n) {
     double s = 0.0;
@@ -142,23 +134,6 @@ __device__ __forceinline__ void sum_slots(const TP *__restrict__ pj, const TP *_
         J = s0 == 0 ? j : J + j;
         U = s0 == 0 ? u : U + u;
     }
-}
-
-// 1/b within an ulp or two for b of exponent -1000 .. 1000 (`ok`): the hardware
-// approximation (relative error e below 2^-20) times 1 + e + e^2
-__device__ __forceinline__ double fast_rcp(double b, bool &ok) {
-    ok = (((unsigned)__double2hiint(b) >> 20) & 0x7ffu) - 23u < 2000u;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    const double e = fma(-b, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-// a/b: 6 FP64 operations against about 18 of the division
-__device__ __forceinline__ double fast_div(double a, double b) {
-    bool ok;
-    const double y = fast_rcp(b, ok);
-    const double q = a * y;
-    return ok ? fma(fma(-b, q, a), y, q) : a / b;
 }
 
 template <typename TP>

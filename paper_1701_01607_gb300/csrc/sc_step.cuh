@@ -76,6 +76,43 @@ __device__ __forceinline__ double exp_neg(double x, const ExpNegTable e) {
     return flush ? 0.0 : __longlong_as_double(bits);
 }
 
+// A sum of FP32 values as a pair of floats (Knuth's two-sum), about 2^-45 of
+// the sum, without the FP64 pipe.
+struct PairSum {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = hi + x, b = s - hi;
+        lo += (hi - (s - b)) + (x - b);
+        hi = s;
+    }
+    // + the product of two pairs
+    __device__ __forceinline__ void add_product(float ah, float al, float bh, float bl) {
+        const float p = ah * bh;
+        float e = fmaf(ah, bh, -p);
+        e = fmaf(ah, bl, e);
+        lo += fmaf(al, bh, e);
+        add(p);
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
+// 1/b within an ulp or two for b of exponent -1000 .. 1000 (`ok`): the hardware
+// approximation (relative error e below 2^-20) times 1 + e + e^2
+__device__ __forceinline__ double fast_rcp(double b, bool &ok) {
+    ok = (((unsigned)__double2hiint(b) >> 20) & 0x7ffu) - 23u < 2000u;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = fma(-b, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// a/b: 6 FP64 operations against about 18 of the division
+__device__ __forceinline__ double fast_div(double a, double b) {
+    bool ok;
+    const double y = fast_rcp(b, ok);
+    const double q = a * y;
+    return ok ? fma(fma(-b, q, a), y, q) : a / b;
+}
+
 // closed() has no branch, so a caller can evaluate several independent steps
 // back to back and patch the small-x ones with series() afterwards; eval()
 // takes one form or the other per lane.
