@@ -495,19 +495,17 @@ int mg3d_get_ml_shape_ex(const mg3d_handle *h, int level, int *bands, int *rays_
 
 /* ------------------------------------------------------------------------
  * Batches: many independent atmospheres of uneven size (two-level and
- * multi-level atoms mixed) iterated in lockstep.  Every formal solution of
- * the batch is one launch per atom kind whose thread-block clusters each
- * take one (member, ray or hemisphere, frequency group) of a shared work
- * table; the other per-node kernels run per member; a whole batched V-cycle
- * is captured once into a CUDA graph and replayed.  Members must share
+ * multi-level atoms mixed) advanced together.  A batched V-cycle runs every
+ * member's own V-cycle (its captured CUDA graph) on a stream of the member's
+ * own, so that the members' kernels overlap on the GPU; results are those of
+ * the members run alone.  Members must share
  * n_grids, the formal-solution precision and the multigrid schedule; creating
- * the batch moves them onto the batch's stream and fixes their sweep shapes
- * (a common number of bands per level), so they should not be autotuned or
- * used alone while the batch exists.  The batch does not own its members. */
+ * the batch moves them onto streams of the batch, so they should not be used
+ * from elsewhere while the batch exists.  The batch does not own its members. */
 typedef struct mg3d_batch mg3d_batch;
 int mg3d_batch_create(int n, mg3d_handle *const *members, mg3d_batch **out);
 int mg3d_batch_destroy(mg3d_batch *b);
-/* One lockstep V-cycle; max_rel_change (nullable) receives C of each member
+/* One V-cycle of every member; max_rel_change (nullable) receives C of each member
  * ([n] doubles).
  * The V-cycle of Sec. 2.2 per member; batching has no counterpart in the
  * paper. */

@@ -628,17 +628,6 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_kernel(const SweepArgs<T> a)
     sweep_body<T, STAGE, MODE>(a, blockIdx.y, blockIdx.z);
 }
 
-// Batched sweep: cluster y of the grid runs work item items[y] = (problem,
-// ray, group) of problems args[]; every problem uses the launch's number of
-// bands.
-template <typename T, int MAXT>
-__global__ void __launch_bounds__(MAXT, 1024 / MAXT) sweep_batch_kernel(
-    const SweepArgs<T> *__restrict__ args, const BatchItem *__restrict__ items) {
-    const BatchItem it = items[blockIdx.y];
-    const SweepArgs<T> a = args[it.member];
-    sweep_body<T, true, kSweepLinear>(a, it.group, it.ray);
-}
-
 __global__ void exp_check_kernel(int n, const double *__restrict__ x, double *__restrict__ out,
                                  const double *__restrict__ tab, double l1, double l2) {
     const ExpNegTable et{tab, l1, l2};
@@ -785,44 +774,6 @@ static cudaError_t clusters_any(const SweepShape &s, int nx, int *n) {
 cudaError_t sweep_active_clusters(int prec, const SweepShape &s, int nx, int *n) {
     *n = 0;
     return prec == 0 ? clusters_any<double>(s, nx, n) : clusters_any<float>(s, nx, n);
-}
-
-template <typename T, int MAXT>
-static cudaError_t launch_sweep_batch_t(const SweepArgs<T> *args, const BatchItem *items,
-                                        int n_items, int bands, int threads, size_t smem,
-                                        cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(sweep_batch_kernel<T, MAXT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kMaxSweepSmem);  // fixed, as for sweep_kernel
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(bands, n_items, 1);
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = bands;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = bands > 1 ? 1 : 0;  // one band: a plain launch
-    return cudaLaunchKernelEx(&cfg, sweep_batch_kernel<T, MAXT>, args, items);
-}
-
-cudaError_t launch_sweep_batch(int prec, const void *args, const BatchItem *items, int n_items,
-                               int bands, int threads, size_t smem, cudaStream_t st) {
-    if (prec == 0)
-        return threads <= 256
-                   ? launch_sweep_batch_t<double, 256>((const SweepArgs<double> *)args, items,
-                                                       n_items, bands, threads, smem, st)
-                   : launch_sweep_batch_t<double, 512>((const SweepArgs<double> *)args, items,
-                                                       n_items, bands, threads, smem, st);
-    return threads <= 256
-               ? launch_sweep_batch_t<float, 256>((const SweepArgs<float> *)args, items, n_items,
-                                                  bands, threads, smem, st)
-               : launch_sweep_batch_t<float, 512>((const SweepArgs<float> *)args, items, n_items,
-                                                  bands, threads, smem, st);
 }
 
 cudaError_t launch_sweep_f64(const SweepArgs<double> &a, const SweepShape &s, cudaStream_t st) {

@@ -203,13 +203,6 @@ cudaError_t launch_prd_collect(int prec, long len, const void *slots, void *jnu,
 cudaError_t launch_xslopes(int prec, int nx, long nvox, const void *a, const void *b, void *da,
                            void *db, cudaStream_t st);
 
-// One cluster of a batched sweep: problem index, ray (two-level) or
-// hemisphere (multi-level), frequency group (two-level) or frequency.
-struct BatchItem {
-    int member, ray, group;
-};
-cudaError_t launch_sweep_batch(int prec, const void *args, const BatchItem *items, int n_items,
-                               int bands, int threads, size_t smem, cudaStream_t st);
 
 // Kernel launchers; each returns the launch error.
 cudaError_t launch_opacity(int prec, long nvox, double g_ratio, double kappa,
@@ -508,8 +501,5 @@ cudaError_t launch_ml_sweep_f32(const MlSweepArgs<float> &a, int bands, int thre
                                 cudaStream_t st);
 cudaError_t launch_ml_accum(const MlAccumArgs &a, cudaStream_t st);
 cudaError_t launch_ml_rates(const MlRateArgs &a, cudaStream_t st);
-cudaError_t launch_ml_sweep_batch(int prec, const void *args, const BatchItem *items,
-                                  int n_items, int bands, int threads, size_t smem,
-                                  cudaStream_t st);
 
 }  // namespace mg3d

@@ -817,15 +817,6 @@ __global__ void __launch_bounds__(MAXT) ml_sweep_kernel(const MlSweepArgs<T> a) 
     ml_sweep_body<T, MODE>(a, blockIdx.y, blockIdx.z);
 }
 
-// Batched: item y = (problem, ray-group slot as ray, frequency as group).
-template <typename T, int MAXT>
-__global__ void __launch_bounds__(MAXT) ml_sweep_batch_kernel(
-    const MlSweepArgs<T> *__restrict__ args, const BatchItem *__restrict__ items) {
-    const BatchItem it = items[blockIdx.y];
-    const MlSweepArgs<T> a = args[it.member];
-    ml_sweep_body<T, kSweepLinear>(a, it.group, it.ray);
-}
-
 size_t ml_sweep_smem_bytes(int prec, int rows, int nx, int rpb, int herm, int moving) {
     const size_t elem = prec == MG3D_PREC_F64 ? sizeof(double) : sizeof(float);
     // moving: intensity, opacity and source planes and the 24-byte table
@@ -865,46 +856,6 @@ static cudaError_t launch_ml_sweep_t(const MlSweepArgs<T> &a, int bands, int thr
     cfg.attrs = attr;
     cfg.numAttrs = bands > 1 ? 1 : 0;  // one band: a plain launch
     return cudaLaunchKernelEx(&cfg, ml_sweep_kernel<T, MAXT, MODE>, a);
-}
-
-template <typename T, int MAXT>
-static cudaError_t launch_ml_sweep_batch_t(const MlSweepArgs<T> *args, const BatchItem *items,
-                                           int n_items, int bands, int threads, size_t smem,
-                                           cudaStream_t st) {
-    // one fixed limit for every launch, so graph replays never meet a lower one
-    cudaError_t e = cudaFuncSetAttribute(ml_sweep_batch_kernel<T, MAXT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kMaxSweepSmem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(bands, n_items, 1);
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = bands;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = bands > 1 ? 1 : 0;  // one band: a plain launch
-    return cudaLaunchKernelEx(&cfg, ml_sweep_batch_kernel<T, MAXT>, args, items);
-}
-
-cudaError_t launch_ml_sweep_batch(int prec, const void *args, const BatchItem *items,
-                                  int n_items, int bands, int threads, size_t smem,
-                                  cudaStream_t st) {
-    if (prec == MG3D_PREC_F64)
-        return threads <= 256
-                   ? launch_ml_sweep_batch_t<double, 256>((const MlSweepArgs<double> *)args,
-                                                          items, n_items, bands, threads, smem, st)
-                   : launch_ml_sweep_batch_t<double, 512>((const MlSweepArgs<double> *)args,
-                                                          items, n_items, bands, threads, smem, st);
-    return threads <= 256
-               ? launch_ml_sweep_batch_t<float, 256>((const MlSweepArgs<float> *)args, items,
-                                                     n_items, bands, threads, smem, st)
-               : launch_ml_sweep_batch_t<float, 512>((const MlSweepArgs<float> *)args, items,
-                                                     n_items, bands, threads, smem, st);
 }
 
 template <typename T>
@@ -1096,7 +1047,7 @@ __global__ void ml_accum64_kernel(const MlAccumArgs a) {
 }
 
 template <bool PLAIN>
-__global__ void ml_accum32_kernel(const MlAccumArgs a) {
+__global__ void __launch_bounds__(256) ml_accum32_kernel(const MlAccumArgs a) {
     const fx::Tables none{nullptr, nullptr};
     const float *__restrict__ jx = (const float *)a.jx;
     const float *__restrict__ ux = (const float *)a.ux;
@@ -1132,19 +1083,24 @@ __global__ void ml_accum32_kernel(const MlAccumArgs a) {
             const float *pu = ux + (long)(fb - a.f0) * nvox + v;
             for (int f = fb; f < fe; f += B, pj += B * nvox, pu += B * nvox) {
                 PairSum J[B], U[B];
-                for (int s = 0; s < a.nslots; ++s) {
-                    float vj[B], vu[B];
+                // two slots (all rays of a hemisphere in one block) at a time
+                for (int s = 0; s < a.nslots; s += 2) {
+                    float vj[2][B], vu[2][B];
 #pragma unroll
-                    for (int k = 0; k < B; ++k) {
-                        const long o = (long)s * hstride + (f + k < fe ? k : 0) * nvox;
-                        vj[k] = pj[o];
-                        vu[k] = pu[o];
-                    }
+                    for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int k = 0; k < B; ++k) {
-                        J[k].add(vj[k]);
-                        U[k].add(vu[k]);
-                    }
+                        for (int k = 0; k < B; ++k) {
+                            const long o = (long)(s + h) * hstride + (f + k < fe ? k : 0) * nvox;
+                            vj[h][k] = pj[o];
+                            vu[h][k] = pu[o];
+                        }
+#pragma unroll
+                    for (int k = 0; k < B; ++k)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            J[k].add(vj[h][k]);
+                            U[k].add(vu[h][k]);
+                        }
                 }
 #pragma unroll
                 for (int k = 0; k < B; ++k) {
