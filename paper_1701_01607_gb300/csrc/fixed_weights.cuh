@@ -192,7 +192,7 @@ __device__ __forceinline__ Weights closed(u64 Y, int ey, u64 V, int ve, const Ta
     w.um = mulhi(w.D, V);
     w.ue = ve;
     w.u = ve >= 0 ? w.um << ve : shr(w.um, -ve);
-    w.w0 = pack32(0ull - w.u, 0);
+    w.w0 = pack32(w.u ? 0ull - w.u : ~0ull, 0);   // x > 2^64: u rounds to 0
     // where e^-x is below 2^-64, w_up = u
     w.wup = Eq ? pack32(w.u - Eq, 0) : pack32(w.um, ve);
     return w;

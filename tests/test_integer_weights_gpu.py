@@ -62,3 +62,22 @@ def test_optical_paths_of_every_size(scale, nx, ny, shape):
     jo, uo = reference(atm, atom, n)
     assert np.max(np.abs(jeff - jo) / np.abs(jo)) < 1e-12
     assert np.max(np.abs(u - uo) / np.abs(uo)) < 1e-12
+
+
+@pytest.mark.parametrize("thick", [1e12, 1e18, 1e24, 1e200])
+def test_thin_layers_above_a_thick_one(thick):
+    """Steps of paths beyond 2^64, whose u is below a unit of the fractions,
+    hand their source function (w0 = 1) to thin layers."""
+    atm, atom = synth.stratified_two_level(8, 8, 9, eps=1e-3, sigma=0.3, seed=5,
+                                           tau_top=1e-2, tau_bottom=1e2,
+                                           atom=synth.TwoLevelAtom(n_freq=9))
+    atm.n_tot[3:6] *= thick
+    h = m.mg3d_create(atm, atom, n_grids=1)
+    try:
+        jeff, u = m.mg3d_formal_solve(h, 1)
+        n = m.mg3d_get_populations(h, 1)
+    finally:
+        m.mg3d_destroy(h)
+    jo, uo = reference(atm, atom, n)
+    assert np.max(np.abs(jeff - jo) / np.abs(jo)) < 1e-12
+    assert np.max(np.abs(u - uo) / np.abs(uo)) < 1e-12
