@@ -85,6 +85,7 @@ struct Level {
     StepGeom *geom = nullptr;    // [kRays][nz]
     void *psteps = nullptr;      // [kRays][nz] PlaneLerp<T> of the shifted-plane sweeps
     SweepShape shape{};
+    SweepShape band_shape{};     // with shape.plane 3: the band sweep's shape, as reported
     // formal solutions in the precision other than the handle's (built on the
     // first request, two-level static CRD handles): chi0, S, the bottom
     // intensity, the plane-sweep step table, and the shape
@@ -529,8 +530,9 @@ int sm_count() {
 // How many clusters of shape s the GPU holds at once (plain launches: blocks).
 int shape_capacity(int prec, const SweepShape &s, int nx) {
     int n = 0;
-    const cudaError_t e = s.plane ? plane_active_clusters(prec, s, nx, &n)
-                                  : sweep_active_clusters(prec, s, nx, &n);
+    const cudaError_t e = s.plane == 3 ? plane_var_clusters(prec, s, nx, &n)
+                          : s.plane    ? plane_active_clusters(prec, s, nx, &n)
+                                       : sweep_active_clusters(prec, s, nx, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -589,6 +591,71 @@ SweepShape choose_plane_shape(int prec, int nx, int ny, int nfreq) {
         if (best_waves) return best;
     }
     return SweepShape{};
+}
+
+// Shape of the variants' shifted-plane sweep with `np` slots per group, `bands`
+// bands and up to 512 threads; ng 0 where it does not fit.
+SweepShape var_shape(int prec, int nx, int ny, int nslots, int prd, int np, int bands, int max_th) {
+    SweepShape s{};
+    const int rows = (ny + bands - 1) / bands;
+    if (bands > ny || (long)(bands - 1) * rows >= ny) return s;
+    // one thread per node; spare threads share a node's slots
+    int th = std::max(32, std::min(max_th, ((rows * nx + 31) / 32) * 32));
+    if (rows * nx <= th)
+        th *= std::max(1, std::min(max_th / th, prec == MG3D_PREC_F64 ? np : (np + 1) / 2));
+    if (plane_var_layout(prec, prd, np, rows, nx, th).smem > plane_smem_max(prec == MG3D_PREC_F64))
+        return s;
+    s = SweepShape{np, (nslots + np - 1) / np, bands, rows, th};
+    s.stage = 0;
+    s.plane = 3;
+    s.np = np;
+    s.prd = prd;
+    s.vel = prd ? 0 : 1;
+    return s;
+}
+
+// Default shape of the variants' sweep: the least estimated time of a plane step
+// times the waves of clusters it takes.  A step is a latency (the barrier, and the
+// chain of a thread's slots) plus the arithmetic of the blocks that share an SM
+// (ns per node and per slot; blocks that share one hide each other's waits).  The
+// constants were fitted to 630 timed shapes on nine grids of 16x16 to 64x64 nodes:
+// the shape picked is within 6 % of the fastest in seven of them (48x48x97, 17
+// frequencies, FP32: one group of 5 bands, 504 us, where three groups take 609;
+// 64x64x65: three groups of 8 bands, 568 against 730 for one group), and within
+// 12 and 29 % at 16x16 nodes (54 us for 42).
+SweepShape choose_var_shape(int prec, int nx, int ny, int nslots, int prd) {
+    const bool f64 = prec == MG3D_PREC_F64;
+    const double t0 = f64 ? 1650.0 : 400.0, chain = f64 ? 700.0 : 900.0;
+    const double node = f64 ? 0.25 : 9.0, slot = f64 ? (prd ? 5.9 : 0.5) : 0.15;
+    const double shared = f64 ? 0.8 : 0.57;
+    SweepShape best{};
+    double best_t = 0.0;
+    for (int groups = 1; groups <= std::min(nslots, 6); ++groups) {
+        const int np = (nslots + groups - 1) / groups;
+        if ((nslots + np - 1) / np != groups) continue;
+        for (int bands = 1; bands <= kPortableBands; ++bands)
+            for (int cap : {256, 512}) {
+                const SweepShape s = var_shape(prec, nx, ny, nslots, prd, np, bands, cap);
+                if (s.ng == 0 || (cap == 512 && s.threads <= 256)) continue;
+                const int held = shape_capacity(prec, s, nx);
+                if (held < 1) continue;
+                const int clusters = kRays * groups;
+                const int waves = (clusters + held - 1) / held;
+                const int at_once = (clusters + waves - 1) / waves * bands;
+                const int per_sm = (at_once + sm_count() - 1) / sm_count();
+                const PlaneLayout l = plane_var_layout(prec, prd, np, s.rows, nx, s.threads);
+                const int nodes = s.rows * nx;
+                const int passes = (l.ipad + s.threads - 1) / s.threads;
+                const double t =
+                    waves * (t0 + chain * passes * l.item_rows * ((np + l.chunks - 1) / l.chunks) +
+                             per_sm * nodes * (node + slot * np) * (per_sm > 1 ? shared : 1.0));
+                if (best.ng == 0 || t < best_t) {
+                    best = s;
+                    best_t = t;
+                }
+            }
+    }
+    return best;
 }
 
 // Grids the shifted-plane sweep's 32-bit node indices cover.
@@ -961,8 +1028,51 @@ int prd_prepare(mg3d_handle *h, int k) {
     return MG3D_OK;
 }
 
+// Launch arguments of the variants' shifted-plane sweep of level L with shape s.
+template <typename T>
+PlaneVarArgs<T> plane_var_args(const mg3d_handle *h, const Level &L, const SweepShape &s) {
+    PlaneVarArgs<T> a{};
+    const int nf = h->atom.n_freq;
+    a.nx = L.nx;
+    a.ny = L.ny;
+    a.nz = L.nz;
+    a.rows = s.rows;
+    a.bands = s.bands;
+    a.ngroups = s.ngroups;
+    a.np = s.np;
+    a.nslots = s.prd ? (nf + 1) / 2 : nf;
+    a.nf = nf;
+    a.up_mask = h->up_mask;
+    a.rmagic = band_magic(s.rows);
+    a.xmagic = band_magic(L.nx);
+    a.chi0 = (const T *)L.chi0;
+    a.S = (const T *)L.S;
+    a.bbot = (const T *)L.bbot;
+    a.steps = (const PlaneLerp<T> *)L.psteps;
+    if (s.prd) {
+        a.slots = (const PlaneSlot<T> *)h->d_pslot[0];   // one slot per group: a flat table
+        a.rhoS = (const T *)L.rhoS;
+        a.rho = (const T *)L.rho;
+        a.jnu = (T *)L.jnu_new;
+    } else {
+        a.uproj = (const T *)L.uproj;
+        a.vnorm = (const T *)L.vnorm;
+        a.xf = (const T *)h->d_vtab;
+        a.wq = (const T *)h->d_vtab + nf;
+    }
+    a.pj = (T *)h->pj;
+    a.pu = (T *)h->pu;
+    a.fx_tab = h->d_fx_tab;
+    return a;
+}
+
 // The sweep launch of level L with shape s (shifted-plane or band sweep).
 cudaError_t launch_level_sweep(const mg3d_handle *h, const Level &L, const SweepShape &s) {
+    if (s.plane == 3) {
+        if (h->prec == MG3D_PREC_F64)
+            return launch_plane_var_f64(plane_var_args<double>(h, L, s), s, h->stream);
+        return launch_plane_var_f32(plane_var_args<float>(h, L, s), s, h->stream);
+    }
     if (s.plane) {
         if (h->prec == MG3D_PREC_F64)
             return launch_plane_sweep_f64(plane_args<double>(h, L, s), s, h->stream);
@@ -1723,7 +1833,34 @@ int autotune_level(mg3d_handle *h, int k, int *evaluated) {
         }
     }
     L.shape = cands[best];
-    if (evaluated) *evaluated = (int)cands.size();
+    // the variants' shifted-plane sweep beside the band sweep
+    int extra = 0;
+    if ((h->moving || h->prd) && !h->params.sc_interp && plane_grid_ok(L.nx, L.ny, L.nz)) {
+        const int nslots = h->prd ? (nf + 1) / 2 : nf;
+        SweepShape best_var{};
+        float best_var_ms = 1e30f;
+        for (int groups = 1; groups <= 4 && groups <= nslots; ++groups)
+            for (int bands = 1; bands <= kMaxBands && bands <= L.ny; ++bands)
+                for (int th : {128, 256, 512}) {
+                    const int np = (nslots + groups - 1) / groups;
+                    const SweepShape s =
+                        var_shape(h->prec, L.nx, L.ny, nslots, h->prd ? 1 : 0, np, bands, th);
+                    if (s.ng == 0 || shape_capacity(h->prec, s, L.nx) < 1) continue;
+                    MG_TRY(ensure_partials(h, (size_t)kRays * s.ngroups * (size_t)L.nvox));
+                    float ms = 0.f;
+                    MG_TRY(time_shape(h, k, s, 2, &ms));
+                    ++extra;
+                    if (ms < best_var_ms) {
+                        best_var_ms = ms;
+                        best_var = s;
+                    }
+                }
+        if (best_var.ng && best_var_ms < best_ms) {
+            L.band_shape = L.shape;
+            L.shape = best_var;
+        }
+    }
+    if (evaluated) *evaluated = (int)cands.size() + extra;
     return MG3D_OK;
 }
 
@@ -1907,6 +2044,15 @@ int create_impl(const mg3d_atmosphere *atm, const mg3d_atom *atom, const mg3d_qu
             MG_TRY(dev_alloc(&L.dS, L.nvox * es));
         }
         if (L.shape.ng == 0) return fail(MG3D_E_ARG, "no sweep shape fits in shared memory");
+        if ((atm->vel || atom->gamma_prd > 0.0) && plane_grid_ok(L.nx, L.ny, L.nz)) {
+            const int prd = atom->gamma_prd > 0.0 ? 1 : 0;
+            const SweepShape v = choose_var_shape(
+                h->prec, L.nx, L.ny, prd ? (atom->n_freq + 1) / 2 : atom->n_freq, prd);
+            if (v.ng) {
+                L.band_shape = L.shape;
+                L.shape = v;
+            }
+        }
         h->partial_elems = std::max(h->partial_elems,
                                     (size_t)kRays * L.shape.ngroups * (size_t)L.nvox);
     }
@@ -2418,8 +2564,9 @@ int setup_ml_prd(mg3d_handle *h, const mg3d_ml_atom *atom) {
 // blocks of at most 256 threads per SM (its 128 registers and half the shared
 // memory), the fewest bands of at most 512 nodes and the most rays that fit.
 // Measured (32x32x65, 120 frequencies): 2 bands x 3 rays 7.2 ms, the other form
-// at its former default, 2 x 12, 17.6 ms.  False where no such shape fits.
-bool choose_ml_plane(Level &L) {
+// at its former default, 2 x 12, 17.6 ms; 8x8x9, 30 frequencies: 1 x 1 105 us, 1 x 12
+// 286 us a MALI sweep.  False where no such shape fits.
+bool choose_ml_plane(Level &L, int nf) {
     constexpr size_t kHalfSmem = 103 * 1024;
     if (!plane_grid_ok(L.nx, L.ny, L.nz)) return false;
     for (int b = 1; b <= kPortableBands && b <= L.ny; ++b) {
@@ -2430,6 +2577,8 @@ bool choose_ml_plane(Level &L) {
         if ((long)rows * L.nx > (long)ml_plane_max_pass(1) * th) continue;
         for (int rpb : {12, 6, 4, 3, 2, 1}) {
             if (ml_plane_smem_bytes(MG3D_PREC_F64, 1, rows, L.nx, rpb) > kHalfSmem) continue;
+            // fewer rays where there would be less than 700 blocks
+            if (rpb > 1 && 2L * (12 / rpb) * nf * b < 700) continue;
             L.ml_bands = b;
             L.ml_rows = rows;
             L.ml_rpb = rpb;
@@ -2618,14 +2767,17 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
         // shared memory, else the largest divisor of 12 that does; bands: the
         // fewest that fit and give >= 300 blocks, else the most that fit
         const bool plain = !atm->vel && !params->sc_interp;
-        if (plain && h->prec == MG3D_PREC_F64 && choose_ml_plane(L)) {
+        if (plain && h->prec == MG3D_PREC_F64 && choose_ml_plane(L, nf)) {
             h->ml_slots = std::max(h->ml_slots, 2 * (12 / L.ml_rpb));
             continue;
         }
         int pick = 0;
         // static linear sweeps: four blocks of 256 threads per SM where at least
-        // three rays leave room for them (FP32 64x64x129, 120 frequencies: 8
-        // bands x 12 rays 7.6 ms, the fewest bands that fit, 3 x 12, 15.6 ms)
+        // three rays leave room for them, one node per thread where 8 bands
+        // allow it, and fewer rays per block where there would be less than
+        // 200 blocks (FP32 64x64x129, 120 frequencies: 8 bands x 12 rays 7.6 ms,
+        // the fewest bands that fit, 3 x 12, 15.6 ms; 20x18x21, 30 frequencies: 1 x 3
+        // 108 us, 1 x 12 167 us a MALI sweep)
         for (int pass = plain ? 0 : 1; pass < 2 && !pick; ++pass)
             for (int rpb : {12, 6, 4, 3, 2, 1}) {
                 if (pass == 0 && rpb < 3) break;
@@ -2637,7 +2789,13 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
                         (pass == 0 ? kMlQuarterSmem : kMaxSweepSmem))
                         continue;
                     pick = b;
-                    if (pass == 0 || 2L * (12 / rpb) * nf * b >= 300) break;
+                    if (pass == 0 ? (long)rows * L.nx <= 256
+                                  : 2L * (12 / rpb) * nf * b >= 300)
+                        break;
+                }
+                if (pass == 0 && rpb > 3 && 2L * (12 / rpb) * nf * pick < 200) {
+                    pick = 0;
+                    continue;
                 }
                 if (pick) {
                     L.ml_rpb = rpb;
@@ -3754,12 +3912,14 @@ int mg3d_get_fs_config(const mg3d_handle *h, int level, int *freq_per_block, int
                        int *threads, int *lean, int *stage) {
     MG_TRY(check_level(h, level));
     const Level &L = h->lev[level];
-    if (freq_per_block)
-        *freq_per_block = L.shape.plane && L.shape.ngroups == 1 ? h->atom.n_freq : L.shape.ng;
-    if (bands) *bands = L.shape.bands;
-    if (threads) *threads = L.shape.threads;
-    if (lean) *lean = L.shape.lean;
-    if (stage) *stage = L.shape.plane ? 1 + L.shape.plane : L.shape.stage;
+    // the variants' own form is not a shape that can be set: their band sweep's is
+    // reported, which setting it would select
+    const SweepShape &s = L.shape.plane == 3 ? L.band_shape : L.shape;
+    if (freq_per_block) *freq_per_block = s.plane && s.ngroups == 1 ? h->atom.n_freq : s.ng;
+    if (bands) *bands = s.bands;
+    if (threads) *threads = s.threads;
+    if (lean) *lean = s.lean;
+    if (stage) *stage = s.plane ? 1 + s.plane : s.stage;
     return MG3D_OK;
 }
 

@@ -41,8 +41,9 @@ struct SweepShape {
     int vel = 0;   // 1: moving atmosphere, ray-dependent profiles (unstaged)
     int prd = 0;   // 1: partial redistribution, frequency-dependent S (unstaged)
     int plane = 0; // shifted-plane sweep (plane_sweep.cuh) with np slots of two
-                   // frequencies: 1 cluster barriers, 2 transaction-counted stores
-    int np = 0;    //    frequencies per group (ng = 2 np table positions per group)
+                   // frequencies: 1 cluster barriers, 2 transaction-counted stores;
+                   // 3: the variants' form (plane_var.cuh)
+    int np = 0;    //    slots per group (forms 1 and 2: ng = 2 np table positions)
 };
 
 // Per (ray, step t) constants of the shifted-plane sweeps (plane_sweep.cuh,
@@ -134,6 +135,31 @@ cudaError_t launch_plane_sweep_f64(const PlaneArgs<double> &a, const SweepShape 
                                    cudaStream_t st);
 cudaError_t launch_plane_sweep_f32(const PlaneArgs<float> &a, const SweepShape &s,
                                    cudaStream_t st);
+// The variants' shifted-plane sweep (plane_var.cuh), SweepShape::plane 3: np slots
+// per group; prd (else moving).
+template <typename T>
+struct PlaneVarArgs {
+    int nx, ny, nz, rows, bands, ngroups, np;
+    int nslots, nf;                      // slots of all groups; frequencies
+    int ahead, chunks, ipad;             // of the launch's PlaneLayout (set by the launch)
+    unsigned up_mask;
+    unsigned long long rmagic, xmagic;   // band_magic(rows), band_magic(nx)
+    const T *chi0, *S, *bbot;            // [nvox], [nvox], [nx*ny]
+    const PlaneLerp<T> *steps;           // [kRays][nz]
+    const PlaneSlot<T> *slots;           // PRD: [nslots]
+    const T *rhoS, *rho;                 // PRD: [nf][nvox]
+    T *jnu;                              // PRD: [kRays][nf][nvox] w_r I
+    const T *uproj, *vnorm;              // moving: [kRays][nvox]
+    const T *xf, *wq;                    // moving: [nf]
+    T *pj, *pu;                          // [kRays*ngroups][nvox] partial Jeff and U
+    const unsigned long long *fx_tab;
+};
+PlaneLayout plane_var_layout(int prec, int prd, int np, int rows, int nx, int threads);
+cudaError_t launch_plane_var_f64(const PlaneVarArgs<double> &a, const SweepShape &s,
+                                 cudaStream_t st);
+cudaError_t launch_plane_var_f32(const PlaneVarArgs<float> &a, const SweepShape &s,
+                                 cudaStream_t st);
+cudaError_t plane_var_clusters(int prec, const SweepShape &s, int nx, int *n);
 cudaError_t launch_plane_async_f64(const PlaneArgs<double> &a, const SweepShape &s,
                                    cudaStream_t st);
 cudaError_t launch_plane_async_f32(const PlaneArgs<float> &a, const SweepShape &s,

@@ -6,7 +6,7 @@ namespace mg3d {
 
 size_t ml_plane_smem_bytes(int prec, int nf, int rows, int nx, int rpb) {
     const int nv = prec == MG3D_PREC_F64 ? mlplane::vectors<double>(nf) : mlplane::vectors<float>(nf);
-    return 2ull * rpb * ((rows + 1) * nx * nv * 16ull + rows * sizeof(mlplane::RowDest));
+    return 2ull * rpb * ((rows + 1) * nx * nv * 16ull + rows * sizeof(plane::RowDest));
 }
 
 cudaError_t launch_ml_plane_f64(const MlPlaneArgs<double> &a, int nf_block, int threads,

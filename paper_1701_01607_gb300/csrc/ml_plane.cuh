@@ -38,13 +38,6 @@ namespace mg3d {
 
 namespace mlplane {
 
-// where a row of the band is stored: in the block that owns it, and in the halo
-// row of the block before (or kNoHalo)
-struct RowDest {
-    unsigned base, halo;
-};
-constexpr unsigned kNoHalo = ~0u;
-
 // 16-byte vectors per node: I, chi, S of nf frequencies
 template <typename T>
 __host__ __device__ constexpr int vectors(int nf) {
@@ -56,8 +49,6 @@ __host__ __device__ constexpr int vectors(int nf) {
 template <typename T, int NF>
 __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
     using namespace plane;
-    using mlplane::kNoHalo;
-    using mlplane::RowDest;
     constexpr bool F64 = sizeof(T) == 8;
     constexpr int VW = vec_width<T>();
     constexpr int NV = mlplane::vectors<T>(NF);

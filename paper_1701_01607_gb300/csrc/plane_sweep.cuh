@@ -97,6 +97,13 @@ __host__ __device__ constexpr int vectors() {
     return (NP + 2 + vec_width<T>() - 1) / vec_width<T>();
 }
 
+// where a row of the band is stored: in the block that owns it, and in the halo
+// row of the block before (or kNoHalo)
+struct RowDest {
+    unsigned base, halo;
+};
+constexpr unsigned kNoHalo = ~0u;
+
 __device__ __forceinline__ unsigned smem_addr(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
