@@ -15,13 +15,13 @@
 // One thread-block cluster per (ray, group of frequencies): the cluster's
 // blocks split the stored frame in bands of rows.  A block owns rows
 // [rank*rows, rank*rows + myrows) of the frame, plus one halo row (the first
-// row of the next band, or row 0 after the last band) and one pad column
-// (a copy of column 0), so all four corners of its nodes are in its own
-// shared memory.  Writes carry the shift instead: a node's values go to the
-// block that owns its stored row (distributed shared memory, st.shared::cluster)
-// and, for the first row of a band or column 0, also to the halo row or pad
-// column that duplicates it.  Two planes are kept (read k-1, write k); one
-// cluster barrier per plane orders the writes of a step before the reads of
+// row of the next band, or row 0 after the last band), so all four corners of
+// its nodes are in its own shared memory (column nx is column 0).  Writes carry
+// the shift instead: a node's values go to the block that owns its stored row
+// (distributed shared memory, st.shared::cluster) and, for the first row of a
+// band, also to the halo row that duplicates it; the addresses are tabulated
+// a row and step.  Two planes are kept (read k-1, write k); one cluster barrier
+// per plane orders the writes of a step before the reads of
 // the next and the reads of a step before the overwrite two steps later.
 //
 // A second completion scheme (stage 3) replaces the barrier's release fence
@@ -103,6 +103,11 @@ struct RowDest {
     unsigned base, halo;
 };
 constexpr unsigned kNoHalo = ~0u;
+// the same with the mbarriers of the async scheme (kNoBar: a row of this block)
+constexpr unsigned kNoBar = ~0u;
+struct __align__(16) RowTarget {
+    unsigned base, halo, bar, hbar;
+};
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
@@ -357,7 +362,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     const int y0 = rank * rows;
     const int myrows = min(rows, ny - y0);
     const int lastrows = ny - (nb - 1) * rows;   // rows of the last band
-    const unsigned pitch = (unsigned)(nx + 1) * 16;      // one stored row of a vector, bytes
+    const unsigned pitch = (unsigned)nx * 16;            // one stored row of a vector, bytes
     const unsigned vs = (unsigned)(rows + 1) * pitch;    // one vector of a frame
     const unsigned frame = NV * vs;                      // one stored frame
     const int nplane = nx * ny;                  // the host keeps nvox below 2^31
@@ -369,8 +374,13 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned buf_addr = smem_addr(smem_raw);
+    RowTarget *dest = reinterpret_cast<RowTarget *>(smem_raw + 2 * (size_t)frame);   // [2][rows]
     // chi0 and S of the band's nodes two steps ahead: [3][2][rows * nx]
-    T *ahead = reinterpret_cast<T *>(smem_raw + 2 * (size_t)frame);
+    T *ahead = reinterpret_cast<T *>(smem_raw + 2 * (size_t)frame + 2 * rows * sizeof(RowTarget));
+    // 16-byte copies: every band of every plane starts on such a boundary
+    constexpr int CW = 16 / (int)sizeof(T);
+    const bool wide = nplane % CW == 0 && (rows * nx) % CW == 0 &&
+                      ((reinterpret_cast<size_t>(a.chi0) | reinterpret_cast<size_t>(a.S)) & 15) == 0;
     __shared__ fx::u64 fx_tab[F64 ? 2 * fx::kTab : 1];   // tables of the integer weights
     __shared__ PlaneSlot<T> stab[NP];
     // step constants two steps ahead
@@ -445,56 +455,51 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
         }
     };
 
-    // Where a node (x, yl) of the band goes in the frame of the next step,
-    // shifted by (sx, sy), in buffer `par`.  A node of column 0 also fills the
-    // pad column, a node of a band's first row also the halo row of the band
-    // before it; few nodes are either, so the copies are behind one branch.
-    struct Dest {
-        unsigned base;     // of vector 0 in the block that owns the row
-        int ob, lr, xs;    // that block, the row in its band, the column
+    // Where the band's rows go in the frame stored at step t, whose reader's row
+    // shift is sy: one entry a row and step, instead of the modulo, band and
+    // peer arithmetic at every node.
+    auto fill_dest = [&](int t, int sy) {
+        const unsigned par = t & 1;
+        for (int yl = threadIdx.x; yl < myrows; yl += nth) {
+            int ys = y0 + yl - sy;
+            ys += ys < 0 ? ny : 0;
+            const int ob = cl ? band_of(ys, a.rmagic) : 0;
+            const int lr = ys - ob * rows;
+            const int hb = ob == 0 ? nb - 1 : ob - 1;   // the band whose halo row is ys
+            RowTarget d;
+            d.base = cluster_addr(buf_addr, (unsigned)ob) + par * frame + (unsigned)lr * pitch;
+            d.halo = lr != 0 ? kNoHalo
+                             : cluster_addr(buf_addr, (unsigned)hb) + par * frame +
+                                   (unsigned)(hb == nb - 1 ? lastrows : rows) * pitch;
+            d.bar = as && ob != rank ? cluster_addr(bar_addr + 8u * par, (unsigned)ob) : kNoBar;
+            d.hbar = as && hb != rank ? cluster_addr(bar_addr + 8u * par, (unsigned)hb) : kNoBar;
+            dest[par * rows + yl] = d;
+        }
     };
-    const unsigned padoff = (unsigned)nx * 16;
-    auto dest_of = [&](int x, int yl, int sx, int sy, int par) {
-        Dest d;
-        d.xs = x - sx;
-        d.xs += d.xs < 0 ? nx : 0;
-        int ys = y0 + yl - sy;
-        ys += ys < 0 ? ny : 0;
-        d.ob = band_of(ys, a.rmagic);
-        d.lr = ys - d.ob * rows;
-        d.base = cluster_addr(buf_addr, (unsigned)d.ob) + par * frame + (unsigned)d.lr * pitch +
-                 (unsigned)d.xs * 16;
-        return d;
+    auto shifted = [&](int x, int sx) {   // byte offset of the stored column
+        const int xs = x - sx;
+        return (unsigned)(xs < 0 ? xs + nx : xs) * 16u;
     };
-    // one copy of vectors v0 .. v0+N-1 at byte offset `off` of block `ob`
-    auto store_to = [&](auto n_tag, unsigned addr, int ob, int par, int v0, const T *cv) {
+    // vectors v0 .. v0+N-1 of the node's channels; to another block in the async
+    // scheme: st.async counted on that block's mbarrier of the buffer
+    auto put = [&](auto n_tag, const RowTarget &d, unsigned xs, int v0, const T *cv) {
         constexpr int N = decltype(n_tag)::value;
-        if constexpr (AS) {
-            // to another block: st.async counted on that block's mbarrier of
-            // the buffer; within the block: plain stores
-            if (as && ob != rank) {
-                const unsigned bar = cluster_addr(bar_addr + 8u * par, (unsigned)ob);
+        if (AS && d.bar != kNoBar) {
+#pragma unroll
+            for (int v = 0; v < N; ++v)
+                st16_async_if(true, d.base + xs + (v0 + v) * vs, cv + v * VW, d.bar);
+        } else {
+#pragma unroll
+            for (int v = 0; v < N; ++v) st16(d.base + xs + (v0 + v) * vs, cv + v * VW);
+        }
+        if (d.halo != kNoHalo) {
+            if (AS && d.hbar != kNoBar) {
 #pragma unroll
                 for (int v = 0; v < N; ++v)
-                    st16_async_if(true, addr + (v0 + v) * vs, cv + v * VW, bar);
-                return;
-            }
-        }
+                    st16_async_if(true, d.halo + xs + (v0 + v) * vs, cv + v * VW, d.hbar);
+            } else {
 #pragma unroll
-        for (int v = 0; v < N; ++v) st16(addr + (v0 + v) * vs, cv + v * VW);
-    };
-    // vectors v0 .. v0+N-1 of the node's channels, with the copies
-    auto put = [&](auto n_tag, const Dest &d, int par, int v0, const T *cv) {
-        store_to(n_tag, d.base, d.ob, par, v0, cv);
-        if (d.xs == 0 || d.lr == 0) {
-            if (d.xs == 0) store_to(n_tag, d.base + padoff, d.ob, par, v0, cv);
-            if (d.lr == 0) {
-                const int hb = d.ob == 0 ? nb - 1 : d.ob - 1;   // the band before
-                const unsigned h = cluster_addr(buf_addr, (unsigned)hb) + par * frame +
-                                   (unsigned)(hb == nb - 1 ? lastrows : rows) * pitch +
-                                   (unsigned)d.xs * 16;
-                store_to(n_tag, h, hb, par, v0, cv);
-                if (d.xs == 0) store_to(n_tag, h + padoff, hb, par, v0, cv);
+                for (int v = 0; v < N; ++v) st16(d.halo + xs + (v0 + v) * vs, cv + v * VW);
             }
         }
     };
@@ -512,9 +517,16 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
         if (a.ahead) {
             const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
             T *dst = ahead + part * 2 * rows * nx;
-            for (int o = threadIdx.x; o < myrows * nx; o += nth) {
-                cp_async(dst + o, a.chi0 + kp + o);
-                cp_async(dst + rows * nx + o, a.S + kp + o);
+            if (wide) {
+                for (int o = CW * threadIdx.x; o < myrows * nx; o += CW * nth) {
+                    cp_async16(dst + o, a.chi0 + kp + o);
+                    cp_async16(dst + rows * nx + o, a.S + kp + o);
+                }
+            } else {
+                for (int o = threadIdx.x; o < myrows * nx; o += nth) {
+                    cp_async(dst + o, a.chi0 + kp + o);
+                    cp_async(dst + rows * nx + o, a.S + kp + o);
+                }
             }
         }
         cp_async_commit();
@@ -536,7 +548,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     // blocks when the plane is stored with row shift sy.  Stored row ys (a
     // row of the band, or the halo row: the next band's first row, row 0
     // after the last band) holds source row (ys + sy) mod ny, all of its nx
-    // nodes and the pad copy, written by the block that owns that row.  Warp
+    // nodes, written by the block that owns that row.  Warp
     // 0 counts the rows with another owner; its lane 0 posts the phase's one
     // arrival with the byte count.
     auto expect_fill = [&](int sy, int par) {
@@ -550,7 +562,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
         }
         cnt = __reduce_add_sync(0xffffffffu, cnt);
         if (threadIdx.x == 0)
-            mbar_arrive_expect(bar_addr + 8u * par, (unsigned)(cnt * (nx + 1) * NV * 16));
+            mbar_arrive_expect(bar_addr + 8u * par, (unsigned)(cnt * nx * NV * 16));
     };
     bool waits_ok = true;   // false once a bounded wait ran out
     auto wait_fill = [&](int s) {   // buffer s & 1 holds the plane stored at step s
@@ -569,6 +581,8 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     // temperature, top: zero), so w0 = 0 and 1 - w0 = 1
     if (nz > 1) prefetch(1, 1);
     if (nz > 2) prefetch(2, 2);
+    if (nz > 1) fill_dest(0, a.steps[(long)r * nz].sy);
+    __syncthreads();
     {
         const int k0 = (up ? 0 : nz - 1) * nplane + y0 * nx;
         const PlaneLerp<T> sp = a.steps[(long)r * nz];
@@ -581,13 +595,12 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                 pj[k0 + o] = Ib * wsum;
                 pu[k0 + o] = wsum;
                 if (nz > 1) {
-                    const Dest d = dest_of(x, yl0 + j, sp.sx, sp.sy, 0);
                     T cv[NV * VW];
 #pragma unroll
                     for (int e = 0; e < NV * VW; ++e) cv[e] = Ib;
                     cv[0] = a.chi0[k0 + o];
                     cv[1] = a.S[k0 + o];
-                    put(All{}, d, 0, 0, cv);
+                    put(All{}, dest[yl0 + j], shifted(x, sp.sx), 0, cv);
                 }
             }
         }
@@ -597,13 +610,20 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     else __syncthreads();
 
     int part = 1;   // t mod 3
+    if (nz > 2) {
+        fill_dest(1, step_ring[1].sy);
+        __syncthreads();
+    }
     for (int t = 1; t < nz; ++t) {
         const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
         const unsigned char *prev = smem_raw + ((t - 1) & 1) * (size_t)frame;
         const PlaneLerp<T> sp = step_ring[t & 3];
         const bool write = t + 1 < nz;
         // part (t + 2) mod 3 was last read at step t - 1
-        if (t + 2 < nz) prefetch(t + 2, part == 0 ? 2 : part - 1);
+        if (t + 2 < nz) {
+            prefetch(t + 2, part == 0 ? 2 : part - 1);
+            fill_dest(t + 1, step_ring[(t + 1) & 3].sy);
+        }
         if (chunks > 1 && t > 1) flush_sums(t - 1);
         if (as) {
             // the other blocks' part of the plane stored at step t - 1
@@ -615,7 +635,6 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
             }
         }
         // the nearer column and row first: H = A + rx B, V = H + ry H'
-        const unsigned near_x = (sp.near & 1) ? 16u : 0u, far_x = 16u - near_x;
         bool down = false;   // FP64: the nearer row is the higher one
         fx::u64 cm = 0;      // FP64: c = (cm, ce)
         int ce = 0;
@@ -632,7 +651,10 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
             // rows in the order they are needed: node j of the item lies
             // between row j (nearer) and row j + 1 of the walk
             const unsigned char *row0 =
-                prev + (unsigned)(down ? yl0 + nr : yl0) * pitch + (unsigned)x * 16;
+                prev + (unsigned)(down ? yl0 + nr : yl0) * pitch;
+            const unsigned xb = (unsigned)x * 16, xb1 = x + 1 == nx ? 0u : xb + 16;
+            const unsigned near_x = (sp.near & 1) ? xb1 : xb, far_x = (sp.near & 1) ? xb : xb1;
+            const unsigned xs = shifted(x, sp.sx);
             const int dpitch = down ? -(int)pitch : (int)pitch;
             auto row_h = [&](int v, int k, T *h) {
                 const unsigned char *p = row0 + k * dpitch + v * vs;
@@ -696,7 +718,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                     if (write) {
                         ch[0] = chi_loc;
                         ch[1] = S_loc;
-                        put(All{}, dest_of(x, yl, sp.sx, sp.sy, t & 1), t & 1, 0, ch);
+                        put(All{}, dest[(t & 1) * rows + yl], xs, 0, ch);
                     }
                 }
             } else {
@@ -724,7 +746,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
             fx::u64 dm[R], dr[R], ud[R];
             int de[R];
             bool dok[R];
-            Dest dst[R];
+            RowTarget dst[R];
 #pragma unroll
             for (int j = 0; j < R; ++j) {
                 if (j < nr) {
@@ -737,7 +759,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                     dr[j] = fx::recip(dm[j]);
                     ud[j] = 0;
                     cj[j] = cu[j] = T(0);
-                    if (write) dst[j] = dest_of(x, yl, sp.sx, sp.sy, t & 1);
+                    if (write) dst[j] = dest[(t & 1) * rows + yl];
                 }
             }
             // slot p's new intensity at node j from the upwind sum i (without c)
@@ -775,7 +797,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                 if (j < nr && chunk == 0) {
                     V0[j][0] = chi_loc[j];
                     V0[j][1] = S_loc[j];
-                    if (write) put(One{}, dst[j], t & 1, 0, V0[j]);
+                    if (write) put(One{}, dst[j], xs, 0, V0[j]);
                 }
 #pragma unroll 1
             for (int v = v_begin; v < v_end; ++v) {
@@ -789,7 +811,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                             const int p = v * VW + e - 2;
                             V[j][e] = p < nslot ? step(j, p, V[j][e]) : T(0);
                         }
-                        if (write) put(One{}, dst[j], t & 1, v, V[j]);
+                        if (write) put(One{}, dst[j], xs, v, V[j]);
                     }
             }
 #pragma unroll

@@ -23,7 +23,7 @@ PlaneLayout plane_layout(int prec, int np, int rows, int nx, int threads) {
     l.item_rows = (long)rows * nx > threads ? 2 : 1;
     l.ipad = ((rows + l.item_rows - 1) / l.item_rows * nx + 31) / 32 * 32;
     l.chunks = prec == 0 ? std::max(1, std::min(threads / l.ipad, nv - 1)) : 1;
-    l.smem = 2ull * nv * (rows + 1) * (nx + 1) * 16;
+    l.smem = 2ull * nv * (rows + 1) * nx * 16 + 2ull * rows * sizeof(plane::RowTarget);
     const size_t next = 6ull * rows * nx * es, sums = 4ull * l.chunks * rows * nx * es;
     if (l.chunks > 1) {
         if (l.smem + sums <= plane_smem_max(prec == 0)) l.smem += sums;
