@@ -78,7 +78,9 @@ __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned buf_addr = smem_addr(smem_raw);
     __shared__ fx::u64 fx_tab[F64 ? 2 * fx::kTab : 1];   // tables of the integer weights
-    // the rays' constants of step t in [t & 3], two steps ahead
+    // the rays' constants of step t in [t & 3], three steps ahead: the row
+    // table of step t + 1 is made during step t, when all copies but the latest
+    // group have landed
     __shared__ __align__(16) PlaneLerp<T> sstep[4][12];
     // where the band's rows go at the end of step t: [t & 1][ray][row]
     RowDest *dest = reinterpret_cast<RowDest *>(smem_raw + 2 * (size_t)frame);
@@ -97,6 +99,7 @@ __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
     fetch_steps(0);
     if (nz > 1) fetch_steps(1);
     if (nz > 2) fetch_steps(2);
+    if (nz > 3) fetch_steps(3);
     cp_async_wait();
     __syncthreads();
     const T wray = T(1.0 / kRays);
@@ -217,10 +220,8 @@ __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
         const long kp = (long)(up ? t : nz - 1 - t) * nplane;
         const unsigned prev = buf_addr + ((t - 1) & 1) * frame;
         const bool write = t + 1 < nz;
-        if (t + 2 < nz) {
-            fetch_steps(t + 2);
-            fill_dest(t + 1);
-        }
+        if (t + 3 < nz) fetch_steps(t + 3);
+        if (t + 2 < nz) fill_dest(t + 1);
         const RowDest *dst = dest + (t & 1) * rpb * rows;
         // angle sums of the first item, stored after the barrier's first half
         T kj[R][NF], ku[R][NF], km[R][NF];
@@ -368,8 +369,8 @@ __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
                 }
             }
         }
-        // the constants of step t + 1 are there before the barrier
-        if (t + 2 < nz) cp_async_wait_but_last();
+        // the constants of step t + 2 are there before the barrier
+        if (t + 3 < nz) cp_async_wait_but_last();
         else cp_async_wait();
         if (write) {
             if (cl) cluster_arrive();

@@ -72,7 +72,7 @@
 // (ray, group); the rate kernel adds the slots in a fixed order.
 //
 // chi0 and S of the block's own nodes on the next plane are copied to shared
-// memory two steps ahead (cp.async), with the step's constants, so their latency
+// memory two steps ahead (cp.async), the step's constants three, so their latency
 // overlaps the steps before; where the shape
 // leaves no room for that they are read from global memory where used.
 #pragma once
@@ -383,7 +383,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
                       ((reinterpret_cast<size_t>(a.chi0) | reinterpret_cast<size_t>(a.S)) & 15) == 0;
     __shared__ fx::u64 fx_tab[F64 ? 2 * fx::kTab : 1];   // tables of the integer weights
     __shared__ PlaneSlot<T> stab[NP];
-    // step constants two steps ahead
+    // step constants up to three steps ahead
     __shared__ __align__(16) PlaneLerp<T> step_ring[4];
     // async scheme: one mbarrier per plane buffer, one phase per filling
     __shared__ __align__(8) unsigned long long full_bar[2];
@@ -503,17 +503,22 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
             }
         }
     };
-    using One = std::integral_constant<int, 1>;
-    using All = std::integral_constant<int, NV>;
-
-    // chi0 and S of step t's plane into part t mod 3 of the ring, and the
-    // constants of step t
-    auto prefetch = [&](int t, int part) {
+    // The constants of step t, three steps ahead: the row table of step t + 1 is
+    // made during step t, when all copies but the latest group have landed.
+    auto fetch_step = [&](int t) {
         constexpr int NC = sizeof(PlaneLerp<T>) / 16;
         if (threadIdx.x < NC)
             cp_async16(reinterpret_cast<unsigned char *>(&step_ring[t & 3]) + 16 * threadIdx.x,
                        reinterpret_cast<const unsigned char *>(&a.steps[(long)r * nz + t]) +
                            16 * threadIdx.x);
+    };
+    using One = std::integral_constant<int, 1>;
+    using All = std::integral_constant<int, NV>;
+
+    // chi0 and S of step t's plane into part t mod 3 of the ring, and the
+    // constants of step t + 1
+    auto prefetch = [&](int t, int part) {
+        if (t + 1 < nz) fetch_step(t + 1);
         if (a.ahead) {
             const int kp = (up ? t : nz - 1 - t) * nplane + y0 * nx;
             T *dst = ahead + part * 2 * rows * nx;
@@ -579,7 +584,10 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
 
     // ---- entering boundary plane: I prescribed (bottom: Planck at the local
     // temperature, top: zero), so w0 = 0 and 1 - w0 = 1
-    if (nz > 1) prefetch(1, 1);
+    if (nz > 1) {
+        fetch_step(1);
+        prefetch(1, 1);
+    }
     if (nz > 2) prefetch(2, 2);
     if (nz > 1) fill_dest(0, a.steps[(long)r * nz].sy);
     __syncthreads();

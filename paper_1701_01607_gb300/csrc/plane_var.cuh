@@ -110,12 +110,17 @@ __device__ __forceinline__ void plane_var_body(const PlaneVarArgs<T> &a) {
         return i == 0 ? a.chi0
                       : i == 1 ? a.S : (i == 2 ? a.uproj : a.vnorm) + (long)r * nvox;
     };
-    auto prefetch = [&](int t, int part) {
+    // The constants of step t, three steps ahead: the row table of step t + 1 is
+    // made during step t, when all copies but the latest group have landed.
+    auto fetch_step = [&](int t) {
         constexpr int NC = sizeof(PlaneLerp<T>) / 16;
         if (threadIdx.x < NC)
             cp_async16(reinterpret_cast<unsigned char *>(&step_ring[t & 3]) + 16 * threadIdx.x,
                        reinterpret_cast<const unsigned char *>(&a.steps[(long)r * nz + t]) +
                            16 * threadIdx.x);
+    };
+    auto prefetch = [&](int t, int part) {
+        if (t + 1 < nz) fetch_step(t + 1);
         if (a.ahead) {
             const int kp = plane_of(t);
             T *dst = ahead + part * NA * rows * nx;
@@ -170,7 +175,10 @@ __device__ __forceinline__ void plane_var_body(const PlaneVarArgs<T> &a) {
     };
 
     // ---- entering boundary plane: I prescribed, w0 = 0
-    if (nz > 1) prefetch(1, 1);
+    if (nz > 1) {
+        fetch_step(1);
+        prefetch(1, 1);
+    }
     if (nz > 2) prefetch(2, 2);
     __syncthreads();   // fx_tab
     if (nz > 1) fill_dest(0, a.steps[(long)r * nz].sy);
