@@ -41,25 +41,24 @@ N_GRIDS = 3
 METRIC = "FS Gvoxel*ray*freq/s (3-grid FAS V-cycle step)"
 UNIT = "Gunit/s"
 FS_UNITS_PER_FINE = GRID[0] * GRID[1] * GRID[2] * 24 * 9
-# FP64 floating-point operations per (node, ray, frequency) of the sweep
-# (bilinear I_up 7, new I 5, two accumulations 4, plus 16 per node and ray
-# shared by the 9 frequencies for the chi/S interpolation and dtau), and the
-# short-characteristics weights (optical path 1, exp 1, u 2, w0 1, w_up 1)
-# once per distinct profile value: phi(x) = phi(-x) gives mirror frequencies
-# the same optical depth, so 5 of the 9 need their own.  exp and the
-# division count as one operation each.
-N_DISTINCT_PHI = (9 + 1) // 2
-ALG_FLOPS_PER_UNIT = 7 + 5 + 4 + (1 + 1 + 2 + 1 + 1) * N_DISTINCT_PHI / 9.0 + 16.0 / 9.0
+# FP64 floating-point operations per (node, ray, frequency) of the sweep.
+# phi(x) = phi(-x) and S does not depend on frequency, so the intensities of a
+# mirror pair are the same and are solved once: 5 of the 9 frequencies.  Per
+# solved frequency bilinear I_up 7, new I 5, two accumulations 4 and the
+# short-characteristics weights (optical path 1, exp 1, u 2, w0 1, w_up 1), plus
+# 16 per node and ray for the chi/S interpolation and dtau.  exp and the
+# division count as one operation each; the FP64 sweep forms the weights in
+# integer arithmetic, so not all of these run on the FP64 pipe.
+N_SOLVED = (9 + 1) // 2
+ALG_FLOPS_PER_UNIT = (7 + 5 + 4 + (1 + 1 + 2 + 1 + 1)) * N_SOLVED / 9.0 + 16.0 / 9.0
 FP64_NOMINAL_TFLOPS = 1.25      # GB300, at the 2070 MHz maximum SM clock
 # FP32 instructions per unit the FP32 sweep needs (each an FMA-pipe
-# instruction): per frequency the bilinear I_up 4, the new I 2 (one of them
-# the w_up S_up term shared by a mirror pair is counted per distinct phi
-# below), the Jeff sum 1; per distinct phi (5 of 9) the optical path 1, the
-# exp2 argument 1, u 1, w0 1, w_up 1, w_up S_up 1, the U sum 1; per node and
-# ray the chi0/S bilinear 8 and dtau 2.  Plus per distinct phi one ex2 and one
-# rcp on the multi-function unit.
-ALG_FP32_OPS_PER_UNIT = 4 + 2 + 1 + 7 * N_DISTINCT_PHI / 9.0 + 10.0 / 9.0
-MUFU_EX2_PER_UNIT = MUFU_RCP_PER_UNIT = N_DISTINCT_PHI / 9.0
+# instruction): per solved frequency the bilinear I_up 4, the new I 2, the Jeff
+# sum 1, the optical path 1, the exp2 argument 1, u 1, w0 1, w_up 1, w_up S_up 1
+# and the U sum 1; per node and ray the chi0/S bilinear 8 and dtau 2.  Plus per
+# solved frequency one ex2 and one rcp on the multi-function unit.
+ALG_FP32_OPS_PER_UNIT = (4 + 2 + 1 + 7) * N_SOLVED / 9.0 + 10.0 / 9.0
+MUFU_EX2_PER_UNIT = MUFU_RCP_PER_UNIT = N_SOLVED / 9.0
 # DRAM bytes (read + write) of one finest-grid FP64 sweep launch on the bench
 # atmosphere per launch shape (ng, bands, threads, lean, stage), from ncu
 # captures of the current kernel; a shape the autotuner picks that is not
@@ -277,6 +276,8 @@ def run_gpu(args):
             "dtype": "f64", "data": "synthetic",
             "config": {"workload": WORKLOAD, "grid": list(GRID), "n_grids": N_GRIDS,
                        "n_freq": 9, "rays": 24, **NU, "fs_precision": "f64",
+                       "frequencies": "9 counted; the 4 mirror pairs x, -x have the same "
+                                      "intensity and are solved once",
                        "parallelism": f"replicas x{world}",
                        "l2": "256 MB buffer written between timed steps",
                        "sweep_autotune": tuning},
@@ -593,9 +594,8 @@ def batch_members(n=32, seed0=100, ml_chunk=100):
 
 
 def run_batch(args):
-    """Batched V-cycles of the 32-atmosphere batch (opt-in, --batch): one
-    batched sweep launch per atom kind (per frequency chunk for the 6-level
-    members), V-cycles replayed from CUDA graphs.  Prints one JSON line."""
+    """Batched V-cycles of the 32-atmosphere batch (opt-in, --batch):
+    every member's V-cycle graph replayed on its own stream.  Prints one JSON line."""
     import torch
 
     from paper_1701_01607_gb300 import mg3d as m

@@ -501,7 +501,8 @@ int mg3d_get_ml_shape_ex(const mg3d_handle *h, int level, int *bands, int *rays_
  * the members run alone.  Members must share
  * n_grids, the formal-solution precision and the multigrid schedule; creating
  * the batch moves them onto streams of the batch, so they should not be used
- * from elsewhere while the batch exists.  The batch does not own its members. */
+ * from elsewhere while the batch exists.  The batch does not own its members.
+ * No counterpart in the paper. */
 typedef struct mg3d_batch mg3d_batch;
 int mg3d_batch_create(int n, mg3d_handle *const *members, mg3d_batch **out);
 int mg3d_batch_destroy(mg3d_batch *b);
@@ -554,6 +555,10 @@ int mg3d_prolong(mg3d_handle *h, int level_fine, int ncomp, const double *coarse
  *         return MG3D_E_CUDA).
  * The library picks a shape at creation (the shifted-plane sweep with
  * cluster barriers where it applies, at most 8 bands); this overrides it.
+ * Moving atmospheres and partial redistribution with the linear upwind
+ * interpolation start on a shifted-plane sweep of their own, whose shape
+ * mg3d_get_fs_config reports as that of the band sweep it stands for
+ * (stage 0) and this call replaces by the band sweep.
  * Returns MG3D_E_ARG if the shape does not fit in shared memory or the GPU
  * cannot hold one of its clusters.
  * No counterpart in the paper (launch control). */
@@ -585,7 +590,8 @@ int mg3d_get_fs_occupancy(mg3d_handle *h, int level, int freq_per_block, int ban
  * to 8 groups, 1-16 bands, 32-1024 threads in powers of two and the block
  * sizes that cover a band in equal passes, both register budgets in FP32 and
  * both completion schemes (stages 2 and 3) with more than one band; other
- * two-level handles (band sweep): every number of frequency groups up to 64, 1-16 bands,
+ * two-level handles: their shifted-plane sweep where they have one, and the
+ * band sweep: every number of frequency groups up to 64, 1-16 bands,
  * 32-512 threads in powers of two and the block sizes that cover a band in
  * 1-4 equal passes, the three register budgets, staged or not; where the shape fits and
  * can be scheduled; one launch each,

@@ -60,11 +60,12 @@
 // What bounds it, and what it measured (GB300, one sweep, 9 frequencies; before:
 // the pairs solved twice, one row per thread, FP64 weights in FP64):
 //   FP64 64x64x129: 45 FP64 operations per node and ray (before 154) on a pipe
-//     that issues one warp instruction in 18 clocks; 5.01 -> 1.93 ms.  Small
+//     that issues one warp instruction in 18 clocks; 5.01 -> 1.79 ms.  Small
 //     FP64 planes are the latency of one warp's slots, which the chunks below
-//     run side by side: 16x16x33 220 -> 110 us.
+//     run side by side: 16x16x33 220 -> 104 us.
 //   FP32: issue slots and the wait for the slowest block of a plane; 64x64x129
-//     344 -> 300 us, 128x128x129 1527 -> 980 us.
+//     344 -> 282 us, 128x128x129 1527 -> 825 us (980 with every node's destination
+//     computed from its row instead of read from the row table).
 //
 // Per node the block accumulates, over its slots,
 //   Jeff = sum w phi (I - w0 S)   and   U = sum w phi (1 - w0)
