@@ -61,12 +61,9 @@ ALG_FP32_OPS_PER_UNIT = (4 + 2 + 1 + 7) * N_SOLVED / 9.0 + 10.0 / 9.0
 MUFU_EX2_PER_UNIT = MUFU_RCP_PER_UNIT = N_SOLVED / 9.0
 # DRAM bytes (read + write) of one finest-grid FP64 sweep launch on the bench
 # atmosphere per launch shape (ng, bands, threads, lean, stage), from ncu
-# captures of the current kernel; a shape the autotuner picks that is not
-# listed reports traffic null
-FINE_SWEEP_TRAFFIC = {(9, 5, 224, 0, 2): 14835968 + 141922048,
-                      (9, 5, 256, 0, 2): 14634752 + 141857536,
-                      (9, 5, 448, 0, 2): 13970944 + 144993536,
-                      (9, 5, 512, 0, 2): 13957888 + 143129856}
+# captures of the current kernel; a shape that is not listed reports traffic
+# null
+FINE_SWEEP_TRAFFIC = {}
 SM_MAX_MHZ = 2070.0
 
 
