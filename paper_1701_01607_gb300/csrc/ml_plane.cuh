@@ -74,6 +74,9 @@ __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
     const unsigned frame = (unsigned)rpb * ray_b;       // all rays of one buffer
     const int nplane = nx * ny;
     const long nvox = (long)nplane * nz;
+    // a block's shared memory may be addressed by its cluster once the block runs:
+    // arrive here, wait before the first store into another block
+    if (cl) cluster_arrive_relaxed();
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned buf_addr = smem_addr(smem_raw);
@@ -173,6 +176,7 @@ __device__ __forceinline__ void ml_plane_body(const MlPlaneArgs<T> &a) {
         if (nz > 2) fill_dest(1);
         __syncthreads();
     }
+    if (cl) cluster_wait();   // every block of the cluster has started
     {
         const long k0 = (long)(up ? 0 : nz - 1) * nplane;
         for (int q = threadIdx.x; q < items; q += nth) {

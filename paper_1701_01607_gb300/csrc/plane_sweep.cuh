@@ -372,6 +372,9 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     T *__restrict__ pj = a.pj + slot * (long)nplane * nz;
     T *__restrict__ pu = a.pu + slot * (long)nplane * nz;
     const PlaneSlot<T> *__restrict__ gs = a.slots + (long)g * NP;
+    // a block's shared memory may be addressed by its cluster once the block runs:
+    // arrive here, wait before the first store into another block
+    if (cl && !as) cluster_arrive_relaxed();
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned buf_addr = smem_addr(smem_raw);
@@ -592,6 +595,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
     if (nz > 2) prefetch(2, 2);
     if (nz > 1) fill_dest(0, a.steps[(long)r * nz].sy);
     __syncthreads();
+    if (cl && !as) cluster_wait();   // every block of the cluster has started
     {
         const int k0 = (up ? 0 : nz - 1) * nplane + y0 * nx;
         const PlaneLerp<T> sp = a.steps[(long)r * nz];

@@ -61,6 +61,9 @@ __device__ __forceinline__ void plane_var_body(const PlaneVarArgs<T> &a) {
     T *__restrict__ pj = a.pj + slot * nvox;
     T *__restrict__ pu = a.pu + slot * nvox;
     const T wray = T(1.0 / kRays);
+    // a block's shared memory may be addressed by its cluster once the block runs:
+    // arrive here, wait before the first store into another block
+    if (cl) cluster_arrive_relaxed();
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const unsigned buf_addr = smem_addr(smem_raw);
@@ -183,6 +186,7 @@ __device__ __forceinline__ void plane_var_body(const PlaneVarArgs<T> &a) {
     __syncthreads();   // fx_tab
     if (nz > 1) fill_dest(0, a.steps[(long)r * nz].sy);
     __syncthreads();
+    if (cl) cluster_wait();   // every block of the cluster has started
     {
         const int k0 = plane_of(0);
         const int sx = a.steps[(long)r * nz].sx;
