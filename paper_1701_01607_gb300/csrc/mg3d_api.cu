@@ -457,12 +457,12 @@ void fixed_slots(PlaneSlot<double> *s, int np) {
     int ea = 0;
     if (sum > 0.0L) fx::split(sum * 1.0000001L, &m, &ea);   // sum < 2^ea
     for (int p = 0; p < np; ++p) {
+        s[p].ea = ea;   // of the whole group: the kernel takes it from the first slot
         if (!s[p].fx) continue;
         fx::split(s[p].phi, &s[p].pm, &s[p].pe);
         fx::split(s[p].phi * 1.442695040888963407359924681L, &s[p].ym, &s[p].ye);
         fx::split(1.0L / s[p].phi, &s[p].im, &s[p].ie);
         s[p].aq = (fx::u64)std::ldexp((long double)s[p].w / s[p].phi, 64 - ea);
-        s[p].ea = ea;
     }
 }
 
