@@ -47,12 +47,8 @@ __global__ void opacity_kernel(long nvox, double g_ratio, double kappa,
                                const double *__restrict__ n, T *__restrict__ chi0,
                                T *__restrict__ S) {
     for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox;
-         v += (long)gridDim.x * blockDim.x) {
-        double nl = n[v], nu = n[nvox + v];
-        double diff = nl * g_ratio - nu;
-        chi0[v] = (T)(kappa * diff);
-        S[v] = (T)(nu / diff);
-    }
+         v += (long)gridDim.x * blockDim.x)
+        node_opacity(n[v], n[nvox + v], g_ratio, kappa, chi0 + v, S + v);
 }
 
 template <typename T>

@@ -174,13 +174,9 @@ __global__ void __launch_bounds__(128) rates_kernel(const RateArgs a) {
                 cmax = fmax(cmax, fmax(cl, cu));
             }
             neg += (nl_new <= 0.0) + (nu_new <= 0.0);
-            if (a.chi0) {
-                // opacity and source function of the new populations, for the
-                // formal solution that follows (as opacity_kernel forms them)
-                const double diff = nl_new * a.g_ratio - nu_new;
-                ((TP *)a.chi0)[v] = (TP)(a.kappa * diff);
-                ((TP *)a.S)[v] = (TP)fast_div(nu_new, diff);
-            }
+            // opacity and source function for the formal solution that follows
+            if (a.chi0)
+                node_opacity(nl_new, nu_new, a.g_ratio, a.kappa, (TP *)a.chi0 + v, (TP *)a.S + v);
         } else {
             const double nl = a.n[v], nu = a.n[nvox + v];
             const double w0 = nl + nu;

@@ -105,12 +105,32 @@ __device__ __forceinline__ double fast_rcp(double b, bool &ok) {
     const double e = fma(-b, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
-// a/b: 6 FP64 operations against about 18 of the division
+// a/b: 6 FP64 operations against about 18 of the division.  With b's reciprocal
+// within an ulp and an exact residual a - b q, q + (a - b q)/b misses the quotient by
+// less than 2^-50 ulp before it is rounded, so the result is the correctly rounded
+// one unless the quotient lies that near to a midpoint (2^30 random pairs: equal
+// to the division, bit for bit).  The residual is exact where a and q stay clear of
+// the ends of the exponent range; other operands (0, infinities, NaN) are divided.
 __device__ __forceinline__ double fast_div(double a, double b) {
     bool ok;
     const double y = fast_rcp(b, ok);
     const double q = a * y;
+    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
+    const unsigned eq = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu;
+    ok = ok && ea - 120u < 1900u && eq - 60u < 1980u;
     return ok ? fma(fma(-b, q, a), y, q) : a / b;
+}
+
+// chi0 and S of a two-level node from its populations.  The opacity kernel and
+// the rate kernel (which leaves them to the formal solution that follows) both
+// take them from here, so that results do not depend on how sweeps are split
+// over calls.
+template <typename T>
+__device__ __forceinline__ void node_opacity(double nl, double nu, double g_ratio, double kappa,
+                                             T *chi0, T *S) {
+    const double diff = fma(nl, g_ratio, -nu);
+    *chi0 = (T)(kappa * diff);
+    *S = (T)fast_div(nu, diff);
 }
 
 // closed() has no branch, so a caller can evaluate several independent steps
