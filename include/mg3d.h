@@ -556,9 +556,12 @@ int mg3d_prolong(mg3d_handle *h, int level_fine, int ncomp, const double *coarse
  * The library picks a shape at creation (the shifted-plane sweep with
  * cluster barriers where it applies, at most 8 bands); this overrides it.
  * Moving atmospheres and partial redistribution with the linear upwind
- * interpolation start on a shifted-plane sweep of their own, whose shape
- * mg3d_get_fs_config reports as that of the band sweep it stands for
- * (stage 0) and this call replaces by the band sweep.
+ * interpolation start on a shifted-plane sweep of their own, which lean = 3
+ * with stage = 0 names: bands 1..16, threads 32..512, freq_per_block >= n_freq
+ * for one group, else the frequencies of a group (an even number with partial
+ * redistribution, whose mirror frequencies are solved together).  lean 0 to 2
+ * select the band sweep for them.  mg3d_get_fs_config reports the shape that
+ * runs, in the form in which this call takes it.
  * Returns MG3D_E_ARG if the shape does not fit in shared memory or the GPU
  * cannot hold one of its clusters.
  * No counterpart in the paper (launch control). */

@@ -85,7 +85,6 @@ struct Level {
     StepGeom *geom = nullptr;    // [kRays][nz]
     void *psteps = nullptr;      // [kRays][nz] PlaneLerp<T> of the shifted-plane sweeps
     SweepShape shape{};
-    SweepShape band_shape{};     // with shape.plane 3: the band sweep's shape, as reported
     // formal solutions in the precision other than the handle's (built on the
     // first request, two-level static CRD handles): chi0, S, the bottom
     // intensity, the plane-sweep step table, and the shape
@@ -527,12 +526,21 @@ int sm_count() {
     return n;
 }
 
-// How many clusters of shape s the GPU holds at once (plain launches: blocks).
+// How many clusters of shape s the GPU holds at once (plain launches: blocks),
+// and its dynamic shared memory per block.
+cudaError_t shape_clusters(int prec, const SweepShape &s, int nx, int *n) {
+    return s.plane == 3 ? plane_var_clusters(prec, s, nx, n)
+           : s.plane    ? plane_active_clusters(prec, s, nx, n)
+                        : sweep_active_clusters(prec, s, nx, n);
+}
+size_t shape_smem(int prec, const SweepShape &s, int nx) {
+    return s.plane == 3 ? plane_var_layout(prec, s.prd, s.np, s.rows, nx, s.threads).smem
+           : s.plane    ? plane_layout(prec, s.np, s.rows, nx, s.threads).smem
+                        : sweep_smem_bytes(prec, s, nx);
+}
 int shape_capacity(int prec, const SweepShape &s, int nx) {
     int n = 0;
-    const cudaError_t e = s.plane == 3 ? plane_var_clusters(prec, s, nx, &n)
-                          : s.plane    ? plane_active_clusters(prec, s, nx, &n)
-                                       : sweep_active_clusters(prec, s, nx, &n);
+    const cudaError_t e = shape_clusters(prec, s, nx, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -1626,6 +1634,36 @@ static int plane_shape_from_args(const mg3d_handle *h, int level, int freq_per_b
     return MG3D_OK;
 }
 
+// Shape of the variants' shifted-plane sweep (lean kLeanVariant, stage 0) of the
+// given launch parameters: freq_per_block >= n_freq takes all frequencies in one
+// group; partial redistribution groups mirror pairs, so it takes an even number.
+constexpr int kLeanVariant = 3;
+static int var_shape_from_args(const mg3d_handle *h, int level, int freq_per_block, int bands,
+                               int threads, SweepShape *out) {
+    const Level &L = h->lev[level];
+    const int nf = h->atom.n_freq, nslots = h->prd ? (nf + 1) / 2 : nf;
+    if (!plane_grid_ok(L.nx, L.ny, L.nz))
+        return fail(MG3D_E_ARG, "grid too large for the shifted-plane sweep");
+    if (bands < 1 || bands > kMaxBands || bands > L.ny || threads < 32 || threads > 512 ||
+        threads % 32 || freq_per_block < 1)
+        return fail(MG3D_E_ARG, "bad sweep shape");
+    if (h->prd && freq_per_block < nf && freq_per_block % 2)
+        return fail(MG3D_E_ARG, "partial redistribution takes all frequencies or an even "
+                                "number per block");
+    const int np = freq_per_block >= nf ? nslots : h->prd ? freq_per_block / 2 : freq_per_block;
+    SweepShape s{np, (nslots + np - 1) / np, bands, (L.ny + bands - 1) / bands, threads};
+    if ((long)(bands - 1) * s.rows >= L.ny) return fail(MG3D_E_ARG, "empty band");
+    s.stage = 0;
+    s.plane = 3;
+    s.np = np;
+    s.prd = h->prd ? 1 : 0;
+    s.vel = h->moving ? 1 : 0;
+    if (shape_smem(h->prec, s, L.nx) > plane_smem_max(h->prec == MG3D_PREC_F64))
+        return fail(MG3D_E_ARG, "sweep shape exceeds shared memory");
+    *out = s;
+    return MG3D_OK;
+}
+
 // Shape of the given launch parameters on a level, validated except for
 // whether the GPU can schedule it.
 static int shape_from_args(const mg3d_handle *h, int level, int freq_per_block, int bands,
@@ -1635,6 +1673,8 @@ static int shape_from_args(const mg3d_handle *h, int level, int freq_per_block, 
     if (stage == 2 || stage == 3)
         return plane_shape_from_args(h, level, freq_per_block, bands, threads, lean, out,
                                      stage - 1);
+    if (lean == kLeanVariant && stage == 0 && (h->moving || h->prd) && !h->params.sc_interp)
+        return var_shape_from_args(h, level, freq_per_block, bands, threads, out);
     if (lean < 0 || lean > 2 || (lean == 2 && threads > 256))
         return fail(MG3D_E_ARG, "lean must be 0, 1 or (up to 256 threads) 2");
     if (stage != 0 && stage != 1) return fail(MG3D_E_ARG, "stage must be 0, 1, 2 or 3");
@@ -1657,8 +1697,7 @@ static int shape_from_args(const mg3d_handle *h, int level, int freq_per_block, 
 // k (clusters of more than 8 blocks are not guaranteed to fit).
 int check_schedulable(const mg3d_handle *h, int k, const SweepShape &s) {
     int n = 0;
-    const cudaError_t e = s.plane ? plane_active_clusters(h->prec, s, h->lev[k].nx, &n)
-                                  : sweep_active_clusters(h->prec, s, h->lev[k].nx, &n);
+    const cudaError_t e = shape_clusters(h->prec, s, h->lev[k].nx, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(MG3D_E_ARG,
@@ -1855,10 +1894,7 @@ int autotune_level(mg3d_handle *h, int k, int *evaluated) {
                         best_var = s;
                     }
                 }
-        if (best_var.ng && best_var_ms < best_ms) {
-            L.band_shape = L.shape;
-            L.shape = best_var;
-        }
+        if (best_var.ng && best_var_ms < best_ms) L.shape = best_var;
     }
     if (evaluated) *evaluated = (int)cands.size() + extra;
     return MG3D_OK;
@@ -2048,10 +2084,7 @@ int create_impl(const mg3d_atmosphere *atm, const mg3d_atom *atom, const mg3d_qu
             const int prd = atom->gamma_prd > 0.0 ? 1 : 0;
             const SweepShape v = choose_var_shape(
                 h->prec, L.nx, L.ny, prd ? (atom->n_freq + 1) / 2 : atom->n_freq, prd);
-            if (v.ng) {
-                L.band_shape = L.shape;
-                L.shape = v;
-            }
+            if (v.ng) L.shape = v;
         }
         h->partial_elems = std::max(h->partial_elems,
                                     (size_t)kRays * L.shape.ngroups * (size_t)L.nvox);
@@ -3868,17 +3901,13 @@ int mg3d_get_fs_occupancy(mg3d_handle *h, int level, int freq_per_block, int ban
     SweepShape s;
     MG_TRY(shape_from_args(h, level, freq_per_block, bands, threads, lean, stage, &s));
     int n = 0;
-    const cudaError_t e = s.plane ? plane_active_clusters(h->prec, s, h->lev[level].nx, &n)
-                                  : sweep_active_clusters(h->prec, s, h->lev[level].nx, &n);
+    const cudaError_t e = shape_clusters(h->prec, s, h->lev[level].nx, &n);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(MG3D_E_CUDA, std::string("occupancy query: ") + cudaGetErrorString(e));
     }
     if (max_clusters) *max_clusters = n;
-    if (smem_bytes)
-        *smem_bytes = (long long)(s.plane ? plane_layout(h->prec, s.np, s.rows,
-                                                         h->lev[level].nx, s.threads).smem
-                                          : sweep_smem_bytes(h->prec, s, h->lev[level].nx));
+    if (smem_bytes) *smem_bytes = (long long)shape_smem(h->prec, s, h->lev[level].nx);
     return MG3D_OK;
 }
 
@@ -3912,14 +3941,16 @@ int mg3d_get_fs_config(const mg3d_handle *h, int level, int *freq_per_block, int
                        int *threads, int *lean, int *stage) {
     MG_TRY(check_level(h, level));
     const Level &L = h->lev[level];
-    // the variants' own form is not a shape that can be set: their band sweep's is
-    // reported, which setting it would select
-    const SweepShape &s = L.shape.plane == 3 ? L.band_shape : L.shape;
-    if (freq_per_block) *freq_per_block = s.plane && s.ngroups == 1 ? h->atom.n_freq : s.ng;
+    const SweepShape &s = L.shape;
+    const bool var = s.plane == 3;
+    if (freq_per_block)
+        *freq_per_block = s.plane && s.ngroups == 1 ? h->atom.n_freq
+                          : var && s.prd            ? 2 * s.np
+                                                    : s.ng;
     if (bands) *bands = s.bands;
     if (threads) *threads = s.threads;
-    if (lean) *lean = s.lean;
-    if (stage) *stage = s.plane ? 1 + s.plane : s.stage;
+    if (lean) *lean = var ? kLeanVariant : s.lean;
+    if (stage) *stage = s.plane && !var ? 1 + s.plane : s.stage;
     return MG3D_OK;
 }
 

@@ -458,7 +458,8 @@ def mg3d_set_fs_config(h, level: int, freq_per_block: int, bands: int, threads: 
 
 
 def mg3d_get_fs_config(h, level: int):
-    """(freq_per_block, bands, threads, lean, stage) of a level's sweep."""
+    """(freq_per_block, bands, threads, lean, stage) of a level's sweep, as
+    mg3d_set_fs_config takes them."""
     v = [_I() for _ in range(5)]
     _check(load().mg3d_get_fs_config(h, level, *[ctypes.byref(x) for x in v]))
     return tuple(x.value for x in v)
