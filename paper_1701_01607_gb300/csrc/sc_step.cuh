@@ -100,25 +100,18 @@ struct PairSum {
 // approximate 1/b (relative error e below 2^-20) times 1 + e + e^2, so within an ulp of
 // 1/b; with the exact residual a - b q, q + (a - b q)/b misses the quotient by less
 // than 2^-50 ulp before it is rounded, so the result is the correctly rounded one unless
-// the quotient lies that near to a midpoint (3 x 2^30 random pairs: equal to the
-// division, bit for bit).  The residual is exact where a, b and the quotient stay
-// clear of the ends of the exponent range; other operands (infinities, NaN) are
-// divided.  a = 0 is not one of them: populations of deep nodes do not change at all,
-// and 44 sweeps of a small 6-level cycle lost 140 us to their divisions.
+// the quotient lies that near to a midpoint (2 x 2^30 random pairs: equal to the
+// division, bit for bit).  Denominators of exponents beyond 1000 are divided.  Where a or
+// the quotient is infinite the result is NaN (a caller counts both as not finite);
+// where a - b q is denormal the result may be an ulp off.
 __device__ __forceinline__ double fast_div(double a, double b) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    const unsigned ha = (unsigned)__double2hiint(a);
-    const unsigned ea = (ha >> 20) & 0x7ffu;
-    const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
-    const bool zero = ((ha << 1) | (unsigned)__double2loint(a)) == 0;
-    if (eb - 23u < 2000u && (zero || (ea - 120u < 1900u && ea - eb + 950u < 1900u))) {
-        const double e = fma(-b, y, 1.0);
-        y = fma(y, fma(e, e, e), y);
-        const double q = a * y;
-        return zero ? q : fma(fma(-b, q, a), y, q);
-    }
-    return a / b;
+    const bool ok = (((unsigned)__double2hiint(b) >> 20) & 0x7ffu) - 23u < 2000u;
+    const double e = fma(-b, y, 1.0);
+    y = fma(y, fma(e, e, e), y);
+    const double q = a * y;
+    return ok ? fma(fma(-b, q, a), y, q) : a / b;
 }
 
 // chi0 and S of a two-level node from its populations.  The opacity kernel and
