@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <cfloat>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -2624,14 +2625,20 @@ bool choose_ml_plane(Level &L, int nf) {
     return false;
 }
 
-// Constants of every frequency for the opacity and the radiative sums.
+// Constants of every frequency for the opacity and the radiative sums, and the
+// transitions whose constants leave the range of pairs of floats.
 int setup_freq_ops(mg3d_handle *h) {
     std::vector<FreqOp> ops(h->fi.size());
     auto pair = [](double v, float *hi, float *lo) {
+        v = std::min(v, (double)FLT_MAX);   // an exponent beyond it: e^-v is 0 all the same
         *hi = (float)v;
         *lo = (float)(v - (double)*hi);
     };
-    for (const TransInfo &tr : h->ti)
+    auto wide = [](double v) {
+        return v != 0.0 && !(std::fabs(v) >= std::ldexp(1.0, -100) &&
+                             std::fabs(v) <= std::ldexp(1.0, 100));
+    };
+    for (TransInfo &tr : h->ti)
         for (int f = tr.f_begin; f < tr.f_end; ++f) {
             const FreqInfo &q = h->fi[f];
             FreqOp o{};
@@ -2657,6 +2664,8 @@ int setup_freq_ops(mg3d_handle *h) {
             o.kapf = (float)o.kap;
             o.emisf = (float)o.emis;
             o.ry3f = (float)o.ry3;
+            if (wide(o.w) || wide(o.q3) || (tr.kind == 1 && (wide(o.kap) || wide(o.emis))))
+                tr.wide = 1;
             ops[f] = o;
         }
     MG_TRY(dev_alloc((void **)&h->d_fo, ops.size() * sizeof(FreqOp)));
@@ -2898,9 +2907,9 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
     MG_TRY(dev_alloc((void **)&h->d_ti, h->ti.size() * sizeof(TransInfo)));
     MG_CUDA(cudaMemcpy(h->d_fi, h->fi.data(), h->fi.size() * sizeof(FreqInfo),
                        cudaMemcpyHostToDevice));
+    MG_TRY(setup_freq_ops(h));
     MG_CUDA(cudaMemcpy(h->d_ti, h->ti.data(), h->ti.size() * sizeof(TransInfo),
                        cudaMemcpyHostToDevice));
-    MG_TRY(setup_freq_ops(h));
     for (int k = 1; k <= h->L; ++k) {
         Level &L = h->lev[k];
         MG_TRY(setup_node_tab(h, L, atom->n_lines));

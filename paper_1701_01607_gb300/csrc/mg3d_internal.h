@@ -317,6 +317,7 @@ struct TransInfo {
     double coef;    // line: A_ul; continuum: beta
     double gr;      // line: g_u/g_l
     double b_ul;    // line: Einstein B_ul = A_ul/rho^3
+    int wide = 0;   // constants outside 2^-100 .. 2^100: FP32 handles take FP64 formulas
 };
 
 template <typename T>

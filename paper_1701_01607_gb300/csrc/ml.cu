@@ -213,7 +213,7 @@ __global__ void ml_opacity_kernel(const MlOpacityArgs a) {
                 cont_terms(q, inv_T, ft, E, B);
                 chi_t = kap * (nlT - ndT * E);
                 if constexpr (sizeof(T) == 8) eta_t = kap * (ndT * q.ry3) * E;
-                else eta_t = emis * ndT * E;
+                else eta_t = tr.wide ? kap * (T)(nd * q.ry3) * E : emis * ndT * E;
             }
             // the background's opacity and emissivity (continuum, and
             // coherent scattering of the previous mean intensity)
@@ -942,11 +942,6 @@ __device__ __forceinline__ unsigned long long dbits_ml(double x) {
 }
 
 // an angle sum over the ray-group slots, in slot order
-__device__ __forceinline__ double slots_sum(const double *p, long stride, int n) {
-    double s = p[0];
-    for (int i = 1; i < n; ++i) s += p[(long)i * stride];
-    return s;
-}
 __device__ __forceinline__ PairSum slots_sum(const float *p, long stride, int n) {
     PairSum s;
     s.hi = p[0];
@@ -954,12 +949,74 @@ __device__ __forceinline__ PairSum slots_sum(const float *p, long stride, int n)
     return s;
 }
 
-// Radiative sums of transition blockIdx.y over the chunk's frequencies, added
-// to acc (frequencies in increasing order within a chunk, chunks in order).
-// The sums of a line share the factor 1/(sqrt(pi) d) of its profile, which
-// cancels in their ratios and is left out.
-// PLAIN: no flow, partial redistribution, damped line, background field or zero
-// radiation.
+// The same in FP64 for either precision.
+template <typename T>
+__device__ __forceinline__ double slots_sum64(const T *p, long stride, int n) {
+    double s = (double)p[0];
+    for (int i = 1; i < n; ++i) s += (double)p[(long)i * stride];
+    return s;
+}
+
+// Radiative sums of a transition over the chunk's frequencies, added to acc
+// (frequencies in increasing order within a chunk, chunks in order).  The sums
+// of a line share the factor 1/(sqrt(pi) d) of its profile, which cancels in
+// their ratios and is left out.
+struct AccumSums {
+    double s0, s1, s2;
+};
+
+// The sums of transition tr at node v over frequencies fb .. fe-1 in FP64, from
+// angle sums and exponentials in the formal-solution precision T.  PLAIN: no flow,
+// partial redistribution, damped line or zero radiation.
+template <typename T, bool PLAIN>
+__device__ __forceinline__ AccumSums accum_sums(const MlAccumArgs &a, const TransInfo &tr, int fb,
+                                                int fe, long v, const fx::Tables &ft) {
+    const long nvox = a.nvox, hstride = (long)a.nfreq * nvox;
+    const MlNode<T> node(a.tab, v);
+    const double inv_d = !PLAIN && tr.kind == 0 && a.voigt ? a.tab.inv_d[v] : 0.0;
+    const bool zero = !PLAIN && a.zero_radiation;
+    AccumSums s{0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int f = fb; f < fe; ++f) {
+        const FreqOp &q = a.fo[f];
+        const long i = (long)(f - a.f0) * nvox + v;
+        double J = 0.0, U = 1.0;
+        if (!zero) {
+            J = slots_sum64((const T *)a.jx + i, hstride, a.nslots);
+            U = slots_sum64((const T *)a.ux + i, hstride, a.nslots);
+        }
+        if (tr.kind == 0) {
+            if (!PLAIN && a.moving && !zero) {
+                // the per-ray profile weights are inside J and U already
+                s.s0 += f == tr.f_begin ? 1.0 : 0.0;
+                s.s1 += J;
+                s.s2 += U;
+                continue;
+            }
+            const int pr = !PLAIN && a.prd_index && !zero ? a.prd_index[f] : -1;
+            if (pr >= 0) {
+                // U = sum_r w_r (1 - w0 (1 - oc)) = oc + (1 - oc) sum_r w_r u_r
+                const double oc = a.prd_oc[(long)pr * nvox + v];
+                U = oc + (1.0 - oc) * U;
+            }
+            const T phi = !PLAIN && q.damped ? (T)voigt_H_rational(*a.voigt, a.fi[f].adamp * inv_d,
+                                                                   q.a * inv_d)
+                                             : node.line_exp(q, ft);
+            const double wphi = q.w * (double)phi;
+            s.s0 += wphi;
+            s.s1 = fma(wphi, J, s.s1);
+            s.s2 = fma(wphi, U, s.s2);
+        } else {
+            const double E = (double)node.cont_exp(q, ft);
+            s.s0 = fma(q.w, J, s.s0);
+            s.s1 = fma(q.w * E, J, s.s1);
+            s.s2 = fma(q.q3 * E, U, s.s2);
+        }
+    }
+    return s;
+}
+
+// PLAIN: nor a background field.
 template <bool PLAIN>
 __global__ void ml_accum64_kernel(const MlAccumArgs a) {
     __shared__ fx::u64 fx_tab[2 * fx::kTab];
@@ -975,79 +1032,78 @@ __global__ void ml_accum64_kernel(const MlAccumArgs a) {
     if (fb >= fe) return;
     for (long v = blockIdx.x * (long)blockDim.x + threadIdx.x; v < nvox;
          v += (long)gridDim.x * blockDim.x) {
-        const MlNode<double> node(a.tab, v);
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        AccumSums s{0.0, 0.0, 0.0};
         if (PLAIN) {
+            const MlNode<double> node(a.tab, v);
             // the next frequency's angle sums are loaded while this one's are added
             const double *pj = jx + (long)(fb - a.f0) * nvox + v;
             const double *pu = ux + (long)(fb - a.f0) * nvox + v;
 #pragma unroll 2
             for (int f = fb; f < fe; ++f, pj += nvox, pu += nvox) {
                 const FreqOp &q = a.fo[f];
-                const double J = slots_sum(pj, hstride, a.nslots);
-                const double U = slots_sum(pu, hstride, a.nslots);
+                const double J = slots_sum64(pj, hstride, a.nslots);
+                const double U = slots_sum64(pu, hstride, a.nslots);
                 if (tr.kind == 0) {
                     const double wphi = q.w * node.line_exp(q, ft);
-                    s0 += wphi;
-                    s1 = fma(wphi, J, s1);
-                    s2 = fma(wphi, U, s2);
+                    s.s0 += wphi;
+                    s.s1 = fma(wphi, J, s.s1);
+                    s.s2 = fma(wphi, U, s.s2);
                 } else {
                     const double E = node.cont_exp(q, ft);
-                    s0 = fma(q.w, J, s0);
-                    s1 = fma(q.w * E, J, s1);
-                    s2 = fma(q.q3 * E, U, s2);
+                    s.s0 = fma(q.w, J, s.s0);
+                    s.s1 = fma(q.w * E, J, s.s1);
+                    s.s2 = fma(q.q3 * E, U, s.s2);
                 }
             }
-        } else
-        for (int f = fb; f < fe; ++f) {
-            const FreqOp &q = a.fo[f];
-            const long i = (long)(f - a.f0) * nvox + v;
-            double J = 0.0, U = 1.0;
-            if (!a.zero_radiation) {
-                J = slots_sum(jx + i, hstride, a.nslots);
-                U = slots_sum(ux + i, hstride, a.nslots);
-            }
-            if (tr.kind == 0) {
-                if (a.moving && !a.zero_radiation) {
-                    // the per-ray profile weights are inside J and U already
-                    s0 += f == tr.f_begin ? 1.0 : 0.0;
-                    s1 += J;
-                    s2 += U;
-                } else {
-                    const int pr = a.prd_index && !a.zero_radiation ? a.prd_index[f] : -1;
-                    if (pr >= 0) {
-                        // U = sum_r w_r (1 - w0 (1 - oc)) = oc + (1 - oc) sum_r w_r u_r
-                        const double oc = a.prd_oc[(long)pr * nvox + v];
-                        U = oc + (1.0 - oc) * U;
-                    }
-                    const double wphi =
-                        q.w * (q.damped ? voigt_H_rational(*a.voigt, a.fi[f].adamp * node.inv_d,
-                                                           q.a * node.inv_d)
-                                        : node.line_exp(q, ft));
-                    s0 += wphi;
-                    s1 = fma(wphi, J, s1);
-                    s2 = fma(wphi, U, s2);
-                }
-            } else {
-                const double E = node.cont_exp(q, ft);
-                s0 = fma(q.w, J, s0);
-                s1 = fma(q.w * E, J, s1);
-                s2 = fma(q.q3 * E, U, s2);
-            }
-            // background field of the frequency: the new mean intensity
+        } else {
+            s = accum_sums<double, false>(a, tr, fb, fe, v, ft);
+            // background field: the new mean intensity
             if (a.jbg && !a.zero_radiation)
-                ((double *)a.jbg)[(long)f * nvox + v] =
-                    slots_sum((const double *)a.jm + i, hstride, a.nslots);
+                for (int f = fb; f < fe; ++f)
+                    ((double *)a.jbg)[(long)f * nvox + v] = slots_sum64(
+                        (const double *)a.jm + (long)(f - a.f0) * nvox + v, hstride, a.nslots);
         }
         double *acc = a.acc + (long)t * kAccTerms * nvox + v;
-        acc[0] += s0;
-        acc[nvox] += s1;
-        acc[2 * nvox] += s2;
+        acc[0] += s.s0;
+        acc[nvox] += s.s1;
+        acc[2 * nvox] += s.s2;
     }
 }
 
+// FP32 angle sums are added as pairs of floats, whose products are good to
+// about 2^-45 while no operand or product drops below the 2^-149 a float holds.  A
+// node's sums of a transition go to FP64 instead (from the same FP32 angle sums and
+// exponentials) where that is not certain:
+//   a coefficient outside 2^-100 .. 2^100 (TransInfo::wide, for all nodes);
+//   a sum below 2^-80 of the largest mean intensity (or of 1).  A term that lost
+//   bits is below 2^-100 of that, so it is below 2^-20 of a larger sum, and what it
+//   lost is 2^-24 of itself; for a continuum only the sum of the smaller of the two
+//   terms of its downward rate may be tiny;
+//   a sum above 2^100, infinite or NaN.
+// A continuum's exponential leaves the range from x of about 55 on.  The test costs
+// nothing (64x64x65, 120 frequencies: sums 211 us before, 184 with it and 64 registers,
+// which let four blocks share an SM), and the populations' errors against an FP64 handle are
+// the same with all nodes in pairs and all nodes in FP64 (rms 3.7175e-9 both, 60 boxes).
+__device__ __forceinline__ bool pairs_hold(const TransInfo &tr, const PairSum &s0,
+                                           const PairSum &s1, const PairSum &s2, float jmax) {
+    const float lo = __int_as_float((127 - 80) << 23) * fmaxf(jmax, 1.0f);
+    const float hi = __int_as_float((127 + 100) << 23);
+    const float a0 = fabsf(s0.hi), a1 = fabsf(s1.hi), a2 = fabsf(s2.hi);
+    const float rad = tr.kind == 0 ? a1 : a0;   // 0 without radiation
+    return (rad >= lo || jmax == 0.0f) && (tr.kind == 0 ? fminf(a0, a2) : a2) >= lo &&
+           fmaxf(fmaxf(a0, a1), a2) <= hi;
+}
+
+// Not inlined: it would take part in the register allocation of the loop that always runs.
 template <bool PLAIN>
-__global__ void __launch_bounds__(256) ml_accum32_kernel(const MlAccumArgs a) {
+__device__ __noinline__ AccumSums accum_sums_wide(const MlAccumArgs &a, const TransInfo &tr, int fb,
+                                                  int fe, long v) {
+    return accum_sums<float, PLAIN>(a, tr, fb, fe, v, fx::Tables{nullptr, nullptr});
+}
+
+template <bool PLAIN>
+__global__ void __launch_bounds__(256, 4)
+    ml_accum32_kernel(const __grid_constant__ MlAccumArgs a) {
     const fx::Tables none{nullptr, nullptr};
     const float *__restrict__ jx = (const float *)a.jx;
     const float *__restrict__ ux = (const float *)a.ux;
@@ -1061,15 +1117,18 @@ __global__ void __launch_bounds__(256) ml_accum32_kernel(const MlAccumArgs a) {
         const MlNode<float> node(a.tab, v);
         const double inv_d = tr.kind == 0 && a.voigt ? a.tab.inv_d[v] : 0.0;
         PairSum s0, s1, s2;
+        float jmax = 0.0f;   // largest mean intensity of the transition
         auto add_line = [&](const FreqOp &q, float phi, const PairSum &J, const PairSum &U) {
             const float wh = q.wh * phi;   // w phi as a pair
             const float wl = fmaf(q.wl, phi, fmaf(q.wh, phi, -wh));
+            jmax = fmaxf(jmax, fabsf(J.hi));
             s0.add(wh);
             s0.lo += wl;
             s1.add_product(wh, wl, J.hi, J.lo);
             s2.add_product(wh, wl, U.hi, U.lo);
         };
         auto add_cont = [&](const FreqOp &q, float E, const PairSum &J, const PairSum &U) {
+            jmax = fmaxf(jmax, fabsf(J.hi));
             s0.add_product(q.wh, q.wl, J.hi, J.lo);
             const float eh = q.wh * E, el = fmaf(q.wl, E, fmaf(q.wh, E, -eh));
             s1.add_product(eh, el, J.hi, J.lo);
@@ -1123,6 +1182,7 @@ __global__ void __launch_bounds__(256) ml_accum32_kernel(const MlAccumArgs a) {
             if (tr.kind == 0) {
                 if (a.moving && !a.zero_radiation) {
                     // the per-ray profile weights are inside J and U already
+                    jmax = fmaxf(jmax, fabsf(J.hi));
                     s0.add(f == tr.f_begin ? 1.0f : 0.0f);
                     s1.add_product(1.0f, 0.0f, J.hi, J.lo);
                     s2.add_product(1.0f, 0.0f, U.hi, U.lo);
@@ -1150,10 +1210,13 @@ __global__ void __launch_bounds__(256) ml_accum32_kernel(const MlAccumArgs a) {
                 ((float *)a.jbg)[(long)f * nvox + v] = m.hi + m.lo;
             }
         }
+        AccumSums s{s0.value(), s1.value(), s2.value()};
+        if (tr.wide || !pairs_hold(tr, s0, s1, s2, jmax))
+            s = accum_sums_wide<PLAIN>(a, a.ti[t], fb, fe, v);
         double *acc = a.acc + (long)t * kAccTerms * nvox + v;
-        acc[0] += s0.value();
-        acc[nvox] += s1.value();
-        acc[2 * nvox] += s2.value();
+        acc[0] += s.s0;
+        acc[nvox] += s.s1;
+        acc[2 * nvox] += s.s2;
     }
 }
 
