@@ -167,11 +167,6 @@ __device__ __forceinline__ double exp_neg_fx(double x, const Tables t) {
     if (x < 1.0) return fma(x, fma(x, fma(x, fma(x, 1.0 / 24.0, -1.0 / 6.0), 0.5), -1.0), 1.0);
     return exp(-x);
 }
-// v 2^-64 2^-n in FP32
-__device__ __forceinline__ float to_float(u64 v, int n) {
-    return __ull2float_rn(v) * 5.4210108624275222e-20f * __int_as_float(max(0, 127 - n) << 23);
-}
-
 struct Weights {
     u64 E;           // e^-x = E 2^-64 2^-n (0: below 2^-1015)
     int n;

@@ -2654,6 +2654,7 @@ int setup_freq_ops(mg3d_handle *h) {
                 o.a = h->theta_ref * q.rho * y;
                 o.kap = q.kappa / (y * y * y);
                 o.ry3 = ry * ry * ry;
+                fx::split(o.ry3, &o.rm, &o.re);
                 o.emis = o.kap * o.ry3;
                 o.w = tr.coef * q.w / (y * y * y * y);
                 o.q3 = o.w * o.ry3;
@@ -2663,7 +2664,6 @@ int setup_freq_ops(mg3d_handle *h) {
             pair(o.w, &o.wh, &o.wl);
             o.kapf = (float)o.kap;
             o.emisf = (float)o.emis;
-            o.ry3f = (float)o.ry3;
             if (wide(o.w) || wide(o.q3) || (tr.kind == 1 && (wide(o.kap) || wide(o.emis))))
                 tr.wide = 1;
             ops[f] = o;

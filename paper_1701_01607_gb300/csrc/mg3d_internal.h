@@ -420,8 +420,9 @@ struct alignas(16) FreqOp {
     // FP32: line: a = x^2, continuum: a = theta_ref rho y; kap, emis as below
     float ah, al, kapf, emisf;
     float wh, wl, q3h, q3l;      // line: w (trapezoid weight); continuum: qa; qa (rho y)^3
-    float ry3f;                  // continuum: (rho y)^3
     int damped;                  // line: Voigt profile
+    int re;                      // continuum: (rho y)^3 = rm 2^-64 2^re
+    unsigned long long rm;
     double a;                    // line: x; continuum: theta_ref rho y
     double kap, emis;            // line: kappa, kappa rho^3; continuum: kappa/y^3 (emis: times
                                  // (rho y)^3 in FP32, unused in FP64)

@@ -133,6 +133,29 @@ struct MlNode<double> {
     }
 };
 
+// f 2^e
+__device__ __forceinline__ float scaled(float f, int e) {
+    return (unsigned)(e + 126) < 253u ? f * __int_as_float((e + 127) << 23) : ldexpf(f, e);
+}
+
+// E/D rm 2^-64 2^e for fractions E, D of 64 bits (E, D and rm 2^-64 at least 2^-12), in
+// FP32, rounded once from 29 bits or more: 1/D from the FP32 reciprocal and one Newton step.
+// (Three FP32 operations instead take 15 us less of the 170 of 64x64x65 nodes and 120
+// frequencies, with a third more error in a thick background: rms 9.4e-8 for 8.1e-8.)
+__device__ __forceinline__ float planck_ratio(fx::u64 E, fx::u64 D, fx::u64 rm, int e) {
+    const int z = __clz((unsigned)(D >> 32));
+    const unsigned Dh = (unsigned)((D << z) >> 32);                       // 2^-32
+    float f;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(__uint2float_rz(Dh)));
+    const unsigned r0 = __float2uint_rz(fminf(f * 9223372036854775808.0f, 4294967040.0f));
+    const long long c = (long long)(0x8000000000000000ull - (fx::u64)Dh * r0);   // 2^-63
+    const long long r1 = (long long)r0 + (((long long)r0 * (int)(c >> 11)) >> 52);
+    const unsigned r = (unsigned)min(r1, 0xffffffffll);                   // 1/D, 2^-31 2^z
+    const unsigned t = (unsigned)(((E >> 32) * r + 0x80000000ull) >> 32);
+    const unsigned b = (unsigned)((t * (rm >> 32) + 0x80000000ull) >> 32);
+    return scaled(__uint2float_rn(b), z + e - 31);
+}
+
 // Bound-free continuum: E = e^-x and the Planck function (rho y)^3/(e^x - 1),
 // x = theta_ref rho y/T.
 __device__ __forceinline__ void cont_terms(const FreqOp &q, double inv_T, const fx::Tables &ft,
@@ -141,8 +164,8 @@ __device__ __forceinline__ void cont_terms(const FreqOp &q, double inv_T, const 
     fx::u64 e, d;
     int n;
     if (fx::exp_parts(x, ft, &e, &n, &d)) {
-        E = fx::to_float(e, n);
-        B = q.ry3f * E / fx::to_float(d, 0);
+        E = scaled(__ull2float_rn(e), -64 - n);
+        B = planck_ratio(e, d, q.rm, q.re - n);
     } else {
         E = expf(-(float)x);
         B = (float)(q.ry3 / expm1(x));
