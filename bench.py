@@ -41,17 +41,15 @@ N_GRIDS = 3
 METRIC = "FS Gvoxel*ray*freq/s (3-grid FAS V-cycle step)"
 UNIT = "Gunit/s"
 FS_UNITS_PER_FINE = GRID[0] * GRID[1] * GRID[2] * 24 * 9
-# FP64 floating-point operations per (node, ray, frequency) of the sweep.
 # phi(x) = phi(-x) and S does not depend on frequency, so the intensities of a
-# mirror pair are the same and are solved once: 5 of the 9 frequencies.  Per
-# solved frequency bilinear I_up 7, new I 5, two accumulations 4 and the
-# short-characteristics weights (optical path 1, exp 1, u 2, w0 1, w_up 1), plus
-# 16 per node and ray for the chi/S interpolation and dtau.  exp and the
-# division count as one operation each; the FP64 sweep forms the weights in
-# integer arithmetic, so not all of these run on the FP64 pipe.
+# mirror pair are the same and are solved once: 5 of the 9 frequencies.
 N_SOLVED = (9 + 1) // 2
-ALG_FLOPS_PER_UNIT = (7 + 5 + 4 + (1 + 1 + 2 + 1 + 1)) * N_SOLVED / 9.0 + 16.0 / 9.0
-FP64_NOMINAL_TFLOPS = 1.25      # GB300, at the 2070 MHz maximum SM clock
+# FP64 instructions per (node, ray, frequency) that the FP64 sweep needs on the
+# FP64 pipe: per node and ray 2.5 multiply-adds of the interpolation for each of the
+# channels (chi0, S and the intensities), the optical path 2, S_up 1 and the U sum 1;
+# per solved frequency w_up S_up, I - w0 S, the Jeff sum and the new I.  The
+# short-characteristics weights are formed on the integer pipes.
+FP64_OPS_PER_UNIT = (2.5 * (N_SOLVED + 2) + 4 + 4 * N_SOLVED) / 9.0
 # FP32 instructions per unit the FP32 sweep needs (each an FMA-pipe
 # instruction): per solved frequency the bilinear I_up 4, the new I 2, the Jeff
 # sum 1, the optical path 1, the exp2 argument 1, u 1, w0 1, w_up 1, w_up S_up 1
@@ -59,12 +57,6 @@ FP64_NOMINAL_TFLOPS = 1.25      # GB300, at the 2070 MHz maximum SM clock
 # solved frequency one ex2 and one rcp on the multi-function unit.
 ALG_FP32_OPS_PER_UNIT = (4 + 2 + 1 + 7) * N_SOLVED / 9.0 + 10.0 / 9.0
 MUFU_EX2_PER_UNIT = MUFU_RCP_PER_UNIT = N_SOLVED / 9.0
-# DRAM bytes (read + write) of one finest-grid FP64 sweep launch on the bench
-# atmosphere per launch shape (ng, bands, threads, lean, stage), from ncu
-# captures of the current kernel; a shape that is not listed reports traffic
-# null
-FINE_SWEEP_TRAFFIC = {}
-SM_MAX_MHZ = 2070.0
 
 
 def env_rank():
@@ -261,10 +253,8 @@ def run_gpu(args):
 
     result = None
     if rank == 0:
-        peak = 2.0 * peaks["dfma"] / 1e12       # measured FP64 TFLOP/s
-        achieved = ALG_FLOPS_PER_UNIT * fine_units / (fine_ms * 1e-3) / 1e12
-        fine_shape = list(tuning.get("f64", {}).get("shapes", {}).get(fine, ()))
-        traffic = FINE_SWEEP_TRAFFIC.get(tuple(fine_shape))
+        peak = peaks["dfma"] / 1e12             # measured FP64 instruction rate
+        achieved = FP64_OPS_PER_UNIT * fine_units / (fine_ms * 1e-3) / 1e12
         result = {
             "metric": METRIC, "value": round(value, 4), "unit": UNIT, "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup,
@@ -280,12 +270,10 @@ def run_gpu(args):
                        "sweep_autotune": tuning},
             "roofline": {"kernel": "plane_sweep_kernel<double> (finest grid)", "bound": "alu",
                          "achieved": round(achieved, 4), "peak": round(peak, 4),
-                         "unit": "TFLOP/s", "frac": round(achieved / peak, 4),
-                         "traffic": traffic,
-                         "peak_source": "measured FP64 FMA rate x 2 (mg3d_probe_alu_peaks, "
-                                        "this run); nominal 1.25 TFLOP/s",
-                         "frac_of_nominal": round(achieved / FP64_NOMINAL_TFLOPS, 4),
-                         "alg_flops_per_unit": round(ALG_FLOPS_PER_UNIT, 3),
+                         "unit": "T FP64 instructions/s", "frac": round(achieved / peak, 4),
+                         "peak_source": "measured FP64 multiply-add rate "
+                                        "(mg3d_probe_alu_peaks, this run)",
+                         "alg_fp64_ops_per_unit": round(FP64_OPS_PER_UNIT, 3),
                          "units_per_launch": fine_units,
                          "ms_per_launch": round(fine_ms, 4),
                          "timing": "sweep launches timed in a separate instrumented pass"},
@@ -308,11 +296,10 @@ def run_gpu(args):
                 "value": round(cnt32["fs_units"] / (sum(ms32) * 1e-3) / 1e9, 4),
                 "ms_per_step": round(sum(ms32) / args.steps, 4),
                 "fine_sweep_ms": round(fine_ms32, 4),
-                "fine_sweep_gunits_s": round(fine_units / (fine_ms32 * 1e-3) / 1e9, 3)},
+                "fine_sweep_gunits_s": round(fine_units / (fine_ms32 * 1e-3) / 1e9, 3),
+                "sweep_ms_per_launch_by_level": sweep_ms_by_level(cnt32_t)},
             "fine_sweep_gunits_s": round(fine_units / (fine_ms * 1e-3) / 1e9, 3),
-            "sweep_ms_per_launch_by_level": {
-                k: round(cnt["level_fs_kernel_ms"][k] / max(1, cnt["level_fs_timed_launches"][k]), 4)
-                for k in range(1, N_GRIDS + 1)},
+            "sweep_ms_per_launch_by_level": sweep_ms_by_level(cnt_t),
             "sweep_launches_per_step_by_level": {
                 k: cnt["level_fs_launches"][k] // args.steps for k in range(1, N_GRIDS + 1)},
         }
@@ -329,6 +316,12 @@ def run_gpu(args):
         dist.barrier()
         dist.destroy_process_group()
     return result
+
+
+def sweep_ms_by_level(counters):
+    """Mean device time of a sweep launch on each grid, of a run with timing on."""
+    ms, n = counters["level_fs_kernel_ms"], counters["level_fs_timed_launches"]
+    return {k: round(ms[k] / max(1, n[k]), 4) for k in range(1, N_GRIDS + 1)}
 
 
 def roofline_fp32(units, ms, peaks, kernel):
