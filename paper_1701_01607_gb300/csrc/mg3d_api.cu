@@ -481,7 +481,6 @@ int build_plane_slots(mg3d_handle *h, void **out) {
             if (j >= nslots) continue;   // inactive slot of the last group
             const int m = nf - 1 - j;
             tab[j].phi = (T)h->phi[j];
-            tab[j].iphi = (T)(1.0 / h->phi[j]);
             tab[j].w = (T)((h->wphi[j] + (m > j ? h->wphi[m] : 0.0)) / kRays);
         }
         if constexpr (sizeof(T) == 8)
@@ -822,9 +821,7 @@ MlOpacityArgs ml_opacity_args(const mg3d_handle *h, const Level &L, int f0, int 
     a.fo = h->d_fo;
     a.ti = h->d_ti;
     a.tab = L.ntab;
-    a.theta_ref = h->theta_ref;
     a.n = L.n;
-    a.T = L.T;
     a.chi_c = L.chi_c;
     a.saha = L.saha;
     a.chi = L.mchi;
@@ -1840,7 +1837,6 @@ int autotune_level(mg3d_handle *h, int k, int *evaluated) {
         }
     g_last_error.clear();
     if (cands.empty()) return fail(MG3D_E_ARG, "no sweep shape fits");
-    (void)0;
     size_t need = 0;
     for (auto &s : cands) need = std::max(need, (size_t)kRays * s.ngroups * (size_t)L.nvox);
     MG_TRY(ensure_partials(h, need));

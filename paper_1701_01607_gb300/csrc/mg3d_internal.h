@@ -74,15 +74,15 @@ struct alignas(16) PlaneLerp<float> {
 // line centre.
 template <typename T>
 struct PlaneSlot {
-    T phi, iphi;   // profile value and its inverse
-    T w;           // ray weight x sum of the frequencies' weights x profile (0: inactive)
+    T phi;   // profile value
+    T w;     // ray weight x sum of the frequencies' weights x profile (0: inactive)
 };
 
 // FP64: the same as operands of the integer weights (fixed_weights.cuh), a value
 // m 2^-64 2^e each.
 template <>
 struct PlaneSlot<double> {
-    double phi, iphi, w;
+    double phi, w;
     unsigned long long pm, ym, im;   // phi, phi log2(e), 1/phi
     unsigned long long aq;           // w/phi in units of 2^(ea - 64); sum over a group < 2^64
     int pe, ye, ie, ea;
@@ -444,8 +444,7 @@ struct MlOpacityArgs {
     const FreqOp *fo;
     const TransInfo *ti;
     MlNodeTab tab;
-    double theta_ref;
-    const double *n, *T, *chi_c, *saha;
+    const double *n, *chi_c, *saha;
     void *chi, *S, *sc, *oc;       // sc = S - rho eta_t/chi, oc = 1 - chi_t/chi (0 for a
                                    // PRD frequency: its 1 - rho chi_t/chi goes in FP64
                                    // to the radiative sums, MlAccumArgs::prd_oc)

@@ -125,7 +125,7 @@ __device__ __forceinline__ unsigned cluster_rank() {
 }
 // 16-byte store of (v[0..VW-1]) at a shared::cluster address (this block's
 // or another block's shared memory; a launch without clusters is a cluster of
-// one block), unconditional or under a predicate.  No memory clobber: the
+// one block).  No memory clobber: the
 // stores go to the plane being written, which no thread reads before the
 // barrier (whose asm carries the clobber) that ends the step.
 __device__ __forceinline__ void st16(unsigned a, const float *v) {
@@ -134,18 +134,6 @@ __device__ __forceinline__ void st16(unsigned a, const float *v) {
 }
 __device__ __forceinline__ void st16(unsigned a, const double *v) {
     asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(v[0]), "d"(v[1]));
-}
-__device__ __forceinline__ void st16_if(bool c, unsigned a, const float *v) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t"
-        "@p st.shared::cluster.v4.f32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"((int)c),
-        "r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]));
-}
-__device__ __forceinline__ void st16_if(bool c, unsigned a, const double *v) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t"
-        "@p st.shared::cluster.v2.f64 [%1], {%2, %3};\n\t}" ::"r"((int)c),
-        "r"(a), "d"(v[0]), "d"(v[1]));
 }
 // one 16-byte vector at an address of this block's shared memory
 __device__ __forceinline__ void lds16(unsigned a, float *o) {
@@ -195,22 +183,19 @@ __device__ __forceinline__ void cluster_wait() {
 }
 // 16-byte store into another block's shared memory that completes 16 bytes of
 // the transaction count of the mbarrier at `bar` (a shared::cluster address
-// in the same block), under a predicate
-__device__ __forceinline__ void st16_async_if(bool c, unsigned a, const float *v, unsigned bar) {
+// in the same block)
+__device__ __forceinline__ void st16_async(unsigned a, const float *v, unsigned bar) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t"
-        "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%1], "
-        "{%2, %3, %4, %5}, [%6];\n\t}" ::"r"((int)c),
-        "r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar)
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], "
+        "{%1, %2, %3, %4}, [%5];" ::"r"(a),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar)
         : "memory");
 }
-__device__ __forceinline__ void st16_async_if(bool c, unsigned a, const double *v,
-                                              unsigned bar) {
+__device__ __forceinline__ void st16_async(unsigned a, const double *v, unsigned bar) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t"
-        "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%1], "
-        "{%2, %3}, [%4];\n\t}" ::"r"((int)c),
-        "r"(a), "d"(v[0]), "d"(v[1]), "r"(bar)
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], "
+        "{%1, %2}, [%3];" ::"r"(a),
+        "d"(v[0]), "d"(v[1]), "r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
@@ -491,7 +476,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
         if (AS && d.bar != kNoBar) {
 #pragma unroll
             for (int v = 0; v < N; ++v)
-                st16_async_if(true, d.base + xs + (v0 + v) * vs, cv + v * VW, d.bar);
+                st16_async(d.base + xs + (v0 + v) * vs, cv + v * VW, d.bar);
         } else {
 #pragma unroll
             for (int v = 0; v < N; ++v) st16(d.base + xs + (v0 + v) * vs, cv + v * VW);
@@ -500,7 +485,7 @@ __device__ __forceinline__ void plane_sweep_body(const PlaneArgs<T> &a) {
             if (AS && d.hbar != kNoBar) {
 #pragma unroll
                 for (int v = 0; v < N; ++v)
-                    st16_async_if(true, d.halo + xs + (v0 + v) * vs, cv + v * VW, d.hbar);
+                    st16_async(d.halo + xs + (v0 + v) * vs, cv + v * VW, d.hbar);
             } else {
 #pragma unroll
                 for (int v = 0; v < N; ++v) st16(d.halo + xs + (v0 + v) * vs, cv + v * VW);
