@@ -22,6 +22,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -3208,18 +3209,17 @@ int mg3d_formal_solve_ml(mg3d_handle *h, int level, double *jx_host, double *ux_
     MG_TRY(check_level(h, level));
     if (h->kind != 1) return fail(MG3D_E_STATE, "not a multi-level handle");
     Level &L = h->lev[level];
-    const size_t es = elem_size(h->prec);
     const size_t nv = (size_t)L.nvox;
-    std::vector<unsigned char> hj, hu;
     MG_TRY(ml_prd_prepare(h, level));
-    // a PRD frequency's sweep sums u alone; its U adds the local term in FP64
-    // (1 - rho chi_t/chi of the ratios kernel), as the radiative sums do
-    std::vector<double> prd_oc;
-    if (h->ml_prd) {
-        prd_oc.resize((size_t)h->n_prd_freq * nv);
-        MG_CUDA(cudaMemcpyAsync(prd_oc.data(), L.prd_oc, prd_oc.size() * sizeof(double),
-                                cudaMemcpyDeviceToHost, h->stream));
-    }
+    // the angle sums of the ray-group slots are added on the device, in slot order,
+    // piece by piece in the radiative sums' buffer (the rates refill it), so that
+    // one value per node and frequency is copied however many slots the shape has;
+    // through a small host buffer, since copies straight into a caller's fresh pages
+    // ran at 1.6 GB/s
+    const size_t piece = std::min<size_t>(1 << 20, (size_t)h->ntrans * kAccTerms *
+                                                       h->lev[h->L].nvox);
+    const std::unique_ptr<double[]> stage(new (std::nothrow) double[piece]);
+    if (!stage) return fail(MG3D_E_OOM, "host allocation failed");
     for (int f0 = 0; f0 < h->nfreq_ml; f0 += h->ml_chunk) {
         const int nc = std::min(h->ml_chunk, h->nfreq_ml - f0);
         MG_TRY(ml_chunk_fs(h, level, f0, nc));
@@ -3229,37 +3229,33 @@ int mg3d_formal_solve_ml(mg3d_handle *h, int level, double *jx_host, double *ux_
             h->force_bg = false;
             MG_TRY(rc);
         }
-        MG_CUDA(cudaStreamSynchronize(h->stream));
-        // the chunk's per-frequency sums of every ray-group slot, added on the
-        // host in slot order
-        const size_t cnt = (size_t)nc * nv;
-        const int slots = 2 * (12 / L.ml_rpb);
-        hj.resize(slots * cnt * es);
-        hu.resize(slots * cnt * es);
-        MG_CUDA(cudaMemcpy(hj.data(), h->ml_jx, slots * cnt * es, cudaMemcpyDeviceToHost));
-        MG_CUDA(cudaMemcpy(hu.data(), h->ml_ux, slots * cnt * es, cudaMemcpyDeviceToHost));
-        auto at = [&](const std::vector<unsigned char> &v, size_t i) {
-            return h->prec == MG3D_PREC_F64 ? ((const double *)v.data())[i]
-                                            : (double)((const float *)v.data())[i];
-        };
-        for (size_t i = 0; i < cnt; ++i) {
-            double J = at(hj, i), U = at(hu, i);
-            for (int sl = 1; sl < slots; ++sl) {
-                J += at(hj, sl * cnt + i);
-                U += at(hu, sl * cnt + i);
+        MlSlotSumArgs a{};
+        a.prec = h->prec;
+        a.len = (size_t)nc * nv;
+        a.nvox = nv;
+        a.slots = 2 * (12 / L.ml_rpb);
+        a.out = h->ml_acc;
+        for (int q = 0; q < 2; ++q) {
+            double *host = q == 0 ? jx_host : ux_host;
+            if (!host) continue;
+            a.src = q == 0 ? h->ml_jx : h->ml_ux;
+            // a PRD frequency's sweep sums u alone; its U adds the local term in FP64
+            // (1 - rho chi_t/chi of the ratios kernel), as the radiative sums do
+            const bool prd = q == 1 && h->ml_prd;
+            a.prd_index = prd ? h->d_prd_index + f0 : nullptr;
+            a.prd_oc = prd ? L.prd_oc : nullptr;
+            for (a.first = 0; a.first < a.len; a.first += piece) {
+                a.count = std::min(piece, a.len - a.first);
+                MG_TRY(launched(h, launch_ml_slot_sum(a, h->stream), "slot sums"));
+                MG_CUDA(cudaMemcpyAsync(stage.get(), a.out, a.count * sizeof(double),
+                                        cudaMemcpyDeviceToHost, h->stream));
+                MG_CUDA(cudaStreamSynchronize(h->stream));
+                std::memcpy(host + (size_t)f0 * nv + a.first, stage.get(),
+                            a.count * sizeof(double));
             }
-            const size_t o = (size_t)f0 * nv + i;
-            if (h->ml_prd) {
-                const int pr = h->prd_index[f0 + i / nv];
-                if (pr >= 0) {
-                    const double oc = prd_oc[(size_t)pr * nv + i % nv];
-                    U = oc + (1.0 - oc) * U;
-                }
-            }
-            if (jx_host) jx_host[o] = J;
-            if (ux_host) ux_host[o] = U;
         }
     }
+    MG_CUDA(cudaStreamSynchronize(h->stream));
     const double units = (double)L.nvox * kRays * h->nfreq_ml;
     ++h->fs_launches;
     h->fs_units += units;

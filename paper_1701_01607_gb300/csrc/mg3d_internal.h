@@ -527,6 +527,18 @@ cudaError_t launch_ml_sweep_f64(const MlSweepArgs<double> &a, int bands, int thr
 cudaError_t launch_ml_sweep_f32(const MlSweepArgs<float> &a, int bands, int threads,
                                 cudaStream_t st);
 cudaError_t launch_ml_accum(const MlAccumArgs &a, cudaStream_t st);
+// out[i - first] = sum over the slots of src[slot][i] (i = first .. first + count - 1 of
+// the chunk's [frequency][nvox] values), in slot order; a PRD frequency's value u as
+// oc + (1 - oc) u.
+struct MlSlotSumArgs {
+    int prec, slots;
+    size_t len, nvox, first, count;   // len: values of a slot
+    const void *src;
+    const int *prd_index;             // per frequency of the chunk: row of prd_oc or -1; or null
+    const double *prd_oc;
+    double *out;
+};
+cudaError_t launch_ml_slot_sum(const MlSlotSumArgs &a, cudaStream_t st);
 cudaError_t launch_ml_rates(const MlRateArgs &a, cudaStream_t st);
 
 }  // namespace mg3d

@@ -1446,6 +1446,31 @@ cudaError_t launch_ml_accum(const MlAccumArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <typename T>
+__global__ void ml_slot_sum_kernel(const MlSlotSumArgs a) {
+    const T *src = (const T *)a.src;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < a.count;
+         i += (size_t)gridDim.x * blockDim.x) {
+        const size_t o = a.first + i;
+        double v = slots_sum64(src + o, (long)a.len, a.slots);
+        if (a.prd_index) {
+            const int pr = a.prd_index[o / a.nvox];
+            if (pr >= 0) {
+                const double oc = a.prd_oc[(size_t)pr * a.nvox + o % a.nvox];
+                v = oc + (1.0 - oc) * v;
+            }
+        }
+        a.out[i] = v;
+    }
+}
+
+cudaError_t launch_ml_slot_sum(const MlSlotSumArgs &a, cudaStream_t st) {
+    const int g = grid_for((long)a.count, 256);
+    if (a.prec == MG3D_PREC_F64) ml_slot_sum_kernel<double><<<g, 256, 0, st>>>(a);
+    else ml_slot_sum_kernel<float><<<g, 256, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_ml_rates(const MlRateArgs &a, cudaStream_t st) {
     const int g = grid_for(a.nvox, kRateThreads);
     switch (a.n_levels) {
