@@ -155,7 +155,8 @@ struct mg3d_handle {
                                  // solutions update its background field
     bool force_bg = false;       // the current formal solution is a Lambda-iteration
     void *ml_jm = nullptr;       // mean intensity per slot [slots][chunk][nvox] (scatter)
-    int ml_slots = 2;            // most ray-group slots of any level (2 x 12 / ml_rpb)
+    size_t ml_slot_nodes = 0;    // values a frequency of the angle-sum buffers holds: the most
+                                 // slots x nodes of any level (2 x 12 / ml_rpb slots)
     void *ml_jx = nullptr, *ml_ux = nullptr;
     double *ml_acc = nullptr;
     mg3d_atom atom{};
@@ -2169,12 +2170,23 @@ void trapezoid_grid(double a, double b, int n, std::vector<double> &x, std::vect
     }
 }
 
+// Slots x nodes of the angle sums of level k with rpb rays per block, and the most
+// of any level with its current shape.
+size_t ml_level_slot_nodes(const mg3d_handle *h, int k, int rpb) {
+    return 2 * (size_t)(12 / rpb) * (size_t)h->lev[k].nvox;
+}
+size_t ml_max_slot_nodes(const mg3d_handle *h) {
+    size_t n = 0;
+    for (int k = 1; k <= h->L; ++k) n = std::max(n, ml_level_slot_nodes(h, k, h->lev[k].ml_rpb));
+    return n;
+}
+
 // Bytes the multi-level formal solution needs per frequency of a chunk:
 // opacity, source function and their two transition shares on every level,
-// and the angle sums of every ray-group slot on the finest.
+// and the angle sums of every ray-group slot (buffers shared by the levels).
 size_t ml_bytes_per_freq(const mg3d_handle *h) {
     const size_t es = elem_size(h->prec);
-    size_t b = (ml_lagged(h) ? 3 : 2) * (size_t)h->ml_slots * h->lev[h->L].nvox * es;
+    size_t b = (ml_lagged(h) ? 3 : 2) * h->ml_slot_nodes * es;
     const size_t per_level = h->params.sc_interp ? 6 : 4;  // Hermite: slopes of chi, S
     for (int k = 1; k <= h->L; ++k) b += per_level * (size_t)h->lev[k].nvox * es;
     return b;
@@ -2215,10 +2227,10 @@ int alloc_ml_chunks(mg3d_handle *h, int chunk) {
         const int nbufs = h->params.sc_interp ? 6 : 4;
         for (int i = 0; i < nbufs; ++i) MG_TRY(dev_alloc(bufs[i], (size_t)chunk * L.nvox * es));
     }
-    const size_t nv = h->lev[h->L].nvox;
-    MG_TRY(dev_alloc(&h->ml_jx, (size_t)h->ml_slots * chunk * nv * es));
-    MG_TRY(dev_alloc(&h->ml_ux, (size_t)h->ml_slots * chunk * nv * es));
-    if (ml_lagged(h)) MG_TRY(dev_alloc(&h->ml_jm, (size_t)h->ml_slots * chunk * nv * es));
+    const size_t bytes = h->ml_slot_nodes * (size_t)chunk * es;
+    MG_TRY(dev_alloc(&h->ml_jx, bytes));
+    MG_TRY(dev_alloc(&h->ml_ux, bytes));
+    if (ml_lagged(h)) MG_TRY(dev_alloc(&h->ml_jm, bytes));
     h->ml_chunk = chunk;
     return MG3D_OK;
 }
@@ -2374,7 +2386,7 @@ int autotune_ml_level(mg3d_handle *h, int k, int nc, int *evaluated) {
     if (!h->moving && !h->params.sc_interp && L.psteps)
         for (int nf : {1, 2, 4})
             for (int rpb : {12, 6, 4, 3, 2, 1}) {
-                if (2 * (12 / rpb) > h->ml_slots) continue;
+                if (ml_level_slot_nodes(h, k, rpb) > h->ml_slot_nodes) continue;
                 for (int bands = 1; bands <= kMaxBands && bands <= L.ny; ++bands) {
                     const int rows = (L.ny + bands - 1) / bands;
                     if ((long)(bands - 1) * rows >= L.ny) continue;
@@ -2391,7 +2403,7 @@ int autotune_ml_level(mg3d_handle *h, int k, int nc, int *evaluated) {
     g_last_error.clear();
     if (cands.empty()) return fail(MG3D_E_ARG, "no multi-level sweep shape fits");
     float warm = 0.f;
-    if (2 * (12 / L.ml_rpb) <= h->ml_slots)
+    if (ml_level_slot_nodes(h, k, L.ml_rpb) <= h->ml_slot_nodes)
         MG_TRY(time_ml_shape(h, k, L.ml_bands, L.ml_rpb, L.ml_threads, nc, 1, &warm, L.ml_plane,
                              L.ml_nf));
     std::vector<std::pair<float, size_t>> t1;
@@ -2433,11 +2445,13 @@ int autotune_ml(mg3d_handle *h, int level, int *evaluated) {
     // 24 where a level fits only one, or where the shifted-plane form applies:
     // wide planes take it with one ray per block), at most 32 frequencies
     // that fit
-    h->ml_slots = 12;
+    h->ml_slot_nodes = 0;
     for (int k = 1; k <= h->L; ++k)
-        if ((level == 0 || k == level) &&
-            (ml_single_ray_only(h, k) || (!h->moving && !h->params.sc_interp && h->lev[k].psteps)))
-            h->ml_slots = 24;
+        if (level == 0 || k == level) {
+            const bool one = ml_single_ray_only(h, k) ||
+                             (!h->moving && !h->params.sc_interp && h->lev[k].psteps);
+            h->ml_slot_nodes = std::max(h->ml_slot_nodes, ml_level_slot_nodes(h, k, one ? 1 : 2));
+        }
     MG_TRY(alloc_ml_chunks(h, 1));
     const int nc = std::min(32, default_ml_chunk(h));
     MG_TRY(alloc_ml_chunks(h, nc));
@@ -2448,8 +2462,7 @@ int autotune_ml(mg3d_handle *h, int level, int *evaluated) {
         MG_TRY(autotune_ml_level(h, k, nc, &c));
         count += c;
     }
-    h->ml_slots = 2;
-    for (int k = 1; k <= h->L; ++k) h->ml_slots = std::max(h->ml_slots, 2 * (12 / h->lev[k].ml_rpb));
+    h->ml_slot_nodes = ml_max_slot_nodes(h);
     MG_TRY(alloc_ml_chunks(h, 1));
     const int chunk = h->ml_chunk_req > 0 ? std::min(h->ml_chunk_req, h->nfreq_ml)
                                           : default_ml_chunk(h);
@@ -2807,7 +2820,6 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
         // fewest that fit and give >= 300 blocks, else the most that fit
         const bool plain = !atm->vel && !params->sc_interp;
         if (plain && h->prec == MG3D_PREC_F64 && choose_ml_plane(L, nf)) {
-            h->ml_slots = std::max(h->ml_slots, 2 * (12 / L.ml_rpb));
             continue;
         }
         int pick = 0;
@@ -2838,7 +2850,6 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
                 }
                 if (pick) {
                     L.ml_rpb = rpb;
-                    h->ml_slots = std::max(h->ml_slots, 2 * (12 / rpb));
                     break;
                 }
             }
@@ -2945,6 +2956,7 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
     MG_TRY(dalloc(&h->ml_acc, (size_t)h->ntrans * kAccTerms * F.nvox));
     if (params && params->ml_chunk < 0) return fail(MG3D_E_ARG, "negative ml_chunk");
     h->ml_chunk_req = params ? params->ml_chunk : 0;
+    h->ml_slot_nodes = ml_max_slot_nodes(h);
     MG_TRY(alloc_ml_chunks(h, params && params->ml_chunk > 0
                                   ? std::min(params->ml_chunk, h->nfreq_ml)
                                   : default_ml_chunk(h)));
@@ -3298,9 +3310,9 @@ int mg3d_set_ml_shape(mg3d_handle *h, int level, int bands, int rays_per_block, 
     L.ml_plane = 0;
     L.ml_nf = 1;
     drop_graphs(h);
-    const int slots = 2 * (12 / rays_per_block);
-    if (slots > h->ml_slots) {
-        h->ml_slots = slots;
+    const size_t need = ml_level_slot_nodes(h, level, rays_per_block);
+    if (need > h->ml_slot_nodes) {
+        h->ml_slot_nodes = need;
         MG_TRY(alloc_ml_chunks(h, h->ml_chunk));
     }
     return MG3D_OK;
@@ -3328,9 +3340,9 @@ int mg3d_set_ml_shape_ex(mg3d_handle *h, int level, int bands, int rays_per_bloc
     L.ml_plane = 1;
     L.ml_nf = freq_per_block;
     drop_graphs(h);
-    const int slots = 2 * (12 / rays_per_block);
-    if (slots > h->ml_slots) {
-        h->ml_slots = slots;
+    const size_t need = ml_level_slot_nodes(h, level, rays_per_block);
+    if (need > h->ml_slot_nodes) {
+        h->ml_slot_nodes = need;
         MG_TRY(alloc_ml_chunks(h, h->ml_chunk));
     }
     return MG3D_OK;
