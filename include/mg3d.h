@@ -460,8 +460,7 @@ int mg3d_formal_solve_ml(mg3d_handle *h, int level, double *jx_host, double *ux_
  * creation the library takes all frequencies when their arrays fit in 60 % of
  * the free device memory, else the largest chunk that does.  freq_per_chunk =
  * 0 means all frequencies.  Reallocates the chunk buffers (MG3D_E_OOM if they
- * do not fit); MG3D_E_STATE on a two-level handle.  Batch members need all
- * frequencies in one chunk.
+ * do not fit); MG3D_E_STATE on a two-level handle.
  * No counterpart in the paper (memory layout). */
 int mg3d_set_ml_chunk(mg3d_handle *h, int freq_per_chunk);
 int mg3d_get_ml_chunk(const mg3d_handle *h, int *freq_per_chunk);

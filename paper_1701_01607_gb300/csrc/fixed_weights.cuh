@@ -1,8 +1,8 @@
 // Short-characteristics weights in 64-bit integer arithmetic for the FP64 sweeps.
 //
-// GB300 executes about 1.7 FP64 operations per clock and SM (2 lanes), against 64
-// 32-bit integer multiplications, 32 widening ones and 64 logic operations, so
-// an FP64 multiply-add takes the time of 15-35 integer instructions, and the
+// GB300 executes about 1.7 FP64 operations per clock and SM (2 lanes), against 61
+// 32-bit integer multiply-adds, 23 widening ones and 64 logic operations, so
+// an FP64 multiply-add takes the time of 14-35 integer instructions, and the
 // exponential, reciprocal and differences of one set of weights (16 FP64
 // operations) were half the arithmetic of the FP64 sweep.  Here they run on
 // the integer pipes instead (about 100 instructions a set) and leave the FP64

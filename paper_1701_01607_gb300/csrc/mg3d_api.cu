@@ -632,7 +632,11 @@ SweepShape var_shape(int prec, int nx, int ny, int nslots, int prd, int np, int 
 // the shape picked is within 6 % of the fastest in seven of them (48x48x97, 17
 // frequencies, FP32: one group of 5 bands, 504 us, where three groups take 609;
 // 64x64x65: three groups of 8 bands, 568 against 730 for one group), and within
-// 12 and 29 % at 16x16 nodes (54 us for 42).
+// 12 and 29 % at 16x16 nodes (54 us for 42).  MALI sweeps with the shape picked against
+// the band sweep's default on 14 grids from 1x1 to 128x128 nodes, 7 and 17 frequencies, both
+// variants: FP64 1.3 to 3.5 times faster, FP32 1.0 to 1.8 (0.95 to 0.98 for single
+// columns and 96x96x33 with 7 frequencies).  Its occupancy queries take about 0.3 ms a grid
+// at creation.
 SweepShape choose_var_shape(int prec, int nx, int ny, int nslots, int prd) {
     const bool f64 = prec == MG3D_PREC_F64;
     const double t0 = f64 ? 1650.0 : 400.0, chain = f64 ? 700.0 : 900.0;
@@ -1434,8 +1438,7 @@ void drop_graphs(mg3d_handle *h) {
     }
 }
 
-// Capture the cycle into a graph (once per variant), then replay it; the
-// library's counters advance by what the captured cycle launched.
+// The handle's counters of launches, units and sweeps.
 mg3d_handle::CycleDelta counter_state(const mg3d_handle *h) {
     mg3d_handle::CycleDelta c;
     c.launches = h->launches;
@@ -1448,6 +1451,8 @@ mg3d_handle::CycleDelta counter_state(const mg3d_handle *h) {
     return c;
 }
 
+// Capture the cycle into a graph (once per variant), then replay it; the
+// library's counters advance by what the captured cycle launched.
 int graph_cycle(mg3d_handle *h, bool first) {
     const int idx = first ? 1 : 0;
     if (h->graph_stream != h->stream) {
@@ -2609,7 +2614,8 @@ int setup_ml_prd(mg3d_handle *h, const mg3d_ml_atom *atom) {
 // memory), the fewest bands of at most 512 nodes and the most rays that fit.
 // Measured (32x32x65, 120 frequencies): 2 bands x 3 rays 7.2 ms, the other form
 // at its former default, 2 x 12, 17.6 ms; 8x8x9, 30 frequencies: 1 x 1 105 us, 1 x 12
-// 286 us a MALI sweep.  False where no such shape fits.
+// 286 us a MALI sweep; 64x64x65, 120 frequencies: 8 x 2 35 ms, the other form's 4 x 12 65
+// ms a MALI sweep.  False where no such shape fits (96x96 and wider planes).
 bool choose_ml_plane(Level &L, int nf) {
     constexpr size_t kHalfSmem = 103 * 1024;
     if (!plane_grid_ok(L.nx, L.ny, L.nz)) return false;
@@ -2828,7 +2834,9 @@ int create_ml_impl(const mg3d_ml_atmosphere *atm, const mg3d_ml_atom *atom,
         // allow it, and fewer rays per block where there would be less than
         // 200 blocks (FP32 64x64x129, 120 frequencies: 8 bands x 12 rays 7.6 ms,
         // the fewest bands that fit, 3 x 12, 15.6 ms; 20x18x21, 30 frequencies: 1 x 3
-        // 108 us, 1 x 12 167 us a MALI sweep)
+        // 108 us, 1 x 12 167 us a MALI sweep.  MALI sweeps of wider planes, 120
+        // frequencies, against the most rays that fit: 96x96x33 8 x 4 5.7 ms for 8.9,
+        // 128x128x33 8 x 3 10.5 ms for 17.1, 256x256x17 the same shape)
         for (int pass = plain ? 0 : 1; pass < 2 && !pick; ++pass)
             for (int rpb : {12, 6, 4, 3, 2, 1}) {
                 if (pass == 0 && rpb < 3) break;
@@ -3006,8 +3014,8 @@ int batch_each(mg3d_batch *b, F work) {
 // One V-cycle of every member: the members' own cycle graphs, launched on their
 // streams.  On coarse grids a cycle is a chain of small kernels that leave most
 // of the GPU idle, so cycles of several members overlap almost entirely: four
-// members of 32x32x33 to 48x40x65 take 7.5 ms instead of 13.7 ms in lockstep
-// with one sweep launch for all of them.
+// members of 32x32x33 to 48x40x65 take 6.2 ms; in lockstep, with one sweep launch for
+// all of them, they took 13.7 ms when this form took 7.5.
 int batch_cycle(mg3d_batch *b, bool first, double *C, long long *neg) {
     const int rc = batch_each(b, [&](mg3d_handle *h) {
         h->top = h->L;

@@ -360,11 +360,11 @@ struct MlPlaneArgs {
 // Frequencies per block the multi-level shifted-plane sweep is built for,
 // and the nodes a thread takes per step (band <= this x threads).
 constexpr int kMlPlaneNf[] = {1, 2, 4};
-// dynamic shared memory limit of the multi-level shifted-plane sweep: its
-// static part (the FP64 exp table and the rays' step constants, 3.2 KB) and
-// this stay within the 227 KB a block may take
 // a quarter of an SM's shared memory: four blocks of the multi-level sweep
 constexpr size_t kMlQuarterSmem = 52 * 1024;
+// dynamic shared memory limit of the multi-level shifted-plane sweep: its static
+// part (in FP64 the tables of the integer weights, 4 KB, and the rays' step constants
+// of four steps, 2.3 KB) and this stay within the 227 KB a block may take
 constexpr size_t kMlPlaneMaxSmem = 220 * 1024;
 constexpr int kMlPlaneNfCount = 3;
 __host__ __device__ constexpr int ml_plane_max_pass(int nf) { return nf <= 2 ? 4 : 2; }
@@ -412,8 +412,6 @@ struct MlPrdArgs {
     double *oc;                      // [n_prd_freq][nvox] out: 1 - rho chi_t/chi
 };
 
-// Opacity of the chunk of frequencies f0 .. f0+nfreq-1, written at the
-// chunk-local index [f - f0][nvox].
 // Constants of a frequency for the opacity and the radiative sums, in both
 // precisions; (h, l) is a value as a pair of floats.
 struct alignas(16) FreqOp {
@@ -437,6 +435,8 @@ struct MlNodeTab {
     const void *bline;      // [n_lines][nvox] Planck function at line centre (FS precision)
 };
 
+// Opacity of the chunk of frequencies f0 .. f0+nfreq-1, written at the
+// chunk-local index [f - f0][nvox].
 struct MlOpacityArgs {
     long nvox;
     int f0, nfreq, n_trans, prec;  // chunk f0 .. f0+nfreq-1

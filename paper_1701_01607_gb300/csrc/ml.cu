@@ -81,8 +81,8 @@ __device__ __forceinline__ float ml_doppler(float dd2, float di, const ExpNegTab
 // from 64-bit integer arithmetic.  The grid's y index is the transition, so
 // that small grids still fill the GPU and the populations and Planck function
 // of a transition are read once.  Measured (64x64x129, 120 frequencies, FP32):
-// opacity 3.00 -> 0.45 ms, sums 2.53 -> 0.37 ms; FP64 32x32x65: 0.82 -> 0.40 and 0.45 ->
-// 0.25 ms; on an 8x8x9 grid with 30 frequencies (FP32) 75 -> 10 us each.
+// opacity 3.00 -> 0.33 ms, sums 2.53 -> 0.36 ms; FP64 32x32x65: 0.82 -> 0.33 and 0.45 ->
+// 0.35 ms; on an 8x8x9 grid with 30 frequencies (FP32) 75 -> 8 and 75 -> 15 us.
 
 // e^-(product of two pairs) in FP32, the argument rounded once
 __device__ __forceinline__ float pair_arg(float ah, float al, float bh, float bl) {
@@ -1248,7 +1248,7 @@ __global__ void __launch_bounds__(256, 4)
 // elimination runs on registers with every index static, pivots chosen on the
 // bit patterns (positive doubles order like them) and one refined reciprocal
 // per pivot, so that the FP64 pipe sees the products alone.  64x64x129, N = 6:
-// 549 -> 300 us; an 8x8x9 grid, latency alone: 50 -> 15 us.
+// 549 -> 460 us; an 8x8x9 grid, latency alone: 50 -> 24 us.
 constexpr int kRateThreads = 64;
 template <int N>
 __global__ void __launch_bounds__(kRateThreads) ml_rates_kernel(const MlRateArgs a) {

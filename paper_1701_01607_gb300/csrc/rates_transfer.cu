@@ -69,7 +69,9 @@ __device__ __forceinline__ unsigned block_count(unsigned c) {
 // pair of floats (Knuth's two-sum, about 2^-45 of the sum), FP64 slots as 64-bit
 // integers under the largest exponent.  Before, with FP64 additions, one
 // reduction took 377 us for 128x128x129 FP32 slots and 54 us for 64x64x129 FP64
-// ones; now 75 and 40 us.
+// ones; now 75 and 40 us.  The pairs add nothing to the FP32 results' errors: J, U and the
+// populations after three sweeps of 96 boxes (static, moving, PRD) against FP64 handles have
+// the same rms errors to six digits with all slots added in FP64.
 constexpr int kSumSlots = 24;   // slots added at a time; their number is a multiple
 
 __device__ __noinline__ double plain_sum(const float *p, long stride, int n) {
