@@ -176,7 +176,9 @@ __device__ __forceinline__ void cont_terms(const FreqOp &q, double inv_T, const 
     const double x = q.a * inv_T;
     fx::u64 e, d;
     int n;
-    if (fx::exp_parts(x, ft, &e, &n, &d)) {
+    // 1 - e^-x as a fraction is good to 2^-55.5, so to FP64 relative to itself from x of
+    // 1/4 on (at 1/1000 it would lose 8 bits)
+    if (x >= 0.25 && fx::exp_parts(x, ft, &e, &n, &d)) {
         E = e ? fx::pack62(e, -n) : 0.0;
         B = q.ry3 * fast_div(E, fx::pack32(d, 0));
     } else {
